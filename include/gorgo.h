@@ -412,18 +412,18 @@ int gorgo_measure_gather(int device, void *buffer, uint64_t buffer_bytes, uint64
                          void *cuda_stream, double *sectors_gb_per_s);
 
 /* Test aid (no counterpart in the paper).  Inside the replay kernel the warps of one candidate
- * wait for one another with bounded polls, and two kinds of helper warps only prepare work
- * ahead of the warps that must do it anyway (the probe warps stage prefix hits, the scout warps
- * pre-validate eviction victims).  These switches let a test take those paths on purpose; none
- * of them makes a kernel fault or hang.  They apply to every later launch of `sim`.
+ * wait for one another with bounded polls, and two of them prepare work ahead of the warp that
+ * decides (prefix hits are read ahead, eviction victims are listed ahead).  These switches let a
+ * test take the other paths on purpose; none of them makes a kernel fault or hang.  They apply to
+ * every later launch of `sim`.
  *   GORGO_DEBUG_POLL_LIMIT  polls after which a warp gives up waiting (default 2^24).  With 0 the
  *                           first wait that is not already satisfied gives up: the candidate
  *                           finishes with wrong results and status GORGO_ERR_DEVICE_LIMIT.
- *   GORGO_DEBUG_RING_POLLS  polls of a commit warp for the scout's next victim before it looks for
- *                           victims itself (default 64; results do not depend on it).
- *   GORGO_DEBUG_PROBE_OFF   nonzero: no probe warps; every request is probed where it is needed
- *                           (results do not depend on it).
- *   GORGO_DEBUG_SCOUT_OFF   nonzero: no scout warps (results do not depend on it). */
+ *   GORGO_DEBUG_RING_POLLS  accepted, without effect (victims are always waited for).
+ *   GORGO_DEBUG_PROBE_OFF   nonzero: requests are not staged several at once from words read ahead;
+ *                           each is staged alone (results do not depend on it).
+ *   GORGO_DEBUG_SCOUT_OFF   nonzero: victims are listed only when a commit asks for one (results do
+ *                           not depend on it). */
 enum {
   GORGO_DEBUG_POLL_LIMIT = 0,
   GORGO_DEBUG_RING_POLLS = 1,

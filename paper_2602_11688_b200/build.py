@@ -9,8 +9,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgorgo_b200.so")
 LIB_PROF = os.path.join(HERE, "libgorgo_b200_prof.so")
-SOURCES = ["gorgo_kernels.cu", "gorgo_host.cu"]
-HEADERS = ["gorgo_internal.h", os.path.join("..", "..", "include", "gorgo.h")]
+SOURCES = ["gorgo_replay.cu", "gorgo_kernels.cu", "gorgo_host.cu"]
+HEADERS = ["gorgo_internal.h", "gorgo_device.cuh", os.path.join("..", "..", "include", "gorgo.h")]
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",

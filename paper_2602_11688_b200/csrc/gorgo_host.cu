@@ -14,61 +14,73 @@
 
 using namespace gorgo;
 
-// 64-bit id -> dense number, open addressing, grows by doubling.
+// 64-bit id -> dense number: open addressing, one 8-byte slot per entry (upper half of the hash,
+// dense number + 1; 0 = empty), so that a lookup costs one cache miss.  The caller's ids by dense
+// number are kept beside it (`raw`) and decide when the upper halves agree.
 struct IdMap {
-  std::vector<uint64_t> keys;
-  std::vector<uint32_t> vals;  // 0 = empty, else dense + 1
-  uint64_t mask = 0, used = 0;
+  std::vector<uint64_t> slot;
+  std::vector<uint64_t> raw;
+  uint64_t mask = 0;
   static uint64_t hash(uint64_t z) {
     z ^= z >> 33; z *= 0xff51afd7ed558ccdULL; z ^= z >> 33; z *= 0xc4ceb9fe1a85ec53ULL;
     return z ^ (z >> 33);
   }
-  explicit IdMap(uint64_t cap_pow2) : keys(cap_pow2), vals(cap_pow2, 0), mask(cap_pow2 - 1) {}
+  explicit IdMap(uint64_t cap_pow2) : slot(cap_pow2, 0), mask(cap_pow2 - 1) {}
+  void prefetch(uint64_t k) const { __builtin_prefetch(&slot[hash(k) & mask], 1); }
   void grow() {
-    IdMap bigger((mask + 1) * 2);
-    for (uint64_t i = 0; i <= mask; ++i)
-      if (vals[i]) bigger.put(keys[i], vals[i]);
-    keys.swap(bigger.keys); vals.swap(bigger.vals); mask = bigger.mask;
+    const uint64_t cap = (mask + 1) * 4;
+    slot.assign(cap, 0);
+    mask = cap - 1;
+    const uint64_t n = raw.size();
+    for (uint64_t d = 0; d < n; ++d) {
+      if (d + 16 < n) prefetch(raw[d + 16]);
+      const uint64_t h = hash(raw[d]);
+      uint64_t i = h & mask;
+      while (slot[i]) i = (i + 1) & mask;
+      slot[i] = (h >> 32 << 32) | (d + 1);
+    }
   }
-  void put(uint64_t k, uint32_t v) {
-    uint64_t i = hash(k) & mask;
-    while (vals[i]) i = (i + 1) & mask;
-    keys[i] = k; vals[i] = v; ++used;
-  }
-  // returns dense number, assigning `next` if the id is new
-  uint32_t get_or_add(uint64_t k, uint32_t& next) {
-    uint64_t i = hash(k) & mask;
-    while (vals[i]) {
-      if (keys[i] == k) return vals[i] - 1;
+  // dense number of k; a new id gets the next one
+  uint32_t get_or_add(uint64_t k) {
+    const uint64_t h = hash(k), tag = h >> 32;
+    uint64_t i = h & mask;
+    while (slot[i]) {
+      if (slot[i] >> 32 == tag && raw[(uint32_t)slot[i] - 1] == k) return (uint32_t)slot[i] - 1;
       i = (i + 1) & mask;
     }
-    if ((used + 1) * 2 > mask + 1) { grow(); return get_or_add(k, next); }
-    keys[i] = k; vals[i] = next + 1; ++used;
-    return next++;
+    const uint32_t d = (uint32_t)raw.size();
+    raw.push_back(k);
+    slot[i] = (tag << 32) | (d + 1u);
+    if (raw.size() * 2 > mask + 1) grow();
+    return d;
   }
 };
 
 // Host side of a trace that is still growing (gorgo_trace_begin / gorgo_trace_append): what the
-// next batch needs to know about the requests before it, and where the device regions lie.
+// next batch needs to know about the requests before it.  A block of a growing trace is an atom of
+// its own: requests to come may share any part of what is known so far.
 struct TraceBuilder {
-  IdMap map{1ull << 16};
-  std::vector<uint32_t> seen_in;          // per dense id: request (+1) that last contained it
-  std::vector<uint32_t> last_g, last_r;   // per dense id: flat position and request of its last occurrence
-  std::vector<uint64_t> raw_new;          // caller's ids of the dense ids added by the current batch
+  IdMap map{1ull << 12};
+  std::vector<uint32_t> last_g, last_r;   // per dense id: touch and request of its last occurrence
   std::vector<double> ts;                 // arrival times so far
-  uint64_t cap_req = 0, cap_ids = 0;      // capacities the device regions were laid out for
-  uint64_t N = 0, T = 0;
-  uint32_t D = 0;
-  double grid_dt = 0.0;
-  uint32_t grid_n = 0;
+  uint64_t T = 0;                         // block ids so far
   uint64_t grid_cursor = 0;               // first request not yet behind the last grid edge
-  unsigned char *d_req = nullptr, *d_ids = nullptr, *d_occ = nullptr, *d_raw = nullptr,
-                *d_prev = nullptr, *d_ts = nullptr, *d_grid = nullptr;
+  std::vector<uint64_t> dup;              // scratch: ids of one request, open addressing
+  std::vector<uint32_t> dup_stamp;
+  uint32_t stamp = 0;
+};
+
+// Where the regions of the trace buffer lie, and the capacities they were laid out for.
+struct TraceRegions {
+  uint64_t cap_req = 0, cap_ids = 0;
+  unsigned char *req = nullptr, *touch = nullptr, *raw = nullptr, *extra = nullptr, *ts = nullptr,
+                *grid = nullptr, *rtt = nullptr;   // extra: first block of each atom, or scratch of an append
 };
 
 struct gorgo_sim {
   Model m;
   std::unique_ptr<TraceBuilder> tb;       // set while the trace can still grow
+  TraceRegions reg;
   uint64_t cap_req = 0, cap_ids = 0;      // appendable trace: sizes the workspaces are laid out for (else 0)
   std::vector<double> rtt;
   std::vector<double> rep_prefill, rep_tpot;   // per-replica speeds; empty: the uniform constants
@@ -82,7 +94,6 @@ struct gorgo_sim {
   bool has_trace = false;
   TraceView tr = {};
   uint32_t poll_limit = 1u << 24;   // bound of the device-side waits of one warp for another
-  uint32_t ring_polls = 64;         // polls for the scout's victims before a commit warp walks itself
   uint32_t probe_off = 0, scout_off = 0;   // test switches (gorgo_debug_set)
   // optional CUDA-event timing of the replay kernel (one pair per wave of the last evaluation)
   bool profiling = false;
@@ -120,25 +131,25 @@ StateLayout make_layout(const Model& m) {
 
 // Byte offsets of the regions of a workspace for `res` resident candidates.
 struct WsLayout {
-  uint64_t params, scales, rtt, speeds, status, p95, forced, draws, series, masks, states, lists, exp_head, exp_rec, lru_next,
+  uint64_t params, scales, speeds, status, p95, forced, draws, series, masks, states, exp_head, exp_rec,
       route_log, finish, ttft, e2e, total;
-  uint64_t mask_stride;
+  uint64_t mask_stride, index_off;
   StateLayout st;
 };
 
-WsLayout make_ws(const gorgo_sim* s, uint64_t res, bool with_latency) {
+WsLayout make_ws(const gorgo_sim* s, uint64_t res, bool with_latency, bool with_index = true) {
   WsLayout w;
   const Model& m = s->m;
   // an appendable trace lays everything out for its capacities, so that a persistent state stays
   // valid while the trace grows
   const uint64_t N = s->cap_req ? s->cap_req : s->tr.n_req;
-  const uint64_t D = s->cap_req ? s->cap_ids : s->tr.n_distinct;
+  const uint64_t A = s->cap_req ? s->cap_ids : s->tr.n_atoms;
   w.st = make_layout(m);
-  w.mask_stride = align_up(D * mask_bytes_for(m.R));
+  w.index_off = align_up(A * mask_bytes_for(m.R));
+  w.mask_stride = with_index ? 2 * w.index_off : w.index_off;
   uint64_t o = 0;
   w.params = o; o = align_up(o + res * m.K * 8);
   w.scales = o; o = align_up(o + res * 8);       // one time scale per candidate (optional)
-  w.rtt = o; o = align_up(o + (uint64_t)m.G * m.R * 8);
   w.speeds = o; o = align_up(o + (uint64_t)m.R * 16);   // per-replica speeds (optional)
   w.series = o; o = align_up(o + (uint64_t)s->n_epochs * m.G * m.R * 16);   // RTT series (optional)
   w.status = o; o = align_up(o + res * 4);
@@ -147,16 +158,31 @@ WsLayout make_ws(const gorgo_sim* s, uint64_t res, bool with_latency) {
   w.draws = o; o = align_up(o + N * 4);       //   and the caller's draws for `random`
   w.masks = o; o = align_up(o + res * w.mask_stride);
   w.states = o; o = align_up(o + res * w.st.bytes);
-  w.lists = o; o = align_up(o + res * evict_list_bytes(m.R));
   w.exp_head = o; o = align_up(o + res * N * 4);
   w.exp_rec = o; o = align_up(o + res * N * 16);
-  w.lru_next = o; o = align_up(o + res * N * 4);
   w.route_log = o; o = align_up(o + res * N);
   w.finish = o; if (!with_latency) o = align_up(o + res * N * 8);   // persistent state only
   w.ttft = o; if (with_latency) o = align_up(o + res * N * 8);
   w.e2e = o; if (with_latency) o = align_up(o + res * N * 8);
   w.total = o;
   return w;
+}
+
+// Bytes of a candidate's words that a replay reads (the proxy-index words only when it is on).
+uint64_t reset_bytes(const gorgo_sim* sim, const WsLayout& w) { return sim->proxy_index ? w.mask_stride : w.index_off; }
+
+// Arguments every replay launch of a simulator shares.
+ReplayArgs base_args(const gorgo_sim* sim, unsigned char* base, const WsLayout& w) {
+  ReplayArgs a = {};
+  a.m = sim->m; a.tr = sim->tr;
+  a.poll_limit = sim->poll_limit;
+  a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
+  a.masks = base + w.masks; a.mask_stride = w.mask_stride; a.index_off = w.index_off;
+  a.states = base + w.states; a.lay = w.st;
+  a.exp_head = reinterpret_cast<uint32_t*>(base + w.exp_head);
+  a.exp_rec = reinterpret_cast<uint4*>(base + w.exp_rec);
+  a.route_log = base + w.route_log; a.route_log_stride = sim->tr.n_req;
+  return a;
 }
 
 // Copies the per-replica speeds (if set) into the workspace and points the launch at them.
@@ -225,7 +251,7 @@ int eval_impl(gorgo_sim* sim, uint32_t P, const double* params, double scale, vo
               uint64_t workspace_bytes, cudaStream_t st, double* p95_ttft, double* p95_e2e,
               uint8_t* route, uint16_t* hit, uint64_t* digest, uint64_t* stats, int32_t* cand_status,
               bool host_io, const WindowSpec* win = nullptr, const PolicySpec* pol = nullptr,
-              const double* scales = nullptr /* HOST [P] or null */) {
+              const double* scales = nullptr /* HOST [P] or null */, bool with_index = true) {
   if (!sim || !params || !workspace || P == 0) return GORGO_ERR_INVALID_ARG;
   if ((!p95_ttft || !p95_e2e) && !win) return GORGO_ERR_INVALID_ARG;
   if (win && (win->window == 0 || win->hop == 0 || win->window > window_max() || !win->best))
@@ -248,20 +274,16 @@ int eval_impl(gorgo_sim* sim, uint32_t P, const double* params, double scale, vo
   uint64_t lo = 0, hi = P;
   while (lo < hi) {
     const uint64_t mid = (lo + hi + 1) / 2;
-    if (make_ws(sim, mid, true).total <= workspace_bytes) lo = mid; else hi = mid - 1;
+    if (make_ws(sim, mid, true, with_index).total <= workspace_bytes) lo = mid; else hi = mid - 1;
   }
   if (lo == 0) return GORGO_ERR_WORKSPACE_TOO_SMALL;
   const uint32_t res = (uint32_t)lo;
-  const WsLayout w = make_ws(sim, res, true);
+  const WsLayout w = make_ws(sim, res, true, with_index);
   unsigned char* base = static_cast<unsigned char*>(workspace);
   double* d_params = reinterpret_cast<double*>(base + w.params);
-  double* d_rtt = reinterpret_cast<double*>(base + w.rtt);
   int32_t* d_status = reinterpret_cast<int32_t*>(base + w.status);
   double* d_p95 = reinterpret_cast<double*>(base + w.p95);
 
-  if (cudaMemcpyAsync(d_rtt, sim->rtt.data(), sim->rtt.size() * 8, cudaMemcpyHostToDevice, st) !=
-      cudaSuccess)
-    return GORGO_ERR_CUDA;
   std::vector<int32_t> h_status;
   if (host_io) h_status.assign(P, 0);
   sim->ev_used = 0;
@@ -278,15 +300,15 @@ int eval_impl(gorgo_sim* sim, uint32_t P, const double* params, double scale, vo
         return GORGO_ERR_CUDA;
       wave_params = d_params;
     }
-    if (launch_reset(base + w.masks, (uint64_t)pw * w.mask_stride,
+    if (launch_reset(base + w.masks, w.mask_stride, reset_bytes(sim, w),
                      reinterpret_cast<uint32_t*>(base + w.exp_head), (uint64_t)pw * N,
                      base + w.states, w.st, m, pw, st) != cudaSuccess)
       return GORGO_ERR_CUDA;
     if (stats && cudaMemsetAsync(stats + (size_t)p0 * 4, 0, (size_t)pw * 32, st) != cudaSuccess)
       return GORGO_ERR_CUDA;
 
-    ReplayArgs a = {};
-    a.m = m; a.tr = sim->tr; a.scale = scale;
+    ReplayArgs a = base_args(sim, base, w);
+    a.scale = scale;
     if (scales) {
       double* d_scales = reinterpret_cast<double*>(base + w.scales);
       if (cudaMemcpyAsync(d_scales, scales + p0, (size_t)pw * 8, cudaMemcpyHostToDevice, st) !=
@@ -295,17 +317,8 @@ int eval_impl(gorgo_sim* sim, uint32_t P, const double* params, double scale, vo
       a.scales = d_scales;
     }
     a.first = 0; a.count = (uint32_t)N; a.check_order = 0;
-    a.poll_limit = sim->poll_limit; a.ring_polls = sim->ring_polls;
-    a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
-    a.rtt = d_rtt; a.params = wave_params;
-    a.masks = base + w.masks; a.mask_stride = w.mask_stride;
-    a.states = base + w.states; a.lay = w.st;
-    a.evict_lists = reinterpret_cast<uint4*>(base + w.lists);
-    a.exp_head = reinterpret_cast<uint32_t*>(base + w.exp_head);
-    a.exp_rec = reinterpret_cast<uint4*>(base + w.exp_rec);
-    a.lru_next = reinterpret_cast<uint32_t*>(base + w.lru_next);
-    a.route_log = route ? route + (size_t)p0 * N : base + w.route_log;
-    a.route_log_stride = N;
+    a.params = wave_params;
+    if (route) a.route_log = route + (size_t)p0 * N;
     a.queue_in_requests = pol && pol->queue_in_requests ? 1u : 0u;
     a.forced_route = pol ? pol->forced_route : nullptr;
     if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
@@ -476,168 +489,68 @@ int gorgo_sim_set_service_model(gorgo_sim_t* sim, double decode_slowdown, uint64
 
 int gorgo_trace_bytes(uint64_t n_requests, uint64_t n_block_ids, uint64_t* bytes_out) {
   if (!bytes_out) return GORGO_ERR_INVALID_ARG;
-  *bytes_out = align_up(n_requests * sizeof(ReqRec)) + align_up(n_block_ids * 4) +
-               align_up(n_block_ids * 8) + align_up(n_block_ids * 8) + align_up(n_block_ids * 8) +
-               align_up(n_requests * 8) +
-               align_up((n_requests + 1) * 4) + kAlign;
+  *bytes_out = align_up(n_requests * sizeof(ReqRec)) + align_up(n_block_ids * sizeof(Touch)) +
+               align_up(n_block_ids * 8) + align_up(n_block_ids * 4) + align_up(n_requests * 8) +
+               align_up((n_requests + 1) * 4) + align_up(4096 * 8) + kAlign;
   return GORGO_OK;
 }
 
-// Appends `n_new` requests to the trace under construction in `sim->tb`.  With `atomic` a trace
-// that fails a check is left as it was; without it the caller discards the builder on failure.
-static int trace_append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms,
-                             const uint32_t* input_tokens, const uint32_t* output_tokens,
-                             const uint16_t* origin, const uint64_t* hash_off,
-                             const uint64_t* hash_ids, cudaStream_t st, bool atomic) {
-  TraceBuilder& tb = *sim->tb;
-  const Model& m = sim->m;
-  if (n_new < 1 || hash_off[0] != 0) return GORGO_ERR_BAD_TRACE;
-  for (uint64_t k = 0; k < n_new; ++k)
-    if (hash_off[k + 1] < hash_off[k]) return GORGO_ERR_BAD_TRACE;
-  const uint64_t Tn = hash_off[n_new];
-  const uint64_t N0 = tb.N, T0 = tb.T, N = N0 + n_new, T = T0 + Tn;
-  if (N > tb.cap_req || T > tb.cap_ids) return GORGO_ERR_WORKSPACE_TOO_SMALL;
-  if (Tn > 0 && !hash_ids) return GORGO_ERR_INVALID_ARG;
+// What does not depend on the block ids: order and domain of the arrivals, block counts, regions.
+// Fills the records up to the touches.
+static int check_requests(const Model& m, uint64_t n, double prev_t, const double* ts_ms, const uint32_t* input_tokens,
+                          const uint32_t* output_tokens, const uint16_t* origin, const uint64_t* hash_off,
+                          ReqRec* req) {
   const uint64_t nmax = m.C < 65535 ? m.C : 65535;
-
-  std::vector<ReqRec> req(n_new);
-  double prev_t = N0 ? tb.ts.back() : 0.0;
-  for (uint64_t k = 0; k < n_new; ++k) {
+  for (uint64_t k = 0; k < n; ++k) {
     const double t = ts_ms[k];
     if (!finite_nonneg(t) || t < prev_t) return GORGO_ERR_BAD_TRACE;
     prev_t = t;
-    const uint64_t n = hash_off[k + 1] - hash_off[k];
+    if (hash_off[k + 1] < hash_off[k]) return GORGO_ERR_BAD_TRACE;
+    const uint64_t nb = hash_off[k + 1] - hash_off[k];
     const uint64_t want = ((uint64_t)input_tokens[k] + m.B - 1) / m.B;
-    if (n != want || n > nmax) return GORGO_ERR_BAD_TRACE;
+    if (nb != want || nb > nmax) return GORGO_ERR_BAD_TRACE;
     const uint16_t g = origin ? origin[k] : (uint16_t)0;
     if (g >= m.G) return GORGO_ERR_BAD_TRACE;
     ReqRec& q = req[k];
-    q.ts_ms = t; q.off = (uint32_t)(T0 + hash_off[k]); q.in_tok = input_tokens[k];
-    q.out_tok = output_tokens[k]; q.nblk = (uint16_t)n; q.origin = g; q.prev_share = kNone; q.pad = 0;
+    q.ts_ms = t; q.off = 0; q.in_tok = input_tokens[k]; q.out_tok = output_tokens[k];
+    q.m = 0; q.origin = g; q.prev_share = kNone; q.nblk = (uint32_t)nb;
   }
-  if (atomic) {   // an id twice in one request: found before anything is changed
-    std::vector<uint64_t> tmp;
-    for (uint64_t k = 0; k < n_new; ++k) {
-      tmp.assign(hash_ids + hash_off[k], hash_ids + hash_off[k + 1]);
-      std::sort(tmp.begin(), tmp.end());
-      if (std::adjacent_find(tmp.begin(), tmp.end()) != tmp.end()) return GORGO_ERR_BAD_TRACE;
-    }
-  }
-
-  // dense renumbering in order of first appearance; per block the previous occurrence, and the
-  // next one where that lies in this batch (an earlier batch's entry is patched on the device)
-  std::vector<uint32_t> ids(Tn);
-  std::vector<uint2> occ(Tn, make_uint2(kNone, kNone)), occ_before(Tn);
-  const uint32_t D0 = tb.D;
-  bool patch_old = false;
-  for (uint64_t k = 0; k < n_new; ++k) {
-    const uint32_t r = (uint32_t)(N0 + k);
-    uint32_t latest = 0;  // latest earlier request (+1) that contains one of this one's blocks
-    for (uint64_t gl = hash_off[k]; gl < hash_off[k + 1]; ++gl) {
-      const uint32_t before = tb.D;
-      const uint32_t d = tb.map.get_or_add(hash_ids[gl], tb.D);
-      if (tb.D != before) {
-        tb.raw_new.push_back(hash_ids[gl]);
-        tb.seen_in.push_back(0); tb.last_g.push_back(kNone); tb.last_r.push_back(kNone);
-      }
-      if (tb.seen_in[d] == r + 1) return GORGO_ERR_BAD_TRACE;   // (not reached when `atomic`)
-      if (tb.seen_in[d] > latest) latest = tb.seen_in[d];
-      tb.seen_in[d] = r + 1;
-      ids[gl] = d;
-      const uint32_t g = (uint32_t)(T0 + gl);
-      const uint32_t pg = tb.last_g[d];
-      occ_before[gl] = make_uint2(pg, tb.last_r[d]);
-      if (pg != kNone) {
-        if (pg >= T0) occ[pg - T0] = make_uint2(g, r);
-        else patch_old = true;
-      }
-      tb.last_g[d] = g; tb.last_r[d] = r;
-    }
-    req[k].prev_share = latest ? latest - 1 : kNone;
-  }
-  tb.ts.insert(tb.ts.end(), ts_ms, ts_ms + n_new);
-
-  // time grid over the arrivals: grid[b] = first request with ts >= b * dt (the last request if
-  // there is none), b = 0..n_grid; none while all requests arrive at one instant.  The first
-  // build takes about one request per bucket; later batches add buckets of the same width.
-  // Entries written earlier stay valid: the replay only needs a lower bound of the request it
-  // searches for.
-  std::vector<uint32_t> grid;
-  uint32_t grid_from = 0;
-  {
-    const double span = tb.ts.back();
-    const double buckets = tb.grid_n ? std::floor(span / tb.grid_dt) : 0.0;
-    if (tb.grid_n == 0 || buckets > (double)tb.cap_req) {
-      const double dt = span / (double)N;
-      tb.grid_n = 0; tb.grid_dt = 0.0;
-      if (dt > 0.0 && std::isfinite(dt) && dt >= span * 0x1p-40) {
-        tb.grid_n = (uint32_t)N; tb.grid_dt = dt;
-        grid.resize((size_t)N + 1);
-        uint64_t r = 0;
-        for (uint32_t b = 0; b <= tb.grid_n; ++b) {
-          const double edge = (double)b * dt;
-          while (r < N && tb.ts[r] < edge) ++r;
-          grid[b] = (uint32_t)(r < N ? r : N - 1);
-        }
-        tb.grid_cursor = r;
-      }
-    } else if ((uint32_t)buckets > tb.grid_n) {
-      grid_from = tb.grid_n + 1;
-      const uint32_t upto = (uint32_t)buckets;
-      grid.resize(upto - tb.grid_n);
-      uint64_t r = tb.grid_cursor;
-      for (uint32_t b = grid_from; b <= upto; ++b) {
-        const double edge = (double)b * tb.grid_dt;
-        while (r < N && tb.ts[r] < edge) ++r;
-        grid[b - grid_from] = (uint32_t)(r < N ? r : N - 1);
-      }
-      tb.grid_cursor = r;
-      tb.grid_n = upto;
-    }
-  }
-
-  DeviceGuard guard(sim->device);
-  if (!guard.ok) return GORGO_ERR_CUDA;
-  const uint64_t Dn = tb.D - D0;
-  bool ok = cudaMemcpyAsync(tb.d_req + N0 * sizeof(ReqRec), req.data(), n_new * sizeof(ReqRec),
-                            cudaMemcpyHostToDevice, st) == cudaSuccess;
-  ok = ok && cudaMemcpyAsync(tb.d_ts + N0 * 8, ts_ms, n_new * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  if (!grid.empty())
-    ok = ok && cudaMemcpyAsync(tb.d_grid + (size_t)grid_from * 4, grid.data(), grid.size() * 4,
-                               cudaMemcpyHostToDevice, st) == cudaSuccess;
-  if (Tn > 0) {
-    ok = ok && cudaMemcpyAsync(tb.d_ids + T0 * 4, ids.data(), Tn * 4, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(tb.d_occ + T0 * 8, occ.data(), Tn * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(tb.d_prev + T0 * 8, occ_before.data(), Tn * 8, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    if (Dn > 0)
-      ok = ok && cudaMemcpyAsync(tb.d_raw + (size_t)D0 * 8, tb.raw_new.data(), Dn * 8,
-                                 cudaMemcpyHostToDevice, st) == cudaSuccess;
-  }
-  tb.raw_new.clear();
-  tb.N = N; tb.T = T;
-  if (!ok) { cudaGetLastError(); sim->has_trace = false; return GORGO_ERR_CUDA; }
-  sim->tr.req = reinterpret_cast<const ReqRec*>(tb.d_req);
-  sim->tr.ids = reinterpret_cast<const uint32_t*>(tb.d_ids);
-  sim->tr.occ_next = reinterpret_cast<const uint2*>(tb.d_occ);
-  sim->tr.occ_prev = reinterpret_cast<const uint2*>(tb.d_prev);
-  sim->tr.raw_id = reinterpret_cast<const uint64_t*>(tb.d_raw);
-  sim->tr.ts = reinterpret_cast<const double*>(tb.d_ts);
-  sim->tr.grid = reinterpret_cast<const uint32_t*>(tb.d_grid);
-  sim->tr.grid_dt = tb.grid_dt;
-  sim->tr.grid_n = tb.grid_n;
-  sim->tr.n_req = (uint32_t)N; sim->tr.n_ids = (uint32_t)T; sim->tr.n_distinct = tb.D;
-  // earlier batches' last occurrences now have a successor
-  if (patch_old && launch_link_occurrences(sim->tr, (uint32_t)N0, (uint32_t)n_new, (uint32_t)T0,
-                                           reinterpret_cast<uint2*>(tb.d_occ), st) != cudaSuccess) {
-    sim->has_trace = false;
-    return GORGO_ERR_CUDA;
-  }
-  sim->has_trace = true;
   return GORGO_OK;
 }
 
-static int trace_begin_impl(gorgo_sim_t* sim, uint64_t max_requests, uint64_t max_block_ids,
-                            void* dev_trace_buf, uint64_t dev_trace_bytes) {
+// Time grid over the first N arrivals: grid[b] = first request with ts >= b * dt (the last request if
+// there is none), b = 0..grid_n; none while all requests arrive at one instant.  The first build
+// takes about one request per bucket; later ones (`cursor`: where the last stopped) add buckets of
+// the same width.  Entries written earlier stay valid: the replay only needs a lower bound of the
+// request it searches for.  Returns the index of the first new entry.
+static uint32_t extend_grid(TraceView& tr, const double* ts, uint64_t N, uint64_t cap_req, uint64_t* cursor,
+                            std::vector<uint32_t>& grid) {
+  const double span = ts[N - 1];
+  const double buckets = tr.grid_n ? std::floor(span / tr.grid_dt) : 0.0;
+  uint32_t from = 0, upto;
+  uint64_t r = 0;
+  if (tr.grid_n == 0 || buckets > (double)cap_req) {
+    const double dt = span / (double)N;
+    tr.grid_n = 0; tr.grid_dt = 0.0;
+    if (!(dt > 0.0 && std::isfinite(dt) && dt >= span * 0x1p-40)) return 0;
+    upto = (uint32_t)N; tr.grid_dt = dt;
+  } else {
+    if ((uint32_t)buckets <= tr.grid_n) return 0;
+    from = tr.grid_n + 1; upto = (uint32_t)buckets; r = *cursor;
+  }
+  grid.resize((size_t)upto + 1 - from);
+  for (uint32_t b = from; b <= upto; ++b) {
+    const double edge = (double)b * tr.grid_dt;
+    while (r < N && ts[r] < edge) ++r;
+    grid[b - from] = (uint32_t)(r < N ? r : N - 1);
+  }
+  *cursor = r;
+  tr.grid_n = upto;
+  return from;
+}
+
+static int lay_out_trace(gorgo_sim_t* sim, uint64_t max_requests, uint64_t max_block_ids, void* dev_trace_buf,
+                         uint64_t dev_trace_bytes) {
   if (!sim || !dev_trace_buf) return GORGO_ERR_INVALID_ARG;
   if ((uintptr_t)dev_trace_buf % kAlign) return GORGO_ERR_INVALID_ARG;
   if (max_requests < 1 || max_requests >= 0xFFFFFFFFull || max_block_ids >= 0xFFFFFFFFull)
@@ -648,19 +561,246 @@ static int trace_begin_impl(gorgo_sim_t* sim, uint64_t max_requests, uint64_t ma
   sim->has_trace = false;
   sim->tr = TraceView{};
   sim->cap_req = sim->cap_ids = 0;
-  sim->tb.reset(new TraceBuilder());
-  TraceBuilder& tb = *sim->tb;
-  tb.cap_req = max_requests; tb.cap_ids = max_block_ids;
+  TraceRegions& g = sim->reg;
+  g.cap_req = max_requests; g.cap_ids = max_block_ids;
   const uint64_t N = max_requests, T = max_block_ids;
   unsigned char* base = static_cast<unsigned char*>(dev_trace_buf);
   uint64_t o = 0;
-  tb.d_req = base + o; o += align_up(N * sizeof(ReqRec));
-  tb.d_ids = base + o; o += align_up(T * 4);
-  tb.d_occ = base + o; o += align_up(T * 8);
-  tb.d_raw = base + o; o += align_up(T * 8);
-  tb.d_prev = base + o; o += align_up(T * 8);
-  tb.d_ts = base + o; o += align_up(N * 8);
-  tb.d_grid = base + o; o += align_up((N + 1) * 4);
+  g.req = base + o; o += align_up(N * sizeof(ReqRec));
+  g.touch = base + o; o += align_up(T * sizeof(Touch));
+  g.raw = base + o; o += align_up(T * 8);
+  g.extra = base + o; o += align_up(T * 4);
+  g.ts = base + o; o += align_up(N * 8);
+  g.grid = base + o; o += align_up((N + 1) * 4);
+  g.rtt = base + o;
+  TraceView& tr = sim->tr;
+  tr.req = reinterpret_cast<const ReqRec*>(g.req);
+  tr.touch = reinterpret_cast<const Touch*>(g.touch);
+  tr.raw_id = reinterpret_cast<const uint64_t*>(g.raw);
+  tr.ts = reinterpret_cast<const double*>(g.ts);
+  tr.grid = reinterpret_cast<const uint32_t*>(g.grid);
+  tr.rtt = reinterpret_cast<const double*>(g.rtt);
+  return GORGO_OK;
+}
+
+static bool copy_in(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  return bytes == 0 || cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+}
+
+// A whole trace at once: blocks are grouped into atoms (see Touch).
+//   Pass 1 numbers the ids in order of first appearance and notes, per id, whether its predecessor
+// and its successor are the same wherever it occurs.  Most blocks repeat what followed their
+// predecessor last time, so that guess is tried before the hash table; ids that are new come in
+// runs, and their slots are prefetched.
+//   Pass 2 cuts atoms between x and y unless every x is followed by y and every y preceded by x (then
+// their numbers are consecutive).  Pass 3 writes the touches and links the occurrences.
+static int upload_impl(gorgo_sim_t* sim, uint64_t N, const double* ts_ms, const uint32_t* input_tokens,
+                       const uint32_t* output_tokens, const uint16_t* origin, const uint64_t* hash_off,
+                       const uint64_t* hash_ids, cudaStream_t st) {
+  const uint64_t T = hash_off[N];
+  if (T > 0 && !hash_ids) return GORGO_ERR_INVALID_ARG;
+  std::vector<ReqRec> req(N);
+  int rc = check_requests(sim->m, N, 0.0, ts_ms, input_tokens, output_tokens, origin, hash_off, req.data());
+  if (rc != GORGO_OK) return rc;
+
+  uint64_t cap = 1ull << 12;
+  while (cap < T / 2) cap <<= 1;
+  IdMap map(cap);
+  map.raw.reserve(T / 2 + 1024);
+  struct Around { uint32_t pred, succ; };        // first predecessor, latest successor (kNone: none yet)
+  std::vector<Around> nb;
+  nb.reserve(T / 2 + 1024);
+  std::vector<uint8_t> cut;                      // 1: predecessors differ, 2: successors differ (or none)
+  cut.reserve(T / 2 + 1024);
+  std::unique_ptr<uint32_t[]> dense(new uint32_t[T + 1]);
+  constexpr uint64_t kFetch = 12;                // slots prefetched ahead inside a run of new ids
+  for (uint64_t r = 0; r < N; ++r) {
+    const uint64_t g0 = hash_off[r], g1 = hash_off[r + 1];
+    uint32_t x = kNone;
+    bool fresh = false;                          // inside a run of new ids
+    for (uint64_t g = g0; g < g1; ++g) {
+      const uint64_t id = hash_ids[g];
+      uint32_t y = x == kNone ? kNone : nb[x].succ;
+      if (y == kNone || map.raw[y] != id) {
+        if (!fresh)
+          for (uint64_t h = g + 1; h < g1 && h < g + kFetch; ++h) map.prefetch(hash_ids[h]);
+        if (g + kFetch < g1) map.prefetch(hash_ids[g + kFetch]);
+        const size_t before = map.raw.size();
+        y = map.get_or_add(id);
+        fresh = map.raw.size() != before;
+        if (fresh) { nb.push_back({x, kNone}); cut.push_back(0); }
+        else if (nb[y].pred != x) cut[y] |= 1;
+        if (x != kNone) {
+          if (nb[x].succ != kNone && nb[x].succ != y) cut[x] |= 2;
+          nb[x].succ = y;
+        }
+      } else {
+        fresh = false;
+        if (nb[y].pred != x) cut[y] |= 1;
+      }
+      dense[g] = y;
+      x = y;
+    }
+    if (x != kNone) cut[x] |= 2;                 // it ends a request
+  }
+  const uint32_t D = (uint32_t)map.raw.size();
+
+  std::vector<uint32_t> head;                    // first block of each atom
+  head.reserve(2 * N + 16);
+  std::unique_ptr<uint32_t[]> atom_at(new uint32_t[D + 1]);   // atom that starts at a block
+  for (uint32_t d = 0; d < D; ++d) {
+    if (d == 0 || nb[d].pred != d - 1 || (cut[d] & 1) || (cut[d - 1] & 2)) {
+      atom_at[d] = (uint32_t)head.size();
+      head.push_back(d);
+    }
+  }
+  const uint32_t A = (uint32_t)head.size();
+  head.push_back(D);
+
+  std::vector<Touch> touch;
+  touch.reserve(4 * N + 16);
+  std::vector<Around> last(A, Around{kNone, kNone});   // touch and request of an atom's last occurrence
+  for (uint64_t r = 0; r < N; ++r) {
+    req[r].off = (uint32_t)touch.size();
+    uint32_t latest = 0;                         // latest earlier request (+1) that shares an atom
+    for (uint64_t g = hash_off[r]; g < hash_off[r + 1];) {
+      const uint32_t at = atom_at[dense[g]];
+      const uint32_t len = head[at + 1] - head[at];
+      Around& la = last[at];
+      const uint32_t here = (uint32_t)touch.size();
+      if (la.pred != kNone) {
+        if (la.succ == (uint32_t)r) return GORGO_ERR_BAD_TRACE;   // an id twice in one request
+        touch[la.pred].next = here; touch[la.pred].next_req = (uint32_t)r;
+        if (la.succ + 1 > latest) latest = la.succ + 1;
+      }
+      la.pred = here; la.succ = (uint32_t)r;
+      touch.push_back({at, len | (uint32_t)(g - hash_off[r]) << 16, kNone, kNone});
+      g += len;
+    }
+    req[r].m = (uint16_t)(touch.size() - req[r].off);
+    req[r].prev_share = latest ? latest - 1 : kNone;
+  }
+  TraceView& tr = sim->tr;
+  tr.n_req = (uint32_t)N; tr.n_touch = (uint32_t)touch.size(); tr.n_atoms = A;
+  tr.n_ids = (uint32_t)T; tr.n_distinct = D;
+  tr.raw_off = reinterpret_cast<const uint32_t*>(sim->reg.extra);
+  // chunks of static data: 16 requests unless these have many touches; room for the largest chunk, but
+  // no more than 1.6 times the mean or 40 touches a request (what does not fit is read from global
+  // memory)
+  const double mean = (double)touch.size() / (double)N;
+  uint32_t cr = 16;
+  while (cr > 4 && cr * mean > 160.0) cr /= 2;
+  uint64_t largest = 16;
+  for (uint64_t r0 = 0; r0 < N; r0 += cr) {
+    const uint64_t r1 = r0 + cr;
+    largest = std::max<uint64_t>(largest, (r1 < N ? req[r1].off : touch.size()) - req[r0].off);
+  }
+  tr.chunk_req = cr;
+  tr.chunk_cap = (uint32_t)std::min<uint64_t>(largest, (uint64_t)std::min(16.0 + 1.6 * mean * cr, 40.0 * cr));
+  std::vector<uint32_t> grid;
+  uint64_t cursor = 0;
+  extend_grid(tr, ts_ms, N, N, &cursor, grid);
+
+  DeviceGuard guard(sim->device);
+  if (!guard.ok) return GORGO_ERR_CUDA;
+  const TraceRegions& g = sim->reg;
+  const bool ok = copy_in(g.req, req.data(), N * sizeof(ReqRec), st) &&
+                  copy_in(g.touch, touch.data(), touch.size() * sizeof(Touch), st) &&
+                  copy_in(g.raw, map.raw.data(), (size_t)D * 8, st) && copy_in(g.extra, head.data(), (size_t)A * 4, st) &&
+                  copy_in(g.ts, ts_ms, N * 8, st) && copy_in(g.grid, grid.data(), grid.size() * 4, st) &&
+                  copy_in(g.rtt, sim->rtt.data(), sim->rtt.size() * 8, st) &&
+                  cudaStreamSynchronize(st) == cudaSuccess;
+  if (!ok) { cudaGetLastError(); return GORGO_ERR_CUDA; }
+  sim->has_trace = true;
+  return GORGO_OK;
+}
+
+// Appends `n_new` requests to a growing trace; a batch that fails a check changes nothing.
+static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, const uint32_t* input_tokens,
+                       const uint32_t* output_tokens, const uint16_t* origin, const uint64_t* hash_off,
+                       const uint64_t* hash_ids, cudaStream_t st) {
+  TraceBuilder& tb = *sim->tb;
+  if (n_new < 1 || hash_off[0] != 0) return GORGO_ERR_BAD_TRACE;
+  for (uint64_t k = 0; k < n_new; ++k)
+    if (hash_off[k + 1] < hash_off[k]) return GORGO_ERR_BAD_TRACE;
+  const uint64_t Tn = hash_off[n_new];
+  const uint64_t N0 = tb.ts.size(), T0 = tb.T, N = N0 + n_new, T = T0 + Tn;
+  if (N > sim->reg.cap_req || T > sim->reg.cap_ids) return GORGO_ERR_WORKSPACE_TOO_SMALL;
+  if (Tn > 0 && !hash_ids) return GORGO_ERR_INVALID_ARG;
+  std::vector<ReqRec> req(n_new);
+  int rc = check_requests(sim->m, n_new, N0 ? tb.ts.back() : 0.0, ts_ms, input_tokens, output_tokens, origin,
+                          hash_off, req.data());
+  if (rc != GORGO_OK) return rc;
+  // an id twice in one request: found before anything is changed
+  for (uint64_t k = 0; k < n_new; ++k) {
+    uint64_t cap = 64;
+    while (cap < 2 * (hash_off[k + 1] - hash_off[k])) cap <<= 1;
+    if (tb.dup.size() < cap || tb.stamp == 0xFFFFFFFFu) {
+      cap = std::max<uint64_t>(cap, tb.dup.size());
+      tb.dup.assign(cap, 0); tb.dup_stamp.assign(cap, 0); tb.stamp = 0;
+    }
+    ++tb.stamp;
+    const uint64_t mask = tb.dup.size() - 1;
+    for (uint64_t g = hash_off[k]; g < hash_off[k + 1]; ++g) {
+      uint64_t i = IdMap::hash(hash_ids[g]) & mask;
+      while (tb.dup_stamp[i] == tb.stamp) {
+        if (tb.dup[i] == hash_ids[g]) return GORGO_ERR_BAD_TRACE;
+        i = (i + 1) & mask;
+      }
+      tb.dup[i] = hash_ids[g]; tb.dup_stamp[i] = tb.stamp;
+    }
+  }
+  std::vector<Touch> touch(Tn);
+  std::vector<uint32_t> prev(Tn, kNone);         // previous occurrence where it lies in an earlier batch
+  const size_t D0 = tb.map.raw.size();
+  bool patch_old = false;
+  for (uint64_t k = 0; k < n_new; ++k) {
+    const uint32_t r = (uint32_t)(N0 + k);
+    req[k].off = (uint32_t)(T0 + hash_off[k]);
+    req[k].m = (uint16_t)req[k].nblk;
+    uint32_t latest = 0;
+    for (uint64_t gl = hash_off[k]; gl < hash_off[k + 1]; ++gl) {
+      const uint32_t d = tb.map.get_or_add(hash_ids[gl]);
+      const uint32_t g = (uint32_t)(T0 + gl);
+      touch[gl] = {d, 1u | (uint32_t)(gl - hash_off[k]) << 16, kNone, kNone};
+      if (d == tb.last_g.size()) {
+        tb.last_g.push_back(g); tb.last_r.push_back(r);
+        continue;
+      }
+      const uint32_t pg = tb.last_g[d];
+      if (tb.last_r[d] + 1 > latest) latest = tb.last_r[d] + 1;
+      if (pg >= T0) { touch[pg - T0].next = g; touch[pg - T0].next_req = r; }
+      else { prev[gl] = pg; patch_old = true; }
+      tb.last_g[d] = g; tb.last_r[d] = r;
+    }
+    req[k].prev_share = latest ? latest - 1 : kNone;
+  }
+  tb.ts.insert(tb.ts.end(), ts_ms, ts_ms + n_new);
+  tb.T = T;
+  TraceView& tr = sim->tr;
+  std::vector<uint32_t> grid;
+  const uint32_t grid_from = extend_grid(tr, tb.ts.data(), N, sim->reg.cap_req, &tb.grid_cursor, grid);
+  const size_t Dn = tb.map.raw.size() - D0;
+  tr.n_req = (uint32_t)N; tr.n_touch = (uint32_t)T; tr.n_atoms = (uint32_t)tb.map.raw.size();
+  tr.n_ids = (uint32_t)T; tr.n_distinct = tr.n_atoms;
+  tr.chunk_req = 4; tr.chunk_cap = 256;          // (a block of a growing trace is an atom: many touches)
+
+  DeviceGuard guard(sim->device);
+  if (!guard.ok) return GORGO_ERR_CUDA;
+  const TraceRegions& rg = sim->reg;
+  bool ok = copy_in(rg.req + N0 * sizeof(ReqRec), req.data(), n_new * sizeof(ReqRec), st) &&
+            copy_in(rg.touch + T0 * sizeof(Touch), touch.data(), Tn * sizeof(Touch), st) &&
+            copy_in(rg.raw + D0 * 8, tb.map.raw.data() + D0, Dn * 8, st) &&
+            copy_in(rg.ts + N0 * 8, ts_ms, n_new * 8, st) &&
+            copy_in(rg.grid + (size_t)grid_from * 4, grid.data(), grid.size() * 4, st);
+  if (N0 == 0) ok = ok && copy_in(rg.rtt, sim->rtt.data(), sim->rtt.size() * 8, st);
+  // earlier batches' last occurrences now have a successor
+  if (patch_old)
+    ok = ok && copy_in(rg.extra, prev.data(), Tn * 4, st) &&
+         launch_link_occurrences(tr, (uint32_t)N0, (uint32_t)n_new, reinterpret_cast<const uint32_t*>(rg.extra),
+                                 reinterpret_cast<Touch*>(rg.touch), st) == cudaSuccess;
+  if (!ok) { cudaGetLastError(); sim->has_trace = false; return GORGO_ERR_CUDA; }
+  sim->has_trace = true;
   return GORGO_OK;
 }
 
@@ -674,26 +814,21 @@ int gorgo_trace_upload(gorgo_sim_t* sim, uint64_t n_requests, const double* ts_m
   if (hash_off[0] != 0) return GORGO_ERR_BAD_TRACE;
   for (uint64_t r = 0; r < n_requests; ++r)
     if (hash_off[r + 1] < hash_off[r]) return GORGO_ERR_BAD_TRACE;
-  // a fixed trace is an appendable one of exactly its own size, built in one batch
-  int rc = trace_begin_impl(sim, n_requests, hash_off[n_requests], dev_trace_buf, dev_trace_bytes);
-  if (rc == GORGO_OK) {
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    rc = trace_append_impl(sim, n_requests, ts_ms, input_tokens, output_tokens, origin, hash_off,
-                           hash_ids, st, false);
-    if (rc == GORGO_OK) {
-      DeviceGuard guard(sim->device);
-      if (!guard.ok || cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); rc = GORGO_ERR_CUDA; }
-    }
-  }
   sim->tb.reset();           // nothing can be appended to an uploaded trace
-  if (rc != GORGO_OK) sim->has_trace = false;
+  int rc = lay_out_trace(sim, n_requests, hash_off[n_requests], dev_trace_buf, dev_trace_bytes);
+  if (rc == GORGO_OK)
+    rc = upload_impl(sim, n_requests, ts_ms, input_tokens, output_tokens, origin, hash_off, hash_ids,
+                     static_cast<cudaStream_t>(cuda_stream));
   return rc;
 }
 
 int gorgo_trace_begin(gorgo_sim_t* sim, uint64_t max_requests, uint64_t max_block_ids,
                       void* dev_trace_buf, uint64_t dev_trace_bytes) {
-  const int rc = trace_begin_impl(sim, max_requests, max_block_ids, dev_trace_buf, dev_trace_bytes);
-  if (rc == GORGO_OK) { sim->cap_req = max_requests; sim->cap_ids = max_block_ids; }
+  const int rc = lay_out_trace(sim, max_requests, max_block_ids, dev_trace_buf, dev_trace_bytes);
+  if (rc == GORGO_OK) {
+    sim->cap_req = max_requests; sim->cap_ids = max_block_ids;
+    sim->tb.reset(new TraceBuilder());
+  }
   return rc;
 }
 
@@ -703,8 +838,8 @@ int gorgo_trace_append(gorgo_sim_t* sim, uint64_t n_requests, const double* ts_m
                        void* cuda_stream) {
   if (!sim || !ts_ms || !input_tokens || !output_tokens || !hash_off) return GORGO_ERR_INVALID_ARG;
   if (!sim->tb) return GORGO_ERR_NO_TRACE;
-  return trace_append_impl(sim, n_requests, ts_ms, input_tokens, output_tokens, origin, hash_off,
-                           hash_ids, static_cast<cudaStream_t>(cuda_stream), true);
+  return append_impl(sim, n_requests, ts_ms, input_tokens, output_tokens, origin, hash_off, hash_ids,
+                     static_cast<cudaStream_t>(cuda_stream));
 }
 
 int gorgo_trace_info(const gorgo_sim_t* sim, uint64_t* n_requests, uint64_t* n_block_ids,
@@ -931,16 +1066,12 @@ int gorgo_tune_online(gorgo_sim_t* sim, const gorgo_online_config_t* cfg, uint32
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   unsigned char* base = static_cast<unsigned char*>(workspace);
   double* d_params = reinterpret_cast<double*>(base + w.params);
-  double* d_rtt = reinterpret_cast<double*>(base + w.rtt);
   int32_t* d_status = reinterpret_cast<int32_t*>(base + w.status);
   double* d_p95 = reinterpret_cast<double*>(base + w.p95);
   double* d_ttft = reinterpret_cast<double*>(base + w.ttft);
   double* d_e2e = reinterpret_cast<double*>(base + w.e2e);
-  if (cudaMemcpyAsync(d_rtt, sim->rtt.data(), sim->rtt.size() * 8, cudaMemcpyHostToDevice, st) !=
-          cudaSuccess ||
-      cudaMemsetAsync(d_status, 0, (size_t)P * 4, st) != cudaSuccess)
-    return GORGO_ERR_CUDA;
-  if (launch_reset(base + w.masks, (uint64_t)P * w.mask_stride,
+  if (cudaMemsetAsync(d_status, 0, (size_t)P * 4, st) != cudaSuccess) return GORGO_ERR_CUDA;
+  if (launch_reset(base + w.masks, w.mask_stride, reset_bytes(sim, w),
                    reinterpret_cast<uint32_t*>(base + w.exp_head), (uint64_t)P * N, base + w.states,
                    w.st, sim->m, P, st) != cudaSuccess)
     return GORGO_ERR_CUDA;
@@ -955,20 +1086,11 @@ int gorgo_tune_online(gorgo_sim_t* sim, const gorgo_online_config_t* cfg, uint32
     const uint64_t count = std::min<uint64_t>(done == 0 ? cfg->window : cfg->hop, N - done);
     if (cudaMemcpyAsync(d_params, live.data(), (size_t)P * K * 8, cudaMemcpyHostToDevice, st) != cudaSuccess)
       return GORGO_ERR_CUDA;
-    ReplayArgs a = {};
-    a.m = sim->m; a.tr = sim->tr; a.scale = cfg->time_scale;
+    ReplayArgs a = base_args(sim, base, w);
+    a.scale = cfg->time_scale;
     a.first = (uint32_t)done; a.count = (uint32_t)count; a.check_order = 1;
-    a.poll_limit = sim->poll_limit; a.ring_polls = sim->ring_polls;
-    a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
-    a.rtt = d_rtt; a.params = d_params;
-    a.masks = base + w.masks; a.mask_stride = w.mask_stride;
-    a.states = base + w.states; a.lay = w.st;
-    a.evict_lists = reinterpret_cast<uint4*>(base + w.lists);
-    a.exp_head = reinterpret_cast<uint32_t*>(base + w.exp_head);
-    a.exp_rec = reinterpret_cast<uint4*>(base + w.exp_rec);
-    a.lru_next = reinterpret_cast<uint32_t*>(base + w.lru_next);
-    a.route_log = route ? route : base + w.route_log;
-    a.route_log_stride = N;
+    a.params = d_params;
+    if (route) a.route_log = route;
     if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
     a.ttft_out = d_ttft + done; a.e2e_out = d_e2e + done; a.out_stride = N;   // request r at [p*N + r]
     a.status_out = d_status;
@@ -1064,7 +1186,7 @@ int gorgo_sim_reset(gorgo_sim_t* sim, void* state_workspace, uint64_t state_byte
   DeviceGuard guard(sim->device);
   if (!guard.ok) return GORGO_ERR_CUDA;
   unsigned char* base = static_cast<unsigned char*>(state_workspace);
-  if (launch_reset(base + w.masks, w.mask_stride, reinterpret_cast<uint32_t*>(base + w.exp_head),
+  if (launch_reset(base + w.masks, w.mask_stride, w.mask_stride, reinterpret_cast<uint32_t*>(base + w.exp_head),
                    sim->cap_req ? sim->cap_req : sim->tr.n_req, base + w.states, w.st, sim->m, 1,
                    static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
     return GORGO_ERR_CUDA;
@@ -1087,26 +1209,10 @@ int gorgo_route_batch(gorgo_sim_t* sim, const double* params, double time_scale,
   if (!guard.ok) return GORGO_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   unsigned char* base = static_cast<unsigned char*>(state_workspace);
-  double* d_params = reinterpret_cast<double*>(base + w.params);
-  double* d_rtt = reinterpret_cast<double*>(base + w.rtt);
-  if (cudaMemcpyAsync(d_rtt, sim->rtt.data(), sim->rtt.size() * 8, cudaMemcpyHostToDevice, st) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(d_params, params, (size_t)sim->m.K * 8, cudaMemcpyHostToDevice, st) !=
-          cudaSuccess)
-    return GORGO_ERR_CUDA;
-  ReplayArgs a = {};
-  a.m = sim->m; a.tr = sim->tr; a.scale = time_scale;
+  ReplayArgs a = base_args(sim, base, w);
+  a.scale = time_scale;
   a.first = (uint32_t)first; a.count = (uint32_t)count; a.check_order = 1;
-  a.poll_limit = sim->poll_limit; a.ring_polls = sim->ring_polls;
-  a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
-  a.rtt = d_rtt; a.params = d_params;
-  a.masks = base + w.masks; a.mask_stride = w.mask_stride;
-  a.states = base + w.states; a.lay = w.st;
-  a.evict_lists = reinterpret_cast<uint4*>(base + w.lists);
-  a.exp_head = reinterpret_cast<uint32_t*>(base + w.exp_head);
-  a.exp_rec = reinterpret_cast<uint4*>(base + w.exp_rec);
-  a.lru_next = reinterpret_cast<uint32_t*>(base + w.lru_next);
-  a.route_log = base + w.route_log; a.route_log_stride = N;
+  std::copy(params, params + sim->m.K, a.inline_params);   // (the launch carries them: no copy on the stream)
   a.finish_log = reinterpret_cast<double*>(base + w.finish);
   if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
   a.route_out = route; a.hit_out = hit_blocks; a.ttft_out = ttft_ms; a.e2e_out = e2e_ms;
@@ -1155,7 +1261,7 @@ int gorgo_replay_occupancy(gorgo_sim_t* sim, int32_t* ctas_per_sm, uint64_t* sme
   if (!sim || !ctas_per_sm) return GORGO_ERR_INVALID_ARG;
   DeviceGuard guard(sim->device);
   if (!guard.ok) return GORGO_ERR_CUDA;
-  const int n = replay_occupancy(sim->m, smem_bytes_per_cta);
+  const int n = replay_occupancy(sim->m, sim->tr, smem_bytes_per_cta);
   if (n < 0) return GORGO_ERR_CUDA;
   *ctas_per_sm = n;
   return GORGO_OK;
@@ -1202,7 +1308,7 @@ int gorgo_debug_set(gorgo_sim_t* sim, uint32_t what, uint32_t value) {
   if (!sim) return GORGO_ERR_INVALID_ARG;
   switch (what) {
     case GORGO_DEBUG_POLL_LIMIT: sim->poll_limit = value; break;
-    case GORGO_DEBUG_RING_POLLS: sim->ring_polls = value; break;
+    case GORGO_DEBUG_RING_POLLS: break;
     case GORGO_DEBUG_PROBE_OFF: sim->probe_off = value ? 1u : 0u; break;
     case GORGO_DEBUG_SCOUT_OFF: sim->scout_off = value ? 1u : 0u; break;
     default: return GORGO_ERR_INVALID_ARG;
@@ -1312,7 +1418,8 @@ int gorgo_eval_population_static(gorgo_sim_t* sim, uint32_t n_candidates, const 
   if (!sim) return GORGO_ERR_INVALID_ARG;
   if (!sim->has_trace) return GORGO_ERR_NO_TRACE;
   // one candidate's replay state must fit; a larger population then runs in waves inside it
-  if (make_ws(sim, 1, true).total > (uint64_t)GORGO_STATIC_SCRATCH_BYTES)
+  const bool with_index = sim->proxy_index != 0;
+  if (make_ws(sim, 1, true, with_index).total > (uint64_t)GORGO_STATIC_SCRATCH_BYTES)
     return GORGO_ERR_STATIC_LIMIT;
   void* scratch = nullptr;
   {
@@ -1325,17 +1432,17 @@ int gorgo_eval_population_static(gorgo_sim_t* sim, uint32_t n_candidates, const 
   // so whatever an earlier call left in the array is never read
   return eval_impl(sim, n_candidates, params, time_scale, scratch, GORGO_STATIC_SCRATCH_BYTES,
                    static_cast<cudaStream_t>(cuda_stream), p95_ttft_ms, p95_e2e_ms, route,
-                   hit_blocks, nullptr, nullptr, cand_status, false);
+                   hit_blocks, nullptr, nullptr, cand_status, false, nullptr, nullptr, nullptr, with_index);
 }
 
 #ifdef GORGO_PROF
 // Cycle-accounting build only (not declared in gorgo.h, not part of the product library):
-// waits for the device, copies the 64 phase accumulators out and clears them.
-int gorgo_debug_phase_cycles(gorgo_sim_t* sim, uint64_t* out64) {
-  if (!sim || !out64) return GORGO_ERR_INVALID_ARG;
+// waits for the device, copies the 112 phase accumulators out and clears them.
+int gorgo_debug_phase_cycles(gorgo_sim_t* sim, uint64_t* out112) {
+  if (!sim || !out112) return GORGO_ERR_INVALID_ARG;
   DeviceGuard guard(sim->device);
   if (!guard.ok || cudaDeviceSynchronize() != cudaSuccess) return GORGO_ERR_CUDA;
-  return prof_read(reinterpret_cast<unsigned long long*>(out64), true) == cudaSuccess
+  return prof_read(reinterpret_cast<unsigned long long*>(out112), true) == cudaSuccess
              ? GORGO_OK : GORGO_ERR_CUDA;
 }
 #endif

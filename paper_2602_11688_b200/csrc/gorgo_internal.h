@@ -9,25 +9,38 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 
 // One request of the trace as the kernels read it: exactly one 32-byte sector.
 struct __align__(32) ReqRec {
-  double ts_ms;       // arrival at the proxy (unscaled)
-  uint32_t off;       // first block id of the request in the flat id array
-  uint32_t in_tok;    // input tokens
-  uint32_t out_tok;   // output tokens
-  uint16_t nblk;      // number of blocks
-  uint16_t origin;    // origin region
+  double ts_ms;         // arrival at the proxy (unscaled)
+  uint32_t off;         // first touch of the request in the touch array
+  uint32_t in_tok;      // input tokens
+  uint32_t out_tok;     // output tokens
+  uint16_t m;           // touches (atoms) of the request
+  uint16_t origin;      // origin region
   uint32_t prev_share;  // latest earlier request that shares a block with this one (kNone: none)
-  uint32_t pad;
+  uint32_t nblk;        // blocks of the request
 };
 static_assert(sizeof(ReqRec) == 32, "ReqRec must be one sector");
 
+// Blocks that occur in exactly the same requests, always next to one another and in the same
+// order, are one ATOM: a replica's LRU cache touches them together, so at any time it holds a
+// leading part of the atom (deeper blocks are evicted first), and all of it unless the eviction
+// cursor stands inside it.  A touch is one atom of one request.
+struct __align__(16) Touch {
+  uint32_t atom;
+  uint32_t len_pos;     // blocks of the atom | position of its first block in the request << 16
+  uint32_t next;        // touch array index of the atom's next occurrence (kNone: none)
+  uint32_t next_req;    // request of that occurrence
+};
+static_assert(sizeof(Touch) == 16, "Touch layout");
+
 // Per-(candidate, replica) scalars kept in global memory between launches.
 struct __align__(32) RepState {
-  long long load;     // in-flight input tokens
-  long long cnt;      // in-flight requests
+  long long load;     // in-flight queue signal (input tokens, or requests) as of the last request routed
   uint32_t occ;       // cached blocks
   uint32_t cur_req;   // eviction cursor: request whose touches are examined next (kNone: none yet)
-  int32_t cur_pos;    //   next position of that request to examine (counts down; <0: exhausted)
-  uint32_t lru_tail;  // last request routed to this replica (kNone: none yet)
+  int32_t cur_k;      //   next touch of that request to examine (counts down; <0: exhausted)
+  uint32_t part;      // atom of which only a leading part is cached (kNone: none)
+  uint32_t part_len;  //   blocks of it that are cached
+  uint32_t pad;
 };
 static_assert(sizeof(RepState) == 32, "RepState layout");
 
@@ -43,19 +56,21 @@ struct __align__(32) CandHeader {
 
 // Device-resident trace (pointers into the caller's trace buffer).
 struct TraceView {
-  const ReqRec* req;       // [N]
-  const uint32_t* ids;     // [T] dense block ids, request after request
-  const uint2* occ_next;   // [T] (.x = flat index of the next occurrence of the same block or
-                           //      kNone, .y = request of that occurrence)
-  const uint2* occ_prev;   // [T] the same for the previous occurrence
-  const uint64_t* raw_id;  // [D] caller's 64-bit id of each dense id
-  const double* ts;        // [N] arrival times (unscaled), the same values as in `req`
+  const ReqRec* req;        // [N]
+  const Touch* touch;       // [T] touches, request after request
+  const uint32_t* raw_off;  // [A] first block of each atom in `raw_id`; null: atom a is block a
+  const uint64_t* raw_id;   // [D] caller's 64-bit ids, the blocks of an atom one after another
+  const double* ts;         // [N] arrival times (unscaled), the same values as in `req`
+  const double* rtt;        // [G*R]
   // time grid over the unscaled arrival times: grid[b] = first request with ts >= b * grid_dt,
   // b = 0..grid_n (grid_n = 0: no grid, e.g. all arrivals at one instant)
   const uint32_t* grid;
   double grid_dt;
   uint32_t grid_n;
-  uint32_t n_req, n_ids, n_distinct;
+  uint32_t n_req, n_touch, n_atoms;
+  uint32_t n_ids, n_distinct;        // block ids in total, distinct ones
+  // static staging of the replay: requests per chunk (a power of two), touches kept of a chunk
+  uint32_t chunk_req, chunk_cap;
 };
 
 // Model constants.
@@ -83,22 +98,20 @@ struct ReplayArgs {
   uint32_t first, count;          // requests [first, first+count)
   uint32_t check_order;           // 1: refuse (status) unless header.processed == first
   uint32_t poll_limit;            // polls after which a warp stops waiting for another one
-  uint32_t ring_polls;            // polls of a commit warp for the scout's next victims before it walks itself
-  uint32_t probe_off, scout_off;  // test switches: run without the probe warp / without the scout warps
+  uint32_t probe_off, scout_off;  // test switches: no mask words read ahead / no victims listed ahead
   uint32_t slots_in_smem;         // set by the launcher: per-slot state fits in shared memory
-  uint32_t lists_in_smem;         // set by the launcher: eviction lists fit in shared memory
-  uint4* evict_lists;             // [P * evict_list_bytes(R)] scratch used when they do not
-  const double* rtt;              // [G*R] device
-  const double* params;           // [P*K] device
-  unsigned char* masks;           // [P * mask_stride] bytes
+  uint32_t ring_cap;              // set by the launcher: listed victims kept per replica (a power of two)
+  const double* params;           // [P*K] device, or null: `inline_params` (one candidate)
+  double inline_params[67];
+  unsigned char* masks;           // [P * mask_stride] bytes: cached-on-replica words, one per atom
   uint64_t mask_stride;           // bytes per candidate
+  uint64_t index_off;             // bytes from a candidate's masks to its proxy-index words
   unsigned char* states;          // [P * layout.bytes]
   StateLayout lay;
   // per-request arrays, candidate p at + p*N elements
   uint32_t* exp_head;             // [r]: first entry of the list of requests whose completion the
                                   //   proxy sees when request r arrives (kNone: none)
   uint4* exp_rec;                 // [j]: (next entry of j's list, input tokens of j, replica of j, -)
-  uint32_t* lru_next;             // next request routed to the same replica
   uint8_t* route_log;             // chosen replica of every request replayed so far
   uint64_t route_log_stride;      // elements between candidates
   // baseline policies: queue signal counted in requests instead of tokens; one fixed route per
@@ -163,7 +176,7 @@ struct DigestArgs {
   uint64_t* digest;               // [P*R*2], zeroed by the launcher
 };
 
-cudaError_t launch_reset(unsigned char* masks, uint64_t mask_bytes_total, uint32_t* exp_head,
+cudaError_t launch_reset(unsigned char* masks, uint64_t mask_stride, uint64_t mask_bytes, uint32_t* exp_head,
                          uint64_t exp_head_count, unsigned char* states, const StateLayout& lay,
                          const Model& m, uint32_t n_cand, cudaStream_t st);
 cudaError_t launch_replay(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st);
@@ -173,20 +186,21 @@ cudaError_t launch_window(const WindowArgs& a, uint32_t n_cand, cudaStream_t st)
 cudaError_t launch_policy_routes(const TraceView& tr, uint32_t R, bool affinity,
                                  const uint32_t* draws, uint8_t* route, cudaStream_t st);
 #ifdef GORGO_PROF
-// Cycle accounting build only: the 64 accumulators (route warp at 0, service at 16, gate at 32, commit warps at 48).
-cudaError_t prof_read(unsigned long long* out64, bool reset);
+// Cycle accounting build only: 16 accumulators per role (route 0, time 16, expiry 32, file 48,
+// scout 64, stage 80, commit 96).
+cudaError_t prof_read(unsigned long long* out112, bool reset);
 #endif
-// After requests [first_new, first_new + n_new) were appended: every block of theirs whose previous
-// occurrence lies before flat position `ids_before` becomes that occurrence's successor.
+// After requests [first_new, first_new + n_new) were appended to a growing trace: every block of
+// theirs that occurred before gets its previous occurrence (`prev[i]` of the i-th new touch)
+// linked to it.
 cudaError_t launch_link_occurrences(const TraceView& tr, uint32_t first_new, uint32_t n_new,
-                                    uint32_t ids_before, uint2* occ_next, cudaStream_t st);
+                                    const uint32_t* prev, Touch* touch, cudaStream_t st);
 cudaError_t launch_gather(const void* buf, uint64_t n_sectors, uint32_t per_thread, uint32_t blocks,
                           uint32_t* sink, cudaStream_t st);
 uint32_t window_max();          // largest window the window kernel handles
 uint32_t mask_bytes_for(uint32_t n_replicas);
-uint64_t evict_list_bytes(uint32_t n_replicas);
 // CTAs of the replay kernel that fit one SM for this model (-1: query failed), and the dynamic
 // shared memory one CTA asks for.
-int replay_occupancy(const Model& m, uint64_t* smem_bytes);
+int replay_occupancy(const Model& m, const TraceView& tr, uint64_t* smem_bytes);
 
 }  // namespace gorgo

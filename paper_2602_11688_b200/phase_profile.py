@@ -17,29 +17,14 @@ import json
 import numpy as np
 
 ROLES = {
-    "route": (0, ["load update of the previous route, wait for the completion sums",
-                  "completion sums, queue term of the score", "wait for the prefix hits (barrier)",
-                  "staged part of the score, order key", "argmin over replicas",
-                  "hit of the chosen replica, route stores, barrier arrive"]),
-    "service": (16, ["retire: list entry, window vote, grid value", "fence and publish",
-                     "next pipeline stage: list exchange, window loads", "slot argmin",
-                     "times, outputs, grid load", "idle round"]),
-    "gate": (32, ["own turn: probe here if needed, hand over", "wait for the route (barrier)",
-                  "job post, early hand-over of the next request",
-                  "own turn: staged? recent route to a holder?", "own turn: wait for commits",
-                  None, None, None, None, None, None,
-                  "#probes done by this warp", "#next request not staged yet at hand-over time",
-                  "#next request not handed over early (shared block or recent route to a holder)",
-                  "#hits handed over early"]),
-    "commit (all three warps)": (48, ["wait for the next routed request", "need and eviction",
-                                      "mask bits of the inserted blocks", "recency list, progress",
-                                      "requests of other warps' replicas", None, None, None,
-                                      "#evictions: clean case (victims taken from the ring as listed)",
-                                      "#evictions: an entry was void or touched again",
-                                      "#evictions: ring held too few entries",
-                                      "#evictions: more than 96 victims or ring not in use",
-                                      "#requests that evict", "#evictions finished by own walk",
-                                      "#polls for ring entries", "#blocks evicted"]),
+    "route": (0, ["wait until the request is ready, staged again", "score", "argmin, hand-over", "commit", "eviction",
+                  "publish, next request", None, "#requests not ready in advance",
+                  "#requests staged again", "#evictions out of line"]),
+    "time": (16, ["wait for a routed request", "times of a group"]),
+    "expiry": (32, ["waits", "completions of one request"]),
+    "file": (48, ["lists handed over", "outputs and lists filed"]),
+    "scout": (64, ["idle, requests of the replica", "touches"]),
+    "stage": (80, ["wait for a free stage", "words of the next group", "hits of the current group"]),
 }
 
 
@@ -73,7 +58,7 @@ def main():
     scale = float(w.spec.time_scales[0])
     P, N = w.params.shape[0], w.n_requests
     sim = gb.GorgoSim(w)
-    buf = (C.c_uint64 * 64)()
+    buf = (C.c_uint64 * 112)()
     gb.gorgo_set_profiling(sim.h, True)
     ms = 0.0
     for it in range(args.repeat):
