@@ -125,6 +125,7 @@ StateLayout make_layout(const Model& m) {
   const uint64_t rs = (uint64_t)m.R * m.S;
   l.slot_off = o; o += rs * 8;
   l.slot_kv_off = o; o += rs * 8;
+  l.more_off = o = (o + 15u) & ~15ull; if (m.R > 32) o += (uint64_t)m.R * 16 * 16;   // (16 listed victims a replica)
   l.bytes = align_up(o);
   return l;
 }

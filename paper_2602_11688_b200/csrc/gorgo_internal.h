@@ -86,6 +86,7 @@ struct StateLayout {
   uint64_t rep_off;        // RepState[R]
   uint64_t slot_off;       // double[R*S]: time each slot frees (finish of its newest request)
   uint64_t slot_kv_off;    // uint64[R*S]: KV tokens held by each slot's newest request
+  uint64_t more_off;       // more than 32 replicas: what is rarely needed of the listed victims
   uint64_t bytes;          // size of the block (multiple of 256)
 };
 

@@ -27,8 +27,8 @@
 // Measured with straight-line loops on eight warps, an SM runs at full rate up to about 28 KB of code
 // and fetches about one instruction per cycle beyond.  Splitting the route warp further (argmin and
 // commits apart, two commit warps) gave 1.07 us per request at one candidate per SM and 1.8 at two;
-// this split gives 0.87 and 0.95 (long-context trace, 16 replicas, 20,000 requests; the twelve-warp
-// kernel on blocks before it 1.1 and 1.35).
+// this split gives 0.73 and 0.78, and 1.35 at four (long-context trace, 16 replicas, 20,000 requests; the
+// twelve-warp kernel on blocks before it 1.1, 1.35 and 2.7).
 #include "gorgo_device.cuh"
 
 namespace gorgo {
@@ -56,25 +56,21 @@ constexpr uint32_t kFar = 0xFFFFu;    // the touches of a request are not in sha
 constexpr uint32_t kGroup = 8;        // most requests staged at once
 constexpr uint32_t kChunkRing = 64;   // requests whose static data is in shared memory, in chunks
 constexpr uint32_t kChunkMin = 4;     // fewest requests of a chunk
-constexpr uint32_t kRing = 128;       // requests between the route warp and the file warp
+constexpr uint32_t kRing = 128;       // requests by request number: routes, completions
+constexpr uint32_t kTimes = 64;       // the same where only those between the file warp and the route warp are needed (> kLead)
 constexpr uint32_t kLead = 60;        // the route warp runs at most this far ahead of the file warp
 constexpr uint32_t kRecent = 62;      // routes of that many requests before a commit are in the ring, older ones in the log
 constexpr uint32_t kNear = 64;        // completions within fewer than this many requests skip the lists in memory
+constexpr uint32_t kFiled = 16;      // requests the file warp waits for
 constexpr uint32_t kList = 64;        // requests whose lists the file warp hands over ahead
 constexpr uint32_t kInline = 3;       // list entries of a request handed over in shared memory
 constexpr uint32_t kMargin = 512;     // list victims once a cache is this close to full (blocks)
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round
-constexpr uint32_t kScanBytes = 16;   // route-log bytes per lane and scout round
-
-// A victim listed by the scout.  `next_req`: request of the atom's first occurrence after the
-// listing; `cum`: blocks listed for the replica up to and with this one (so that the victims of a
-// commit are found by one comparison per entry, without a scan over their lengths).
-struct __align__(16) Victim { uint32_t atom, next_req, cum, k; };   // k: index of the touch in its request
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
 // on the build.  want: the route warp waits for a victim of this replica (+ 1).
 struct Control {
-  volatile uint32_t routed, timed, filed, listed, exp_ready, committed, want, abort_flag;
+  volatile uint32_t routed, timed, filed, listed, exp_ready, committed, want, want_timed, abort_flag;
   volatile int32_t status;
 };
 
@@ -85,7 +81,13 @@ template <typename MaskT, bool kExt>
 struct Shared {
   static constexpr uint32_t kR = sizeof(MaskT) == 8 ? 64 : 32;
   static constexpr uint32_t kRows = sizeof(MaskT) == 8 ? 8 : 16;   // completion rows published ahead of the route warp
-  static constexpr uint32_t kVictims = 512;   // listed victims of all replicas together
+  // Listed victims of all replicas together, [R][ring_cap].  Of a victim the route warp needs its atom,
+  // the blocks listed for the replica up to and with it (so that the victims of a commit are found by
+  // one comparison per entry, without a scan over their lengths) and the request of the atom's first
+  // occurrence after the listing.  The rest (that occurrence's touch, the victim's request, its index there,
+  // -) is read rarely; with 64 replicas it lies in memory, so that three candidates fit an SM.
+  static constexpr uint32_t kVictims = sizeof(MaskT) == 8 ? 1024 : 512;
+  static constexpr uint32_t kMore = sizeof(MaskT) == 8 ? 1 : kVictims;
   Control c;
   uint64_t mbar[kChunkRing / kChunkMin];
   // stages: request + 1; (input tokens, -, blocks | origin << 16, where its touches are in shared
@@ -96,15 +98,14 @@ struct Shared {
   uint16_t ihits[kExt ? kStages : 1][kExt ? kR : 1];   // and in the proxy's index
   uint32_t epoch[kExt ? kStages : 1];                  // epoch under a time-varying network
   MaskT words[kStages][32];           // mask words of the first 32 atoms
-  double2 times[kRing];               // first-token and finish time
-  uint2 what[kRing];                  // (tokens, replica) of a routed request
+  double2 times[kTimes];              // first-token and finish time
+  uint2 what[kTimes];                 // (tokens, replica) of a routed request
   uint32_t near_head[kRing];          // request whose completion is seen first by request x, near ones (kNone: none)
-  uint32_t near_next[kRing];          // next of the same x
+  uint32_t near_next[kTimes];         // next of the same x
   double ts[2 * kNear];               // arrivals around the time warp's position
   uint2 listed_e[kList][kInline + 1]; // (rest of the list, entries), (tokens, replica) x 3
   double rows[kRows][kR];             // queue signal gone by the request's arrival
   double w[3 + 64];                   // weights
-  double load[kR];                    // in-flight signal at the end (route warp)
   uint32_t route_ring[kRing];         // replica | prefix hit << 8
   uint2 part[kR];                     // atom held in part (kNone: none), blocks of it
   uint32_t occ[kR];                   // cached blocks
@@ -117,8 +118,9 @@ struct Shared {
   uint32_t scan_list[kMatches];       // requests found in the log this round
   ReqRec c_req[kChunkRing];           // static data of the requests
   uint32_t c_at[kChunkRing];          // index of a request's touches in c_touch (kNone: they are not all there)
-  uint32_t victim_q[kVictims];        // request of a victim
-  Victim victims[kVictims];           // [R][ring_cap]
+  uint4 victim_more[kMore];
+  uint2 victims[kVictims];            // (atom, blocks listed)
+  uint32_t victim_next[kVictims];     // request of its next occurrence
   Touch c_touch[1];                   // [chunks][chunk_cap], then the regions of Dyn
 };
 // Regions whose size depends on the model: [G*R] RTT, [G*R] w_net * RTT, [R*S] time each slot frees.
@@ -233,12 +235,12 @@ __device__ __forceinline__ uint64_t score_key(double v, bool first) {
   if ((hi & 0x7FFFFFFFu) >= 0x7FF00000u && v != v) b = first ? 0xFFF0000000000000ULL : 0x7FF0000000000000ULL;
   return (b >> 63) ? ~b : (b | 0x8000000000000000ULL);
 }
-// Lanes that hold the smallest 64-bit key.
-__device__ __forceinline__ unsigned lanes_of_min(uint64_t key) {
+// The lowest `index` among the lanes that hold the smallest key.
+__device__ __forceinline__ uint32_t argmin(uint64_t key, uint32_t index) {
   const uint32_t hi = (uint32_t)(key >> 32), lo = (uint32_t)key;
   const uint32_t mh = __reduce_min_sync(kFull, hi);
   const uint32_t ml = __reduce_min_sync(kFull, hi == mh ? lo : 0xFFFFFFFFu);
-  return __ballot_sync(kFull, hi == mh && lo == ml);
+  return __reduce_min_sync(kFull, hi == mh && lo == ml ? index : 0xFFFFFFFFu);
 }
 
 // Set / clear `bit` of mask[a] without reading it back (reductions performed in L2).
@@ -578,23 +580,20 @@ __device__ __forceinline__ uint32_t dirty_from(const Touch* touch, uint32_t next
   }
   return d;
 }
-// A listed victim whose atom occurs again before r + kStages: is its touch (index k of request vq)
-// still the latest on replica `rep` as of the commit of request r there?  `dirty` gets what comes after r.
-__device__ __forceinline__ bool victim_live(const TraceView& tr, const uint8_t* route_log, uint32_t ring, uint32_t vq,
-                                            uint32_t k, uint32_t since, uint32_t r, uint32_t rep, uint32_t& dirty) {
-  const uint4* tp = reinterpret_cast<const uint4*>(tr.touch);
-  uint4 t = __ldg(tp + tr.req[vq].off + k);
+// A listed victim whose atom occurs again before r + kStages, first at touch `next` of request
+// `next_req`: is its touch still the latest on replica `rep` as of the commit of request r there?
+// `dirty` gets what comes after r.
+__device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* route_log, uint32_t ring, uint32_t next,
+                                            uint32_t next_req, uint32_t r, uint32_t rep, uint32_t& dirty) {
   #pragma unroll 1
-  while (t.z != kNone && t.w <= r) {
-    const uint32_t y = t.w;
-    if (y >= since) {                                // (occurrences before were looked at when it was listed)
-      const uint32_t rt = y == r ? rep : r - y < kRecent ? (lds32(ring + (y % kRing) * 4u) & 0xFFu)
-                                                         : (uint32_t)__ldcg(route_log + y);
-      if (rt == rep) return false;
-    }
-    t = __ldg(tp + t.z);
+  while (next != kNone && next_req <= r) {
+    const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[next].next));
+    const uint32_t rt = next_req == r ? rep : r - next_req < kRecent ? (lds32(ring + (next_req % kRing) * 4u) & 0xFFu)
+                                                                     : (uint32_t)__ldcg(route_log + next_req);
+    if (rt == rep) return false;
+    next = nx.x; next_req = nx.y;
   }
-  dirty = dirty_from(tr.touch, t.z, t.w, r);
+  dirty = dirty_from(touch, next, next_req, r);
   return true;
 }
 
@@ -604,7 +603,7 @@ __device__ __forceinline__ bool victim_live(const TraceView& tr, const uint8_t* 
 // itself.)
 template <typename MaskT, bool kExt>
 __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, kExt>& sh, MaskT* mask,
-                                            const uint8_t* route_log, uint32_t rep, uint32_t r, uint32_t need) {
+                                            const uint8_t* route_log, const uint4* more, uint32_t rep, uint32_t r, uint32_t need) {
   using Sh = Shared<MaskT, kExt>;
   const uint32_t lane = threadIdx.x & 31u, sb = smem_addr(&sh), cap_mask = a.ring_cap - 1u;
   const uint32_t p_take = sb + (uint32_t)offsetof(Sh, take) + rep * 8u;
@@ -627,13 +626,16 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
       if ((int32_t)avail <= 0) break;               // gave up
     }
     const uint32_t e = rep * a.ring_cap + ((head + lane) & cap_mask);
-    const uint4 v = lds128(sb + (uint32_t)offsetof(Sh, victims) + e * 16u);   // atom, next request, cum, k
+    const uint2 v = lds64(sb + (uint32_t)offsetof(Sh, victims) + e * 8u);
+    const uint32_t next_req = lds32(sb + (uint32_t)offsetof(Sh, victim_next) + e * 4u);
     const bool listed = lane < avail;
-    const uint32_t upto = v.z - cons;               // blocks gone with this entry
+    const uint32_t upto = v.y - cons;               // blocks gone with this entry
     bool live = listed;
     uint32_t d = 0;
-    if (listed && v.y < r + kStages)                // it occurred again since it was listed, or will soon
-      live = victim_live(a.tr, route_log, sb + (uint32_t)offsetof(Sh, route_ring), sh.victim_q[e], v.w, v.y, r, rep, d);
+    if (listed && next_req < r + kStages) {         // it occurred again since it was listed, or will soon
+      const uint32_t next = sizeof(MaskT) == 8 ? __ldcg(&more[e].x) : lds32(sb + (uint32_t)offsetof(Sh, victim_more) + e * 16u);
+      live = victim_live(a.tr.touch, route_log, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, rep, d);
+    }
     dirty |= __reduce_or_sync(kFull, d);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
     uint32_t dead = listed && !live ? upto - (lane ? prev : 0u) : 0u;   // blocks that are no victims
@@ -698,12 +700,14 @@ __device__ __noinline__ uint32_t commit_slow(const ReplayArgs& a, Shared<MaskT, 
 // the scout has listed (one victim per lane).  An atom that a commit changes is changed for its coming
 // occurrences too: those that may be staged already are noted (`dirty`) and staged again when their
 // turn comes.
-//   What bounds it is the latency of its own instructions, so the usual request takes one straight
-// path: whether the next request is ready is read and voted on while this one is decided, its rows are
-// loaded at the same time, and everything unusual is out of line.
+//   What bounds it is the latency of its own instructions.  The usual request takes one straight path in
+// which the commit of request q - 1 and the score of q run side by side, their shared-memory reads and
+// reductions interleaved, before it is known whether q is ready and its stage up to date; if not
+// (about 1.5 requests in 100), q is decided once more with nothing to commit.  Everything unusual is out of line
+// behind one vote.  (Commit after score: 0.85 us per request at one candidate per SM; side by side 0.73.)
 template <typename MaskT, bool kExt>
 __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, uint32_t sb, const Dyn& dy,
-                                           const StageArgs<MaskT>& sa, const uint8_t* route_log, const RepState* rep,
+                                           const StageArgs<MaskT>& sa, const uint8_t* route_log, const uint4* more, const RepState* rep,
                                            uint32_t p, uint32_t lane) {
   using Sh = Shared<MaskT, kExt>;
   constexpr bool kWide = sizeof(MaskT) == 8;
@@ -714,176 +718,180 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
   if (in0) { ld0 = (double)rep[lane].load; if (K != 3) nrm0 = sh.w[3 + lane]; }
   if (in1) { ld1 = (double)rep[lane + 32].load; if (K != 3) nrm1 = sh.w[35 + lane]; }
   const uint32_t i0 = min(lane, R - 1u), i1 = min(lane + 32u, R - 1u);
-  const double net0 = dy.wrtt[i0], net1 = dy.wrtt[i1];          // (one region: no look-up)
   const uint32_t cap_mask = a.ring_cap - 1u;
   const uint32_t C = a.m.C < 0xFFFFFFF0ull ? (uint32_t)a.m.C : 0xFFFFFFF0u;   // (its domain)
-  uint32_t dirty = 0;                               // bit k: an atom of request r + k has changed since it was staged
+  uint32_t dirty = 0;                               // bit k: an atom of request q + k has changed since it was staged
   unsigned long long st_probe = 0, st_hit = 0, st_blk = 0, st_evict = 0;
   // What a request has to wait for, one counter per lane: its stage (lane 0), its completions (lane 1),
   // the file warp (the others).
   const uint32_t p_wait = sb + (lane == 0 ? (uint32_t)offsetof(Sh, tag) : lane == 1 ? (uint32_t)offsetof(Control, exp_ready)
                                                                                    : (uint32_t)offsetof(Control, filed));
   const uint32_t ahead = lane < 2u ? 1u : 1u - kLead;
-  auto ready = [&](uint32_t r) {
-    return (int32_t)(lds32(p_wait + (lane == 0 ? (r % kStages) * 4u : 0u)) - (r + ahead)) >= 0;
-  };
-  struct Rows { uint4 f; uint32_t hit0, hit1; double gone0, gone1; };
-  auto load_rows = [&](uint32_t r, Rows& w) {
-    const uint32_t slot = r % kStages;
-    const uint32_t ph = sb + (uint32_t)offsetof(Sh, hits) + (slot * Sh::kR + lane) * 2u;
-    const uint32_t pr = sb + (uint32_t)offsetof(Sh, rows) + ((r % Sh::kRows) * Sh::kR + lane) * 8u;
-    w.f = lds128(sb + (uint32_t)offsetof(Sh, facts) + slot * 16u);
-    w.hit0 = lds16(ph);
-    w.gone0 = lds_f64(pr);
-    if (kWide) { w.hit1 = lds16(ph + 64u); w.gone1 = lds_f64(pr + 256u); }
-  };
-  Rows cur = {}, nxt = {};
-  bool slow = true;                                 // request r is not known to be ready, or its stage is dirty
-  bool good = true;
+  // The request that awaits its commit, q - 1 (if `pend`): its replica, this lane's atom of it (lanes
+  // without one have all bits set in the word), and whether the commit is an unusual one.
+  bool pend = false, odd = false;
+  uint32_t istar = 0, atom = kNone - 1u, len = 0, next_req = kNone;
+  MaskT word = ~(MaskT)0;
+  uint32_t q = a.first;
   PROF_BEGIN();
   #pragma unroll 1
-  for (uint32_t r = a.first; r < end; ++r) {
-    if (slow) {
-      wait_slow(sb + (uint32_t)offsetof(Sh, tag) + (r % kStages) * 4u, r + 1u, sb, a.poll_limit);
-      wait_slow(sb + offsetof(Control, exp_ready), r + 1u, sb, a.poll_limit);
-      wait_slow(sb + offsetof(Control, filed), r + 1u - kLead, sb, a.poll_limit);
-      if (!__all_sync(kFull, ready(r))) { good = false; break; }   // gave up
-      if (dirty & 1u) {
-        PROF_ADD(8, 1);
-        stage_now<MaskT, kExt>(a, sh, sa, r);
-      }
-      load_rows(r, cur);
-      PROF_ADD(7, 1);
-    }
-    PROF_LAP(0);
-    // ---- the next request: is it ready?  (Its rows are read after that.)
-    const bool next_ready = ready(r + 1u);
-    load_rows(r + 1u, nxt);
-    // ---- this lane's atom, for the commit
-    const uint32_t in_tok = cur.f.x, nblk = cur.f.z & 0xFFFFu, at = cur.f.w & 0xFFFFu, m = cur.f.w >> 16;
-    const bool odd = at == kFar || m > 32u || (kExt && opaque(a.proxy_index));
-    uint4 x = make_uint4(kNone, 0u, kNone, kNone);
-    MaskT word = 0;
-    if (lane < m && !odd) {
-      x = *reinterpret_cast<const uint4*>(&sh.c_touch[at + lane]);
-      word = *const_cast<const volatile MaskT*>(&sh.words[r % kStages][lane]);
-    }
-    // ---- score of Eq. 3 (fixed order, no FMA) and lowest-index argmin
-    const double* net = dy.wrtt + (cur.f.z >> 16) * R;
-    uint32_t s0 = cur.hit0, s1 = cur.hit1;
-    if (kExt && opaque(a.proxy_index)) {
-      s0 = sh.ihits[kExt ? r % kStages : 0][kExt ? lane : 0];
-      if (kWide) s1 = sh.ihits[kExt ? r % kStages : 0][kExt && kWide ? lane + 32u : 0u];
-    }
-    auto score = [&](uint32_t i, uint32_t h, double load, double nrm, double one) {   // (h < n blocks: h * B < input tokens)
-      const double qd = K != 3 ? __dmul_rn(load, nrm) : load;
-      const uint32_t unc = h >= nblk ? 0u : in_tok - h * a.m.B;
-      double nt = one;
-      if (a.m.G != 1u) nt = net[i];
-      if (kExt && opaque(a.rtt_ewma != nullptr))     // time-varying network: signal of the request's epoch
-        nt = __dmul_rn(sh.w[0], __ldg(a.rtt_ewma + ((size_t)sh.epoch[kExt ? r % kStages : 0] * a.m.G + (cur.f.z >> 16)) * R + i));
-      return __dadd_rn(__dadd_rn(nt, __dmul_rn(w_pre, (double)unc)), __dmul_rn(w_que, qd));
-    };
-    uint64_t key = score_key(score(i0, s0, ld0 - cur.gone0, nrm0, net0), lane == 0);
-    if (!in0) key = ~0ull;
-    bool upper = false;
-    if (kWide) {
-      uint64_t k1 = score_key(score(i1, s1, ld1 - cur.gone1, nrm1, net1), false);
-      if (!in1) k1 = ~0ull;
-      upper = k1 < key;
-      key = upper ? k1 : key;
-    }
-    PROF_LAP(1);
-    unsigned win = lanes_of_min(key);
-    if (kWide) {
-      const unsigned low = __ballot_sync(kFull, !upper) & win;   // winners in the lower half come first
-      win = low ? low : win;
-    }
-    uint32_t lead = (uint32_t)__ffs((int)win) - 1u;
-    if (kExt && opaque(a.forced_route != nullptr)) {
-      const uint32_t f = __ldg(a.forced_route + r);
-      lead = f & 31u;
-      upper = f >= 32u;
-    }
-    const bool mine = lane == lead;
-    double add = (double)in_tok;
-    if (kExt && opaque(a.queue_in_requests)) add = 1.0;          // baseline "least-request"
-    const bool up = kWide && upper;
-    if (mine) {
-      sts32(sb + (uint32_t)offsetof(Sh, route_ring) + (r % kRing) * 4u, (up ? lane + 32u : lane) | (up ? cur.hit1 : cur.hit0) << 8);
-      sts32(sb + offsetof(Control, routed), r + 1u);
-    }
-    ld0 += mine && !up ? add : 0.0;
-    if (kWide) ld1 += mine && up ? add : 0.0;
-    if (opaque(a.stats != nullptr)) {
-      if (in0) st_probe += min(cur.hit0 + 1u, nblk);
-      if (in1) st_probe += min(cur.hit1 + 1u, nblk);
-      if (mine) st_hit += up ? cur.hit1 : cur.hit0;
-      st_blk += nblk;
-    }
-    PROF_LAP(2);
-
-    // ---- cache commit: set the replica's bit on the atoms that do not have it
-    uint32_t istar = lead;
-    if (kWide) istar += (__ballot_sync(kFull, upper) >> lead & 1u) * 32u;
+  while (true) {
+    // ---- what the commit of q - 1 and the score of q need from shared memory
     const MaskT bit = (MaskT)1 << istar;
     const uint32_t p_part = sb + (uint32_t)offsetof(Sh, part) + istar * 8u;
     const uint32_t p_occ = sb + (uint32_t)offsetof(Sh, occ) + istar * 4u;
     const uint32_t p_take = sb + (uint32_t)offsetof(Sh, take) + istar * 8u;
-    const uint32_t part = lds32(p_part);
-    uint32_t occ = lds32(p_occ);
     const uint2 tk = lds64(p_take);                             // entries taken, blocks taken from the list
     const uint32_t tail = lds32(sb + (uint32_t)offsetof(Sh, ring_tail) + istar * 4u);
-    const bool changes = x.x != kNone && !(word & bit);
-    dirty >>= 1;
-    if (changes && !odd) mask_set(sa.mask, x.x, bit);
-    uint32_t missing = __reduce_add_sync(kFull, changes ? x.y & 0xFFFFu : 0u);
-    const uint4 v = lds128(sb + (uint32_t)offsetof(Sh, victims) + (istar * a.ring_cap + ((tk.x + lane) & cap_mask)) * 16u);
-    if (__any_sync(kFull, odd || (x.x == part && x.x != kNone) || (changes && x.w - r < kStages)))
-      missing = commit_slow<MaskT, kExt>(a, sh, sa, istar, r, dirty);
-    occ += missing;
-    PROF_LAP(3);
-
-    // ---- eviction: the victims are listed, none occurred again since, none occurs again soon
-    if (occ > C) {
-      const uint32_t need = occ - C;
-      occ = C;
-      st_evict += need;
-      const uint32_t upto = v.z - tk.y;                         // blocks gone with this entry
-      const unsigned enough = __ballot_sync(kFull, lane < tail - tk.x && upto >= need);
-      const unsigned near = __ballot_sync(kFull, v.y < r + kStages);
-      const unsigned taken = enough ^ (enough - 1u);            // lanes up to the first that is enough (all if none)
-      if (enough && !(near & taken)) {
-        const uint32_t keep = upto - need;                      // (last of them: blocks the last victim keeps)
-        const bool last = taken >> lane == 1u;
-        if (((taken >> lane) & 1u) && !(last && keep)) mask_clear(sa.mask, v.x, bit);
-        if (last) {
-          sts64(p_part, make_uint2(keep ? v.x : kNone, keep));
-          sts64(p_take, make_uint2(tk.x + lane + (keep ? 0u : 1u), tk.y + need));
-        }
-      } else {
-        PROF_ADD(9, 1);
-        dirty |= evict_slow<MaskT, kExt>(a, sh, sa.mask, route_log, istar, r, need);
-      }
+    const uint32_t slot = q % kStages;
+    const bool rdy = (int32_t)(lds32(p_wait + (lane == 0 ? slot * 4u : 0u)) - (q + ahead)) >= 0;
+    // (valid if q is ready: read after that)
+    const uint4 f = lds128(sb + (uint32_t)offsetof(Sh, facts) + slot * 16u);
+    const uint32_t p_hit = sb + (uint32_t)offsetof(Sh, hits) + (slot * Sh::kR + lane) * 2u;
+    const uint32_t p_row = sb + (uint32_t)offsetof(Sh, rows) + ((q % Sh::kRows) * Sh::kR + lane) * 8u;
+    const uint32_t hit0 = lds16(p_hit), hit1 = kWide ? lds16(p_hit + 64u) : 0u;
+    const double gone0 = lds_f64(p_row), gone1 = kWide ? lds_f64(p_row + 256u) : 0.0;
+    const uint32_t part = lds32(p_part), occ = lds32(p_occ);
+    // ---- commit: set the replica's bit on the atoms that do not have it
+    const bool changes = !(word & bit);
+    if (changes) mask_set(sa.mask, atom, bit);
+    uint32_t missing = __reduce_add_sync(kFull, changes ? len & 0xFFFFu : 0u);
+    const uint32_t entry = istar * a.ring_cap + ((tk.x + lane) & cap_mask);
+    const uint2 v = lds64(sb + (uint32_t)offsetof(Sh, victims) + entry * 8u);
+    const uint32_t v_next = lds32(sb + (uint32_t)offsetof(Sh, victim_next) + entry * 4u);
+    const bool special = odd || atom == part || (changes && next_req - (q - 1u) < kStages);
+    // ---- score of Eq. 3 (fixed order, no FMA) and lowest-index argmin
+    const uint32_t in_tok = f.x, nblk = f.z & 0xFFFFu, at = f.w & 0xFFFFu, m = f.w >> 16;
+    const double* net = dy.wrtt + (f.z >> 16) * R;
+    uint32_t s0 = hit0, s1 = hit1;
+    if (kExt && opaque(a.proxy_index)) {
+      s0 = sh.ihits[kExt ? slot : 0][kExt ? lane : 0];
+      if (kWide) s1 = sh.ihits[kExt ? slot : 0][kExt && kWide ? lane + 32u : 0u];
     }
-    if (lane == 0) sts32(p_occ, occ);
-    PROF_LAP(4);
+    auto score = [&](uint32_t i, uint32_t h, double load, double nrm) {   // (h < n blocks: h * B < input tokens)
+      const double qd = K != 3 ? __dmul_rn(load, nrm) : load;
+      const uint32_t unc = h >= nblk ? 0u : in_tok - h * a.m.B;
+      double nt = net[i];
+      if (kExt && opaque(a.rtt_ewma != nullptr))     // time-varying network: signal of the request's epoch
+        nt = __dmul_rn(sh.w[0], __ldg(a.rtt_ewma + ((size_t)sh.epoch[kExt ? slot : 0] * a.m.G + (f.z >> 16)) * R + i));
+      return __dadd_rn(__dadd_rn(nt, __dmul_rn(w_pre, (double)unc)), __dmul_rn(w_que, qd));
+    };
+    uint64_t key = score_key(score(i0, s0, ld0 - gone0, nrm0), lane == 0);
+    if (!in0) key = ~0ull;
+    uint32_t index = lane;
+    if (kWide) {
+      uint64_t k1 = score_key(score(i1, s1, ld1 - gone1, nrm1), false);
+      if (!in1) k1 = ~0ull;
+      if (k1 < key) { key = k1; index = lane + 32u; }
+    }
+    PROF_LAP(0);
+    uint32_t sel = argmin(key, index);
+    // ---- this lane's atom of q
+    const bool far = at == kFar || m > 32u || (kExt && opaque(a.proxy_index));
+    const bool has = lane < m && !far;
+    const uint4 x = *reinterpret_cast<const uint4*>(&sh.c_touch[has ? at + lane : 0u]);
+    const MaskT x_word = *const_cast<const volatile MaskT*>(&sh.words[slot][lane]);
+    // ---- eviction for q - 1: the victims are listed, none occurred again since, none occurs again soon
+    dirty >>= pend ? 1u : 0u;
+    uint32_t held = occ + missing, need = held > C ? held - C : 0u;
+    const uint32_t upto = v.y - tk.y;                           // blocks gone with this entry
+    const unsigned enough = __ballot_sync(kFull, lane < tail - tk.x && upto >= need);
+    const unsigned taken = enough ^ (enough - 1u);              // lanes up to the first that is enough (all if none)
+    const bool soon = (taken >> lane & 1u) && v_next < q - 1u + kStages;
+    bool valid = !(dirty & 1u);
+    PROF_LAP(1);
+    if (__any_sync(kFull, special || !rdy || (need != 0u && (soon || enough == 0u)))) {
+      const bool again = __any_sync(kFull, special);
+      if (again) {
+        uint32_t d = dirty;
+        missing = commit_slow<MaskT, kExt>(a, sh, sa, istar, q - 1u, d);
+        dirty = d;
+        held = occ + missing;
+        need = held > C ? held - C : 0u;
+      }
+      if (need != 0u && (again || enough == 0u || __any_sync(kFull, soon))) {
+        PROF_ADD(9, 1);
+        dirty |= evict_slow<MaskT, kExt>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
+        if (kExt) st_evict += need;
+        need = 0u;
+        held = C;
+      }
+      valid = __all_sync(kFull, rdy) && !(dirty & 1u);
+    }
+    PROF_LAP(2);
+    if (need != 0u) {
+      const uint32_t keep = upto - need;                        // (last of them: blocks the last victim keeps)
+      const bool last = taken >> lane == 1u;
+      if ((taken >> lane & 1u) && !(last && keep)) mask_clear(sa.mask, v.x, bit);
+      if (last) {
+        sts64(p_part, make_uint2(keep ? v.x : kNone, keep));
+        sts64(p_take, make_uint2(tk.x + lane + (keep ? 0u : 1u), tk.y + need));
+      }
+      if (kExt) st_evict += need;
+      held = C;
+    }
+    if (lane == 0) sts32(p_occ, held);
+    PROF_LAP(3);
     // words are visible with `committed`; the fence waits for the reductions in flight, so it is made
     // only every kPublish requests
-    if ((r + 1u) % kPublish == 0u || r + 1u == end) {
+    if (pend && (q % kPublish == 0u || q == end)) {
       __syncwarp();
       __threadfence_block();
-      if (lane == 0) sts32(sb + offsetof(Control, committed), r + 1u);
-      if (aborted(sb)) { good = false; break; }
+      if (lane == 0) sts32(sb + offsetof(Control, committed), q);
+      if (q == end || aborted(sb)) break;
     }
-    slow = !__all_sync(kFull, next_ready) || (dirty & 1u);
-    if (r + 1u < end) cur = nxt;
+    if (!valid) {
+      // ---- q was not ready, or its stage has changed: decide again, with nothing to commit
+      wait_slow(sb + (uint32_t)offsetof(Sh, tag) + slot * 4u, q + 1u, sb, a.poll_limit);
+      wait_slow(sb + offsetof(Control, exp_ready), q + 1u, sb, a.poll_limit);
+      wait_slow(sb + offsetof(Control, filed), q + 1u - kLead, sb, a.poll_limit);
+      if (aborted(sb)) break;                                   // gave up
+      if (dirty & 1u) {
+        PROF_ADD(8, 1);
+        __syncwarp();
+        __threadfence_block();                                  // (the words of the last commits)
+        stage_now<MaskT, kExt>(a, sh, sa, q);
+        dirty &= ~1u;
+      }
+      PROF_ADD(7, 1);
+      pend = odd = false;
+      word = ~(MaskT)0;
+      atom = kNone - 1u;
+      PROF_LAP(4);
+      continue;
+    }
+    // ---- hand the route over; q awaits its commit
+    if (kExt && opaque(a.forced_route != nullptr)) sel = __ldg(a.forced_route + q);
+    const bool mine = lane == (sel & 31u), up = kWide && sel >= 32u;
+    double add = (double)in_tok;
+    if (kExt && opaque(a.queue_in_requests)) add = 1.0;         // baseline "least-request"
+    if (mine) {
+      sts32(sb + (uint32_t)offsetof(Sh, route_ring) + (q % kRing) * 4u, sel | (up ? hit1 : hit0) << 8);
+      sts32(sb + offsetof(Control, routed), q + 1u);
+    }
+    ld0 += mine && !up ? add : 0.0;
+    if (kWide) ld1 += mine && up ? add : 0.0;
+    if (kExt && opaque(a.stats != nullptr)) {
+      if (in0) st_probe += min(hit0 + 1u, nblk);
+      if (in1) st_probe += min(hit1 + 1u, nblk);
+      if (mine) st_hit += up ? hit1 : hit0;
+      st_blk += nblk;
+    }
+    istar = sel;
+    odd = far;
+    atom = has ? x.x : kNone - 1u;
+    len = x.y;
+    next_req = x.w;
+    word = has ? x_word : ~(MaskT)0;
+    pend = true;
+    ++q;
     PROF_LAP(5);
   }
   PROF_END(0);
-  if (in0) sh.load[lane] = ld0 - cur.gone0;
-  if (in1) sh.load[kWide ? lane + 32u : 0u] = ld1 - cur.gone1;
-  if (a.stats) {
+  const uint32_t last_row = (end - 1u) % Sh::kRows;
+  if (in0) sh.rows[last_row][lane] = ld0 - sh.rows[last_row][lane];   // (the signal left)
+  if (in1) sh.rows[last_row][kWide ? lane + 32u : 0u] = ld1 - sh.rows[last_row][kWide ? lane + 32u : 0u];
+  if (kExt && a.stats) {
     unsigned long long* s4 = reinterpret_cast<unsigned long long*>(a.stats) + (size_t)p * 4;
     atomicAdd(s4, st_probe);
     if (st_hit) atomicAdd(s4 + 1, st_hit);
@@ -914,8 +922,16 @@ __device__ __forceinline__ void time_warp(const ReplayArgs& a, Shared<MaskT, kEx
   PROF_BEGIN();
   #pragma unroll 1
   while (s0 < end) {
-    const uint32_t seen = wait_counter(sb + offsetof(Control, routed), s0 + 1u, sb, a.poll_limit);
+    // a full round, unless the expiry warp waits for less
+    uint32_t seen = wait_counter(sb + offsetof(Control, routed), s0 + 1u, sb, a.poll_limit);
     if ((int32_t)(seen - (s0 + 1u)) < 0) break;            // gave up
+    const uint32_t full = min(s0 + kTimed, end);
+    #pragma unroll 1
+    for (uint32_t polls = 0; (int32_t)(seen - full) < 0 && polls < 64u; ++polls) {
+      if ((int32_t)(__shfl_sync(kFull, lds32(sb + offsetof(Control, want_timed)), 0) - s0) > 0) break;
+      __nanosleep(50);
+      seen = __shfl_sync(kFull, lds32(sb + offsetof(Control, routed)), 0);
+    }
     PROF_LAP(0);
     if (s0 - base >= 32u) {                                // the next 32 arrivals
       base += 32u;
@@ -1005,10 +1021,10 @@ __device__ __forceinline__ void time_warp(const ReplayArgs& a, Shared<MaskT, kEx
     if (on && sub == 0) {
       if (kExt && opaque(a.kv_budget > 0)) slot_kv[(size_t)i * S + bs] = need_kv;
       fa[bs] = finish;
-      sts_f64(sb + (uint32_t)offsetof(Sh, times) + (s % kRing) * 16u, first);
-      sts_f64(sb + (uint32_t)offsetof(Sh, times) + (s % kRing) * 16u + 8u, finish);
-      sts64(sb + (uint32_t)offsetof(Sh, what) + (s % kRing) * 8u, make_uint2(in_tok, i));
-      if (e8 && x < end) sts32(sb + (uint32_t)offsetof(Sh, near_next) + (s % kRing) * 4u, atomicExch(&sh.near_head[x % kRing], s));
+      sts_f64(sb + (uint32_t)offsetof(Sh, times) + (s % kTimes) * 16u, first);
+      sts_f64(sb + (uint32_t)offsetof(Sh, times) + (s % kTimes) * 16u + 8u, finish);
+      sts64(sb + (uint32_t)offsetof(Sh, what) + (s % kTimes) * 8u, make_uint2(in_tok, i));
+      if (e8 && x < end) sts32(sb + (uint32_t)offsetof(Sh, near_next) + (s % kTimes) * 4u, atomicExch(&sh.near_head[x % kRing], s));
     }
     __syncwarp();
     s0 += n;
@@ -1078,7 +1094,10 @@ __device__ __forceinline__ void expiry_warp(const ReplayArgs& a, Shared<MaskT, k
     if (r - a.first >= Sh::kRows && (int32_t)(routed - (r + 1u - Sh::kRows)) < 0)
       routed = wait_counter(sb + offsetof(Control, routed), r + 1u - Sh::kRows, sb, a.poll_limit);
     if ((int32_t)(listed - (r + 1u)) < 0) listed = wait_counter(sb + offsetof(Control, listed), r + 1u, sb, a.poll_limit);
-    if ((int32_t)(timed - want) < 0) timed = wait_counter(sb + offsetof(Control, timed), want, sb, a.poll_limit);
+    if ((int32_t)(timed - want) < 0) {
+      if (lane == 0) sts32(sb + offsetof(Control, want_timed), want);
+      timed = wait_counter(sb + offsetof(Control, timed), want, sb, a.poll_limit);
+    }
     PROF_LAP(0);
     // near completions
     const uint32_t p_head = sb + (uint32_t)offsetof(Sh, near_head) + (r % kRing) * 4u;
@@ -1086,8 +1105,8 @@ __device__ __forceinline__ void expiry_warp(const ReplayArgs& a, Shared<MaskT, k
     if (nj != kNone) {
       #pragma unroll 1
       for (uint32_t guard = 0; nj != kNone && guard < kNear; ++guard) {
-        take(lds64(sb + (uint32_t)offsetof(Sh, what) + (nj % kRing) * 8u));
-        nj = __shfl_sync(kFull, lds32(sb + (uint32_t)offsetof(Sh, near_next) + (nj % kRing) * 4u), 0);
+        take(lds64(sb + (uint32_t)offsetof(Sh, what) + (nj % kTimes) * 8u));
+        nj = __shfl_sync(kFull, lds32(sb + (uint32_t)offsetof(Sh, near_next) + (nj % kTimes) * 4u), 0);
       }
       if (lane == 0) sts32(p_head, kNone);
     }
@@ -1169,13 +1188,15 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
       const uint32_t timed = __shfl_sync(kFull, sh.c.timed, 0);
       smem_order();
       const uint32_t n = min(timed - filed, 32u);
-      if (n > 0) {
+      // many at a time (a pass costs the same for one and for 32), unless the route warp waits for a
+      // victim among them
+      if (n >= kFiled || (n > 0 && (timed == end || __any_sync(kFull, sh.c.want != 0)))) {
         uint32_t old = kNone, x = kNone;
         const uint32_t j = filed + lane;
         if (lane < n) {
-          const double2 tm = sh.times[j % kRing];
+          const double2 tm = sh.times[j % kTimes];
           const uint32_t rq = sh.route_ring[j % kRing];
-          const uint2 what = sh.what[j % kRing];
+          const uint2 what = sh.what[j % kTimes];
           const uint32_t istar = rq & 0xFFu;
           const double t = __dmul_rn(scale, a.tr.ts[j]);
           const double t_far = __dmul_rn(scale, a.tr.ts[min(j + kNear - 1u, end - 1)]);
@@ -1243,7 +1264,8 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
 // 32 touches per round, one per lane, and appends those that are still the latest touch of their
 // atom.  The route warp checks again what occurs between the listing and the eviction.
 template <typename MaskT, bool kExt>
-__device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, uint32_t sb, const Cand<MaskT>& cd, uint32_t lane) {
+__device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const Cand<MaskT>& cd, uint4* more,
+                                           uint32_t lane) {
   const uint32_t R = a.m.R, end = a.first + a.count;
   const Touch* touch = a.tr.touch;
   uint32_t dry0 = kNone, dry1 = kNone;                 // requests known when the replica's order ran out
@@ -1261,7 +1283,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     smem_order();
     uint32_t best = kNone;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < (sizeof(MaskT) == 8 ? 2 : 1); ++half) {
       const uint32_t i = lane + 32u * half;
       if (i < R && (want == i + 1u || (!opaque(a.scout_off) && (uint64_t)*(volatile uint32_t*)&sh.occ[i] + kMargin >= a.m.C))) {
         const uint32_t fill = sh.ring_tail[i] - *(volatile uint32_t*)&sh.take[i].x;
@@ -1286,23 +1308,37 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     uint32_t stop = pos;                               // requests < stop are looked at this round
     const uint32_t budget = room - min(room, (uint32_t)(vk + 1));
     if (budget > 0 && pos < seen) {
+      // (a word of four routes per lane and load; the loads of a stretch are in flight together)
+      const uint32_t mis = (uint32_t)(uintptr_t)cd.route_log & 3u, lo = pos + mis, hi = seen + mis, word0 = lo & ~3u;
+      auto routes = [&](uint32_t u) -> uint32_t {
+        const uint32_t x = word0 + 128u * u + 4u * lane;
+        return x < hi ? __ldcg(reinterpret_cast<const uint32_t*>(cd.route_log - mis + x)) : 0u;
+      };
+      uint32_t rt = routes(0), rt1 = routes(1), rt2 = routes(2), rt3 = routes(3);
       #pragma unroll 1
-      for (uint32_t b = 0; b < kScanBytes && stop < seen && n_match < budget; b += 4) {
-        uint32_t rt[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint32_t r = stop + 32u * u + lane;
-          rt[u] = r < seen ? (uint32_t)__ldcg(cd.route_log + r) : 255u;
+      for (uint32_t u = 0; u < 4u && n_match < budget && stop < seen; ++u) {
+        const uint32_t x = word0 + 128u * u + 4u * lane;
+        uint32_t hit = x < hi ? __vcmpeq4(rt, i * 0x01010101u) : 0u;   // 0xFF in the bytes that are equal
+        if (x < lo) hit &= kFull << (8u * (lo - x));
+        if (x < hi && hi - x < 4u) hit &= kFull >> (8u * (4u - (hi - x)));
+        const uint32_t cnt = (uint32_t)__popc(hit) / 8u;
+        uint32_t at = cnt;
+        #pragma unroll 1
+        for (uint32_t d = 1; d < 32u; d <<= 1) {
+          const uint32_t up = __shfl_up_sync(kFull, at, d);
+          if (lane >= d) at += up;
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool hit = rt[u] == i;
-          const unsigned bal = __ballot_sync(kFull, hit);
-          const uint32_t at = n_match + __popc(bal & ((1u << lane) - 1u));
-          if (hit && at < kMatches) sh.scan_list[at] = stop + 32u * u + lane;
-          n_match += __popc(bal);
+        const uint32_t total = __shfl_sync(kFull, at, 31);
+        at += n_match - cnt;
+        #pragma unroll 1
+        while (hit && at < kMatches) {
+          const uint32_t b = ((uint32_t)__ffs((int)hit) - 1u) / 8u;
+          sh.scan_list[at++] = x + b - mis;
+          hit &= ~(0xFFu << (8u * b));
         }
-        stop = min(stop + 128u, seen);
+        n_match += total;
+        stop = min(word0 + 128u * (u + 1u) - mis, seen);
+        rt = rt1; rt1 = rt2; rt2 = rt3;
       }
       __syncwarp();
       if (n_match > kMatches) { n_match = kMatches; stop = sh.scan_list[kMatches - 1] + 1u; }
@@ -1333,21 +1369,19 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     }
     // requests of the stretch that were not reached are looked at again next time
     pos = mi < n_match ? __shfl_sync(kFull, rq, mi & 31u) : stop;
-    Victim v = {0u, kNone, 0u, 0u};
     uint32_t len = 0;
+    Touch t = {0u, 0u, kNone, kNone};
     bool live = my_q != kNone;
     if (live) {
-      Touch t = touch[my_off + my_k];
-      v.atom = t.atom; v.k = my_k;
+      t = touch[my_off + my_k];
       len = t.len_pos & 0xFFFFu;
       if (sh.scan_plen[i] && my_q == sh.cur_req[i] && (int32_t)my_k == sh.cur_k[i]) len = sh.scan_plen[i];   // (partly evicted before)
       #pragma unroll 1
       while (t.next != kNone && t.next_req < seen) {   // later occurrences known to the log
+        const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[t.next].next));
         if ((uint32_t)__ldcg(cd.route_log + t.next_req) == i) { live = false; break; }
-        const uint2 nx = *reinterpret_cast<const uint2*>(&touch[t.next].next);
         t.next = nx.x; t.next_req = nx.y;
       }
-      v.next_req = t.next == kNone ? kNone : t.next_req;
     }
     const unsigned lv = __ballot_sync(kFull, live);
     uint32_t cum = live ? len : 0u;
@@ -1359,12 +1393,13 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     cum += sh.scan_cum[i];
     if (live) {
       const uint32_t slot = i * a.ring_cap + ((tail + (uint32_t)__popc(lv & ((1u << lane) - 1u))) & (a.ring_cap - 1u));
-      v.cum = cum;
-      sh.victims[slot] = v;
-      sh.victim_q[slot] = my_q;
+      sh.victims[slot] = make_uint2(t.atom, cum);
+      sh.victim_next[slot] = t.next == kNone ? kNone : t.next_req;
+      more[slot] = make_uint4(t.next, my_q, my_k, 0u);
     }
     cum = __shfl_sync(kFull, cum, 31);
     // every lane's entries are stored before lane 0 publishes the new tail
+    if (sizeof(MaskT) == 8) __threadfence_block();
     __syncwarp();
     smem_order();
     if (lane == 0) {
@@ -1445,11 +1480,15 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) dy.free_at[x] = g_slot[x];
   for (uint32_t i = R + threadIdx.x; i < Shared<MaskT, kExt>::kR; i += blockDim.x) sh.part[i] = make_uint2(kNone, 0u);
   if (threadIdx.x < kRing) sh.near_head[threadIdx.x] = kNone;
-  if (threadIdx.x < kStages) sh.tag[threadIdx.x] = 0u;
+  if (threadIdx.x < kStages) {                               // (stages are read before it is known that they are ready)
+    sh.tag[threadIdx.x] = 0u;
+    sh.facts[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+    if (kExt) sh.epoch[kExt ? threadIdx.x : 0] = 0u;
+  }
   if (threadIdx.x == 0) {
     sh.c.routed = a.first; sh.c.timed = a.first; sh.c.filed = a.first; sh.c.listed = a.first; sh.c.exp_ready = a.first;
     sh.c.abort_flag = 0; sh.c.status = 0;
-    sh.c.committed = a.first; sh.c.want = 0;
+    sh.c.committed = a.first; sh.c.want = 0; sh.c.want_timed = a.first;
 #pragma unroll
     for (uint32_t k = 0; k < kChunkRing / kChunkMin; ++k) mbar_init(sh.mbar + k);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1482,26 +1521,28 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
 
   const uint32_t sb = smem_addr(smem_raw);
   const StageArgs<MaskT> sa = {cd.mask, cd.index, cd.scale};
-  if (warp == kRoleRoute) route_warp<MaskT, kExt>(a, sh, sb, dy, sa, cd.route_log, cd.rep, p, lane);
+  uint4* more = sizeof(MaskT) == 8 ? reinterpret_cast<uint4*>(st + a.lay.more_off) : sh.victim_more;
+  if (warp == kRoleRoute) route_warp<MaskT, kExt>(a, sh, sb, dy, sa, cd.route_log, more, cd.rep, p, lane);
   else if (warp == kRoleStage) stage_warp<MaskT, kExt>(a, sh, sb, sa, lane);
   else if (warp == kRoleTime) time_warp<MaskT, kExt>(a, sh, sb, dy, cd.slot_kv, cd.scale, lane);
   else if (warp == kRoleExpiry) expiry_warp<MaskT, kExt>(a, sh, sb, cd.exp_rec, cd.scale, lane);
   else if (warp == kRoleFile) file_warp<MaskT, kExt>(a, sh, cd, p, lane);
-  else scout_warp<MaskT, kExt>(a, sh, sb, cd, lane);
+  else scout_warp<MaskT, kExt>(a, sh, cd, more, lane);
   __syncthreads();
 
   // ---- write the small state back; the eviction cursor stands at the next listed touch, or behind
   //      the last one taken
   for (uint32_t i = threadIdx.x; i < R; i += blockDim.x) {
-    RepState s = {(long long)sh.load[i], sh.occ[i], sh.cur_req[i], sh.cur_k[i], sh.part[i].x, sh.part[i].y, 0u};
+    RepState s = {(long long)sh.rows[(a.first + a.count - 1u) % Shared<MaskT, kExt>::kRows][i], sh.occ[i], sh.cur_req[i], sh.cur_k[i], sh.part[i].x, sh.part[i].y, 0u};
     const uint32_t head = sh.take[i].x, tail = sh.ring_tail[i], b = i * a.ring_cap, cap_mask = a.ring_cap - 1u;
     if (tail != head) {
-      s.cur_req = sh.victim_q[b + (head & cap_mask)];
-      s.cur_k = (int32_t)sh.victims[b + (head & cap_mask)].k;
+      const uint4 x = more[b + (head & cap_mask)];
+      s.cur_req = x.y;
+      s.cur_k = (int32_t)x.z;
     } else if (head != 0) {
       const uint32_t e = b + ((head - 1u) & cap_mask);
-      s.cur_req = sh.victim_q[e];
-      s.cur_k = (int32_t)sh.victims[e].k - 1;
+      s.cur_req = more[e].y;
+      s.cur_k = (int32_t)more[e].z - 1;
     }
     cd.rep[i] = s;
   }
@@ -1523,7 +1564,7 @@ size_t replay_smem_bytes(ReplayArgs& a) {
   a.slots_in_smem = (size_t)a.m.R * a.m.S * 8 <= kSlotBytes ? 1u : 0u;
   // victims listed ahead per replica: enough for a few commits, no more, because an entry listed
   // long ago has more often been touched again
-  a.ring_cap = a.m.R <= 16 ? 32u : a.m.R <= 32 ? 16u : 8u;
+  a.ring_cap = a.m.R <= 16 ? 32u : 16u;
   return shared_bytes<MaskT, kExt>(a.m, a.tr.chunk_req, a.tr.chunk_cap, a.slots_in_smem != 0);
 }
 
@@ -1575,7 +1616,7 @@ uint32_t mask_bytes_for(uint32_t n_replicas) { return n_replicas <= 32 ? 4u : 8u
 cudaError_t launch_replay(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st) {
   // the plain cost-model replay carries none of the optional model parts
   const bool ext = a.queue_in_requests || a.forced_route || a.rep_prefill_ms || a.rep_tpot_ms ||
-                   a.decode_slowdown > 0.0 || a.kv_budget > 0 || a.rtt_ewma || a.proxy_index;
+                   a.decode_slowdown > 0.0 || a.kv_budget > 0 || a.rtt_ewma || a.proxy_index || a.stats;
   if (a.m.R <= 32) return ext ? launch_replay_t<uint32_t, true>(a, n_cand, st) : launch_replay_t<uint32_t, false>(a, n_cand, st);
   return ext ? launch_replay_t<unsigned long long, true>(a, n_cand, st)
              : launch_replay_t<unsigned long long, false>(a, n_cand, st);
