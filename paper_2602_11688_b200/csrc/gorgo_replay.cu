@@ -98,6 +98,7 @@ struct Shared {
   uint16_t ihits[kExt ? kStages : 1][kExt ? kR : 1];   // and in the proxy's index
   uint32_t epoch[kExt ? kStages : 1];                  // epoch under a time-varying network
   MaskT words[kStages][32];           // mask words of the first 32 atoms
+  MaskT iwords[kExt ? kStages : 1][kExt ? 32 : 1];     // and of the proxy's index
   double2 times[kTimes];              // first-token and finish time
   uint2 what[kTimes];                 // (tokens, replica) of a routed request
   uint32_t near_head[kRing];          // request whose completion is seen first by request x, near ones (kNone: none)
@@ -365,8 +366,7 @@ __device__ __forceinline__ void stage_facts(const ReplayArgs& a, Shared<MaskT, k
 }
 
 // Stages one request with the whole warp, from the words in memory as they are now: requests with more
-// than 32 atoms, or whose touches are not in shared memory, or that are staged again, and every request
-// when the score uses the proxy's index.
+// than 32 atoms, or whose touches are not in shared memory, or that are staged again.
 template <typename MaskT, bool kExt>
 __device__ __noinline__ void stage_now(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const StageArgs<MaskT> sa,
                                        uint32_t r) {
@@ -389,7 +389,10 @@ __device__ __noinline__ void stage_now(const ReplayArgs& a, Shared<MaskT, kExt>&
       atom = at != kNone ? sh.c_touch[at + k].atom : __ldg(&a.tr.touch[q.off + k].atom);
       word = __ldcg(sa.mask + atom);
       if (index) iword = __ldcg(sa.index + atom);
-      if (base == 0) sh.words[slot][lane] = word;
+      if (base == 0) {
+        sh.words[slot][lane] = word;
+        if (index) sh.iwords[kExt ? slot : 0][kExt ? lane : 0] = iword;
+      }
     }
     const MaskT w0 = __shfl_sync(kFull, word, 0);
     MaskT hold = w0 & alive, all = 0;
@@ -456,14 +459,15 @@ __device__ __forceinline__ void stage_warp(const ReplayArgs& a, Shared<MaskT, kE
   // the group whose words are on their way: its first request, its size (0: none);
   // per lane: request and atom of it, its first lane, word and atom
   uint32_t q = a.first, n = 0, g = 0, seg = 0, m_seg = 0, atom = kNone, pos = 0;
-  MaskT word = 0;
+  MaskT word = 0, iword = 0;
+  const bool use_index = kExt && opaque(a.proxy_index);
   uint32_t next_q = a.first;                        // first request that is not in a group yet
   PROF_BEGIN();
   #pragma unroll 1
   while (q < end) {
     // ---- the next group: as many requests as there are free stages, landed chunks and lanes
     uint32_t n2 = 0, view2 = 0, g2 = 0, seg2 = 0, m2 = 0, atom2 = kNone, pos2 = 0;
-    MaskT word2 = 0;
+    MaskT word2 = 0, iword2 = 0;
     bool slow = false;
     if (next_q < end) {
       view2 = __shfl_sync(kFull, lds32(sb + offsetof(Control, committed)), 0);
@@ -497,7 +501,7 @@ __device__ __forceinline__ void stage_warp(const ReplayArgs& a, Shared<MaskT, kE
         if (lane < kGroup && lane < room) {
           at = sh.c_at[(next_q + lane) % kChunkRing];
           m = sh.c_req[(next_q + lane) % kChunkRing].m;
-          if (at == kNone || opaque(a.probe_off) || (kExt && opaque(a.proxy_index))) m = 64u;
+          if (at == kNone || opaque(a.probe_off)) m = 64u;
         }
         const Pack pk = pack_lanes(m, min(room, kGroup), lane);
         n2 = pk.n;
@@ -510,6 +514,7 @@ __device__ __forceinline__ void stage_warp(const ReplayArgs& a, Shared<MaskT, kE
           const uint2 x = *reinterpret_cast<const uint2*>(&sh.c_touch[at + k]);
           atom2 = x.x; pos2 = x.y >> 16;
           word2 = __ldcg(sa.mask + atom2);
+          if (use_index) iword2 = __ldcg(sa.index + atom2);
         }
         if (lane >= pk.total) { g2 = kNone; m2 = 0; }
       }
@@ -522,26 +527,39 @@ __device__ __forceinline__ void stage_warp(const ReplayArgs& a, Shared<MaskT, kE
       #pragma unroll 1
       for (uint32_t t = lane; t < n * row_words; t += 32)
         reinterpret_cast<uint32_t*>(&sh.hits[(q + t / row_words) % kStages][0])[t % row_words] = 0u;
+      if (use_index) {
+        #pragma unroll 1
+        for (uint32_t t = lane; t < n * row_words; t += 32)
+          reinterpret_cast<uint32_t*>(&sh.ihits[kExt ? (q + t / row_words) % kStages : 0][0])[kExt ? t % row_words : 0] = 0u;
+      }
       __syncwarp();
       const uint32_t r = q + g, k = lane - seg;
-      if (k < m_seg) sh.words[r % kStages][k] = word;
-      const MaskT first = __shfl_sync(kFull, word, seg);
-      MaskT hold = g < n ? first : 0;
-      const uint32_t full = low_bits(m_seg);
-      #pragma unroll 1
-      while (__any_sync(kFull, hold != 0)) {        // once per replica that holds the first atom: usually 0 to 2
-        const uint32_t i = hold ? (uint32_t)first_bit<MaskT>(hold) : 0u;
-        const uint2 part = lds64(sb + (uint32_t)offsetof(Sh, part) + i * 8u);
-        const uint32_t b = __ballot_sync(kFull, (word >> i) & 1) >> seg;
-        const uint32_t pb = __ballot_sync(kFull, k < m_seg && atom == part.x) >> seg;
-        const uint32_t run = (b & full) == full ? m_seg : (uint32_t)__ffs((int)~b) - 1u;
-        const uint32_t pm = pb & low_bits(run);     // its partly held atom among the leading ones
-        const uint32_t kk = pm ? (uint32_t)__ffs((int)pm) - 1u : run;
-        const uint32_t ps = __shfl_sync(kFull, pos, min(seg + kk, 31u));
-        if (hold && k == 0)
-          sh.hits[r % kStages][i] = (uint16_t)(pm ? ps + part.y : run == m_seg ? sh.c_req[r % kChunkRing].nblk : ps);
-        hold &= hold - 1;
+      if (k < m_seg) {
+        sh.words[r % kStages][k] = word;
+        if (use_index) sh.iwords[kExt ? r % kStages : 0][kExt ? k : 0] = iword;
       }
+      const uint32_t full = low_bits(m_seg);
+      auto prefixes = [&](MaskT wd, bool parts, uint16_t* rows) {   // (rows: [kStages][kR] hits)
+        const MaskT first = __shfl_sync(kFull, wd, seg);
+        MaskT hold = g < n ? first : 0;
+        #pragma unroll 1
+        while (__any_sync(kFull, hold != 0)) {      // once per replica that holds the first atom: usually 0 to 2
+          const uint32_t i = hold ? (uint32_t)first_bit<MaskT>(hold) : 0u;
+          uint2 part = make_uint2(kNone, 0u);
+          if (parts) part = lds64(sb + (uint32_t)offsetof(Sh, part) + i * 8u);
+          const uint32_t b = __ballot_sync(kFull, (wd >> i) & 1) >> seg;
+          const uint32_t pb = __ballot_sync(kFull, k < m_seg && atom == part.x) >> seg;
+          const uint32_t run = (b & full) == full ? m_seg : (uint32_t)__ffs((int)~b) - 1u;
+          const uint32_t pm = pb & low_bits(run);   // its partly held atom among the leading ones
+          const uint32_t kk = pm ? (uint32_t)__ffs((int)pm) - 1u : run;
+          const uint32_t ps = __shfl_sync(kFull, pos, min(seg + kk, 31u));
+          if (hold && k == 0)
+            rows[(r % kStages) * Sh::kR + i] = (uint16_t)(pm ? ps + part.y : run == m_seg ? sh.c_req[r % kChunkRing].nblk : ps);
+          hold &= hold - 1;
+        }
+      };
+      prefixes(word, true, &sh.hits[0][0]);
+      if (use_index) prefixes(iword, false, &sh.ihits[0][0]);
       __syncwarp();
       if (g < n && k == 0) stage_facts<MaskT, kExt>(a, sh, sa, r);
       q += n;
@@ -555,7 +573,7 @@ __device__ __forceinline__ void stage_warp(const ReplayArgs& a, Shared<MaskT, kE
       n = 0;
     } else {
       next_q += n2;
-      n = n2; g = g2; seg = seg2; m_seg = m2; atom = atom2; pos = pos2; word = word2;
+      n = n2; g = g2; seg = seg2; m_seg = m2; atom = atom2; pos = pos2; word = word2; iword = iword2;
     }
     if (aborted(sb)) break;
   }
@@ -685,7 +703,11 @@ __device__ __noinline__ uint32_t commit_slow(const ReplayArgs& a, Shared<MaskT, 
     changes = changes || fills;
     if (changes) missing += (x.y & 0xFFFFu) - (fills ? part.y : 0u);
     filled = filled || fills;
-    if (kExt && opaque(a.proxy_index)) { mask_set(sa.index, x.x, bit); changes = true; }
+    if (kExt && opaque(a.proxy_index)) {
+      const MaskT iword = k < 32u ? *const_cast<const volatile MaskT*>(&sh.iwords[kExt ? r % kStages : 0][kExt ? k : 0])
+                                  : (MaskT)__ldcg(sa.index + x.x);
+      if (!(iword & bit)) { mask_set(sa.index, x.x, bit); changes = true; }
+    }
     if (changes && x.w - r < kStages) later |= dirty_from(a.tr.touch, x.z, x.w, r);
   }
   dirty |= __reduce_or_sync(kFull, later);
@@ -731,7 +753,8 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
   // without one have all bits set in the word), and whether the commit is an unusual one.
   bool pend = false, odd = false;
   uint32_t istar = 0, atom = kNone - 1u, len = 0, next_req = kNone;
-  MaskT word = ~(MaskT)0;
+  MaskT word = ~(MaskT)0, iword = ~(MaskT)0;         // (iword: of the proxy's index)
+  const bool use_index = kExt && opaque(a.proxy_index);
   uint32_t q = a.first;
   PROF_BEGIN();
   #pragma unroll 1
@@ -755,16 +778,18 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
     // ---- commit: set the replica's bit on the atoms that do not have it
     const bool changes = !(word & bit);
     if (changes) mask_set(sa.mask, atom, bit);
+    const bool indexed = use_index && !(iword & bit);
+    if (indexed) mask_set(sa.index, atom, bit);
     uint32_t missing = __reduce_add_sync(kFull, changes ? len & 0xFFFFu : 0u);
     const uint32_t entry = istar * a.ring_cap + ((tk.x + lane) & cap_mask);
     const uint2 v = lds64(sb + (uint32_t)offsetof(Sh, victims) + entry * 8u);
     const uint32_t v_next = lds32(sb + (uint32_t)offsetof(Sh, victim_next) + entry * 4u);
-    const bool special = odd || atom == part || (changes && next_req - (q - 1u) < kStages);
+    const bool special = odd || atom == part || ((changes || indexed) && next_req - (q - 1u) < kStages);
     // ---- score of Eq. 3 (fixed order, no FMA) and lowest-index argmin
     const uint32_t in_tok = f.x, nblk = f.z & 0xFFFFu, at = f.w & 0xFFFFu, m = f.w >> 16;
     const double* net = dy.wrtt + (f.z >> 16) * R;
     uint32_t s0 = hit0, s1 = hit1;
-    if (kExt && opaque(a.proxy_index)) {
+    if (use_index) {
       s0 = sh.ihits[kExt ? slot : 0][kExt ? lane : 0];
       if (kWide) s1 = sh.ihits[kExt ? slot : 0][kExt && kWide ? lane + 32u : 0u];
     }
@@ -787,10 +812,11 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
     PROF_LAP(0);
     uint32_t sel = argmin(key, index);
     // ---- this lane's atom of q
-    const bool far = at == kFar || m > 32u || (kExt && opaque(a.proxy_index));
+    const bool far = at == kFar || m > 32u;
     const bool has = lane < m && !far;
     const uint4 x = *reinterpret_cast<const uint4*>(&sh.c_touch[has ? at + lane : 0u]);
     const MaskT x_word = *const_cast<const volatile MaskT*>(&sh.words[slot][lane]);
+    const MaskT x_iword = use_index ? *const_cast<const volatile MaskT*>(&sh.iwords[kExt ? slot : 0][kExt ? lane : 0]) : ~(MaskT)0;
     // ---- eviction for q - 1: the victims are listed, none occurred again since, none occurs again soon
     dirty >>= pend ? 1u : 0u;
     uint32_t held = occ + missing, need = held > C ? held - C : 0u;
@@ -855,7 +881,7 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
       }
       PROF_ADD(7, 1);
       pend = odd = false;
-      word = ~(MaskT)0;
+      word = iword = ~(MaskT)0;
       atom = kNone - 1u;
       PROF_LAP(4);
       continue;
@@ -883,6 +909,7 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
     len = x.y;
     next_req = x.w;
     word = has ? x_word : ~(MaskT)0;
+    if (use_index) iword = has ? x_iword : ~(MaskT)0;
     pend = true;
     ++q;
     PROF_LAP(5);
