@@ -130,7 +130,13 @@ def load():
 
 
 def _np_ptr(a: Optional[np.ndarray]):
-    return None if a is None else a.ctypes.data_as(C.c_void_p)
+    """Address of an array's data (the caller keeps the array)."""
+    if a is None:
+        return None
+    try:
+        return C.addressof(C.c_char.from_buffer(a))          # a sixth of the time of ``a.ctypes``
+    except (TypeError, ValueError):                          # read-only or empty
+        return a.ctypes.data
 
 
 def _dev_ptr(t) -> Optional[int]:

@@ -754,7 +754,7 @@ static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, co
   std::vector<Touch> touch(Tn);
   std::vector<uint32_t> prev(Tn, kNone);         // previous occurrence where it lies in an earlier batch
   const size_t D0 = tb.map.raw.size();
-  bool patch_old = false;
+  uint64_t n_links = 0;
   for (uint64_t k = 0; k < n_new; ++k) {
     const uint32_t r = (uint32_t)(N0 + k);
     req[k].off = (uint32_t)(T0 + hash_off[k]);
@@ -771,7 +771,7 @@ static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, co
       const uint32_t pg = tb.last_g[d];
       if (tb.last_r[d] + 1 > latest) latest = tb.last_r[d] + 1;
       if (pg >= T0) { touch[pg - T0].next = g; touch[pg - T0].next_req = r; }
-      else { prev[gl] = pg; patch_old = true; }
+      else { prev[gl] = pg; ++n_links; }
       tb.last_g[d] = g; tb.last_r[d] = r;
     }
     req[k].prev_share = latest ? latest - 1 : kNone;
@@ -789,17 +789,40 @@ static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, co
   DeviceGuard guard(sim->device);
   if (!guard.ok) return GORGO_ERR_CUDA;
   const TraceRegions& rg = sim->reg;
-  bool ok = copy_in(rg.req + N0 * sizeof(ReqRec), req.data(), n_new * sizeof(ReqRec), st) &&
-            copy_in(rg.touch + T0 * sizeof(Touch), touch.data(), Tn * sizeof(Touch), st) &&
-            copy_in(rg.raw + D0 * 8, tb.map.raw.data() + D0, Dn * 8, st) &&
-            copy_in(rg.ts + N0 * 8, ts_ms, n_new * 8, st) &&
-            copy_in(rg.grid + (size_t)grid_from * 4, grid.data(), grid.size() * 4, st);
-  if (N0 == 0) ok = ok && copy_in(rg.rtt, sim->rtt.data(), sim->rtt.size() * 8, st);
-  // earlier batches' last occurrences now have a successor
-  if (patch_old)
-    ok = ok && copy_in(rg.extra, prev.data(), Tn * 4, st) &&
-         launch_link_occurrences(tr, (uint32_t)N0, (uint32_t)n_new, reinterpret_cast<const uint32_t*>(rg.extra),
-                                 reinterpret_cast<Touch*>(rg.touch), st) == cudaSuccess;
+  const struct { unsigned char* dst; const void* src; size_t bytes; } part[5] = {
+      {rg.req + N0 * sizeof(ReqRec), req.data(), n_new * sizeof(ReqRec)},
+      {rg.touch + T0 * sizeof(Touch), touch.data(), Tn * sizeof(Touch)},
+      {rg.raw + D0 * 8, tb.map.raw.data() + D0, Dn * 8},
+      {rg.ts + N0 * 8, ts_ms, n_new * 8},
+      {rg.grid + (size_t)grid_from * 4, grid.data(), grid.size() * 4}};
+  size_t words = 0;
+  for (const auto& x : part) words += x.bytes / 4;
+  bool ok = true;
+  if (N0 == 0) ok = copy_in(rg.rtt, sim->rtt.data(), sim->rtt.size() * 8, st);
+  if (words + 3 * n_links <= AppendPayload::kWords) {
+    // the usual case of a proxy that appends requests as they arrive
+    AppendPayload a;
+    uint32_t* w = a.words;
+    for (int k = 0; k < 5; ++k) {
+      a.dst[k] = reinterpret_cast<uint32_t*>(part[k].dst);
+      a.n_words[k] = (uint32_t)(part[k].bytes / 4);
+      if (part[k].bytes) std::memcpy(w, part[k].src, part[k].bytes);
+      w += a.n_words[k];
+    }
+    a.n_links = (uint32_t)n_links;
+    a.touch = reinterpret_cast<Touch*>(rg.touch);
+    for (uint64_t k = 0; k < n_new && n_links; ++k)
+      for (uint64_t gl = hash_off[k]; gl < hash_off[k + 1]; ++gl)
+        if (prev[gl] != kNone) { *w++ = prev[gl]; *w++ = (uint32_t)(T0 + gl); *w++ = (uint32_t)(N0 + k); }
+    ok = ok && launch_append(a, st) == cudaSuccess;
+  } else {
+    for (const auto& x : part) ok = ok && copy_in(x.dst, x.src, x.bytes, st);
+    // earlier batches' last occurrences now have a successor
+    if (n_links)
+      ok = ok && copy_in(rg.extra, prev.data(), Tn * 4, st) &&
+           launch_link_occurrences(tr, (uint32_t)N0, (uint32_t)n_new, reinterpret_cast<const uint32_t*>(rg.extra),
+                                   reinterpret_cast<Touch*>(rg.touch), st) == cudaSuccess;
+  }
   if (!ok) { cudaGetLastError(); sim->has_trace = false; return GORGO_ERR_CUDA; }
   sim->has_trace = true;
   return GORGO_OK;

@@ -48,9 +48,9 @@ static_assert(sizeof(RepState) == 32, "RepState layout");
 struct __align__(32) CandHeader {
   uint32_t processed;  // requests replayed so far
   int32_t status;      // 0, or a gorgo_status recorded by a kernel
-  uint32_t overflow;   // persistent state: 1 + the newest request that completes after the end of
-                       // the trace known so far (0: none); such requests are chained through
-                       // their completion records until an appended request takes them
+  uint32_t overflow;   // persistent state: requests that complete after the end of the trace known so
+                       // far; they are listed in the fourth words of the completion records until
+                       // an appended request takes them
   uint32_t pad[5];
 };
 
@@ -112,7 +112,7 @@ struct ReplayArgs {
   // per-request arrays, candidate p at + p*N elements
   uint32_t* exp_head;             // [r]: first entry of the list of requests whose completion the
                                   //   proxy sees when request r arrives (kNone: none)
-  uint4* exp_rec;                 // [j]: (next entry of j's list, input tokens of j, replica of j, -)
+  uint4* exp_rec;                 // [j]: (next entry of j's list, input tokens of j, replica of j, list of late completions)
   uint8_t* route_log;             // chosen replica of every request replayed so far
   uint64_t route_log_stride;      // elements between candidates
   // baseline policies: queue signal counted in requests instead of tokens; one fixed route per
@@ -194,6 +194,17 @@ cudaError_t prof_read(unsigned long long* out112, bool reset);
 // After requests [first_new, first_new + n_new) were appended to a growing trace: every block of
 // theirs that occurred before gets its previous occurrence (`prev[i]` of the i-th new touch)
 // linked to it.
+// What a small append writes, carried by the launch itself: runs of words for up to five places, then the
+// triples (touch of an earlier batch, its new successor, the successor's request).
+struct AppendPayload {
+  uint32_t* dst[5];
+  uint32_t n_words[5];
+  uint32_t n_links;
+  Touch* touch;
+  static constexpr uint32_t kWords = 1000 - 18;   // (all of it within the 4,000 bytes of a small launch)
+  uint32_t words[kWords];
+};
+cudaError_t launch_append(const AppendPayload& a, cudaStream_t st);
 cudaError_t launch_link_occurrences(const TraceView& tr, uint32_t first_new, uint32_t n_new,
                                     const uint32_t* prev, Touch* touch, cudaStream_t st);
 cudaError_t launch_gather(const void* buf, uint64_t n_sectors, uint32_t per_thread, uint32_t blocks,

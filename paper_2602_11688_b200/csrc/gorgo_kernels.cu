@@ -21,6 +21,22 @@ __global__ void link_occurrences_kernel(TraceView tr, uint32_t first_new, uint32
   }
 }
 
+// A small append in one launch whose parameters are the data: bound by launch latency.  (It replaces
+// six copies and a launch; appending one request takes the host 13 us instead of 26.)
+__global__ void append_kernel(const __grid_constant__ AppendPayload a) {
+  uint32_t at = 0;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    for (uint32_t i = threadIdx.x; i < a.n_words[k]; i += blockDim.x) a.dst[k][i] = a.words[at + i];
+    at += a.n_words[k];
+  }
+  for (uint32_t i = threadIdx.x; i < a.n_links; i += blockDim.x) {
+    const uint32_t* x = a.words + at + 3u * i;
+    a.touch[x[0]].next = x[1];
+    a.touch[x[0]].next_req = x[2];
+  }
+}
+
 __global__ void reset_states_kernel(unsigned char* states, StateLayout lay, uint32_t R, uint32_t S,
                                     uint32_t n_cand) {
   const uint32_t p = blockIdx.x;
@@ -292,6 +308,11 @@ cudaError_t launch_reset(unsigned char* masks, uint64_t mask_stride, uint64_t ma
   e = cudaMemsetAsync(exp_head, 0xFF, exp_head_count * sizeof(uint32_t), st);   // kNone: empty lists
   if (e != cudaSuccess) return e;
   reset_states_kernel<<<n_cand, 128, 0, st>>>(states, lay, m.R, m.S, n_cand);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_append(const AppendPayload& a, cudaStream_t st) {
+  append_kernel<<<1, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

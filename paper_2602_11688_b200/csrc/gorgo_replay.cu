@@ -66,6 +66,7 @@ constexpr uint32_t kList = 64;        // requests whose lists the file warp hand
 constexpr uint32_t kInline = 3;       // list entries of a request handed over in shared memory
 constexpr uint32_t kMargin = 512;     // list victims once a cache is this close to full (blocks)
 constexpr uint32_t kHops = 4;         // occurrences looked at before the replica's next requests are asked
+constexpr uint32_t kFew = 8;          // requests of a launch up to which victims are not listed ahead
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
@@ -1235,6 +1236,10 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
           if (opaque(a.ttft_out != nullptr)) a.ttft_out[o] = __dsub_rn(tm.x, t);
           if (opaque(a.e2e_out != nullptr)) a.e2e_out[o] = __dsub_rn(tm.y, t);
           const double f = tm.y;
+          auto record = [&](uint32_t next) {           // (the fourth word is the state's list of late completions)
+            *reinterpret_cast<uint2*>(cd.exp_rec + j) = make_uint2(next, what.x);
+            cd.exp_rec[j].z = istar;
+          };
           if (f > t_far) {
             const uint32_t lo = max(j + 1u, min(j + kNear, end));      // (later than every near request)
             if (lo < N && t_last >= f) {
@@ -1259,12 +1264,12 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
               }
               x = found ? min(g, N - 1) : first_arrival_at_or_after(a.tr.ts, scale, f, min(g, N - 1), N - 1);
               old = atomicExch(cd.exp_head + x, j);
-              cd.exp_rec[j] = make_uint4(old, what.x, istar, 0u);
+              record(old);
             } else if (opaque(cd.finish_log != nullptr)) {
-              // completes after the last known arrival: chained in the state (read by the next launch)
+              // completes after the last known arrival: listed in the state (read by the next launch)
               cd.finish_log[j] = f;
-              const uint32_t before = atomicExch(&cd.hdr->overflow, j + 1u);
-              cd.exp_rec[j] = make_uint4(before - 1u, what.x, istar, 0u);
+              reinterpret_cast<uint32_t*>(cd.exp_rec)[4 * (size_t)atomicAdd(&cd.hdr->overflow, 1u) + 3] = j;
+              record(kNone);
             }
           }
         }
@@ -1296,6 +1301,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
                                            uint32_t lane) {
   const uint32_t R = a.m.R, end = a.first + a.count;
   const Touch* touch = a.tr.touch;
+  // a launch of a few requests is over before lists made ahead are of use: only what is waited for
+  const bool ahead = !a.scout_off && a.count > kFew;
   uint32_t dry0 = kNone, dry1 = kNone;                 // requests known when the replica's order ran out
   uint32_t idle = 0;
   PROF_BEGIN();
@@ -1313,7 +1320,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
 #pragma unroll
     for (int half = 0; half < (sizeof(MaskT) == 8 ? 2 : 1); ++half) {
       const uint32_t i = lane + 32u * half;
-      if (i < R && (want == i + 1u || (!opaque(a.scout_off) && (uint64_t)*(volatile uint32_t*)&sh.occ[i] + kMargin >= a.m.C))) {
+      if (i < R && (want == i + 1u || (ahead && (uint64_t)*(volatile uint32_t*)&sh.occ[i] + kMargin >= a.m.C))) {
         const uint32_t fill = sh.ring_tail[i] - *(volatile uint32_t*)&sh.take[i].x;
         if (fill * 2u <= a.ring_cap && (half ? dry1 : dry0) != seen) best = min(best, (fill << 8) | i);
       }
@@ -1546,29 +1553,35 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     for (uint32_t k = 0; k < kChunkRing / kChunkMin; ++k) mbar_init(sh.mbar + k);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (cd.finish_log && threadIdx.x == 32) {
-    // the trace may have grown since the last batch: requests that were to complete after its
-    // old end are filed under the first request, not yet replayed, that arrives at or after
-    // their finish time; the rest stay chained
+  if (cd.finish_log) {
+    // The trace may have grown since the last batch: requests that were to complete after its old
+    // end are filed under the first request, not yet replayed, that arrives at or after their finish
+    // time; the rest stay listed.  (Their list is an array, in the fourth words of the completion
+    // records: as a chain, one thread followed it in every launch, one memory latency per request in flight.)
+    uint32_t* list = reinterpret_cast<uint32_t*>(cd.exp_rec) + 3;
+    const uint32_t n = cd.hdr->overflow;
+    uint32_t& kept = sh.scan_list[0];
+    if (threadIdx.x == 0) kept = 0;
     const double t_last = __dmul_rn(cd.scale, a.tr.ts[N - 1]);
-    uint32_t e = cd.hdr->overflow - 1u, keep = kNone;
     #pragma unroll 1
-    for (uint32_t guard = 0; e != kNone && guard < N; ++guard) {
-      uint4 rec = cd.exp_rec[e];
-      const uint32_t nxt = rec.x;
-      const double f = cd.finish_log[e];
-      if (e + 1 < N && t_last >= f) {
-        const uint32_t x = first_arrival_at_or_after(a.tr.ts, cd.scale, f, max(e + 1u, a.first), N - 1);
-        rec.x = cd.exp_head[x];
-        cd.exp_head[x] = e;
-      } else {
-        rec.x = keep;
-        keep = e;
+    for (uint32_t base = 0; base < n; base += blockDim.x) {
+      const bool on = base + threadIdx.x < n;
+      bool keep = false;
+      uint32_t e = 0;
+      if (on) {
+        e = list[4 * (size_t)(base + threadIdx.x)];
+        const double f = cd.finish_log[e];
+        keep = !(e + 1 < N && t_last >= f);
+        if (!keep) {
+          const uint32_t x = first_arrival_at_or_after(a.tr.ts, cd.scale, f, max(e + 1u, a.first), N - 1);
+          cd.exp_rec[e].x = atomicExch(cd.exp_head + x, e);
+        }
       }
-      cd.exp_rec[e] = rec;
-      e = nxt;
+      __syncthreads();                                 // (entries move down only, to places that are read)
+      if (keep) list[4 * (size_t)atomicAdd(&kept, 1u)] = e;
     }
-    cd.hdr->overflow = keep + 1u;
+    __syncthreads();
+    if (threadIdx.x == 0 && n > 0) cd.hdr->overflow = kept;
   }
   __syncthreads();
 
