@@ -101,6 +101,10 @@ struct gorgo_sim {
   uint32_t ev_used = 0;
   std::vector<cudaEvent_t> wev;   // pairs around the window-objective launches
   uint32_t wev_used = 0;
+  // pinned host memory of the online tuner, kept between its calls (the largest so far; one call at a time)
+  std::mutex pin_mutex;
+  double* pin = nullptr;
+  size_t pin_doubles = 0;
 };
 
 namespace {
@@ -116,6 +120,26 @@ struct DeviceGuard {
     if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
   }
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+};
+
+// The simulator's pinned memory for one call; null while another thread's call has it, or if there is
+// none to be had.  Nothing of the stream uses it any more when it is given back.
+struct PinLease {
+  std::unique_lock<std::mutex> lock;
+  cudaStream_t st;
+  double* p = nullptr;
+  PinLease(gorgo_sim* sim, size_t doubles, cudaStream_t stream) : lock(sim->pin_mutex, std::try_to_lock), st(stream) {
+    if (!lock.owns_lock()) return;
+    if (sim->pin_doubles < doubles) {
+      if (sim->pin) cudaFreeHost(sim->pin);
+      sim->pin = nullptr; sim->pin_doubles = 0;
+      void* q = nullptr;
+      if (cudaHostAlloc(&q, doubles * 8, cudaHostAllocDefault) != cudaSuccess) { cudaGetLastError(); return; }
+      sim->pin = static_cast<double*>(q); sim->pin_doubles = doubles;
+    }
+    p = sim->pin;
+  }
+  ~PinLease() { if (p) cudaStreamSynchronize(st); }
 };
 
 StateLayout make_layout(const Model& m) {
@@ -427,6 +451,10 @@ int gorgo_sim_destroy(gorgo_sim_t* sim) {
     DeviceGuard guard(sim->device);
     for (cudaEvent_t e : sim->ev) cudaEventDestroy(e);
     for (cudaEvent_t e : sim->wev) cudaEventDestroy(e);
+  }
+  if (sim->pin) {
+    DeviceGuard guard(sim->device);
+    cudaFreeHost(sim->pin);
   }
   delete sim;
   return GORGO_OK;
@@ -1100,20 +1128,26 @@ int gorgo_tune_online(gorgo_sim_t* sim, const gorgo_online_config_t* cfg, uint32
                    w.st, sim->m, P, st) != cudaSuccess)
     return GORGO_ERR_CUDA;
 
-  std::vector<double> parent(x0, x0 + (size_t)P * K), live(parent), f_parent(P, 0.0), sigma(P, cfg->sigma0),
-      value(P, 0.0);
+  // The weights and a step's objective values pass through pinned memory that the kernels read and
+  // write themselves: a hop is two launches and one wait, without copies.
+  const PinLease pin(sim, (size_t)P * (K + 1), st);
+  std::vector<double> own(pin.p ? 0 : (size_t)P * (K + 1));
+  double* const live = pin.p ? pin.p : own.data();          // [P][K]
+  double* const value = live + (size_t)P * K;               // [P]
+  std::copy(x0, x0 + (size_t)P * K, live);
+  std::vector<double> parent(x0, x0 + (size_t)P * K), f_parent(P, 0.0), sigma(P, cfg->sigma0);
   const double down = std::pow(cfg->sigma_up, -0.25);   // one success in five keeps sigma in place
   const uint32_t hist_w = 4 + 2 * T;
   uint64_t done = 0;
   uint32_t step = 0;
   while (done < N) {
     const uint64_t count = std::min<uint64_t>(done == 0 ? cfg->window : cfg->hop, N - done);
-    if (cudaMemcpyAsync(d_params, live.data(), (size_t)P * K * 8, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    if (!pin.p && cudaMemcpyAsync(d_params, live, (size_t)P * K * 8, cudaMemcpyHostToDevice, st) != cudaSuccess)
       return GORGO_ERR_CUDA;
     ReplayArgs a = base_args(sim, base, w);
     a.scale = cfg->time_scale;
     a.first = (uint32_t)done; a.count = (uint32_t)count; a.check_order = 1;
-    a.params = d_params;
+    a.params = pin.p ? live : d_params;
     if (route) a.route_log = route;
     if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
     a.ttft_out = d_ttft + done; a.e2e_out = d_e2e + done; a.out_stride = N;   // request r at [p*N + r]
@@ -1126,15 +1160,15 @@ int gorgo_tune_online(gorgo_sim_t* sim, const gorgo_online_config_t* cfg, uint32
     WindowArgs wa = {};
     wa.values = d_ttft + (done - cfg->window); wa.stride = N;
     wa.window = cfg->window; wa.hop = cfg->hop; wa.n_win = 1;
-    wa.win_p95 = d_p95; wa.win_stride = 1;
-    wa.best = d_p95 + P; wa.best_win = nullptr;
+    wa.win_p95 = pin.p ? value : d_p95; wa.win_stride = 1;
+    wa.best = nullptr; wa.best_win = nullptr;                 // (one window)
     if (launch_window(wa, P, st) != cudaSuccess) return GORGO_ERR_CUDA;
-    if (cudaMemcpyAsync(value.data(), d_p95 + P, (size_t)P * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if ((!pin.p && cudaMemcpyAsync(value, d_p95, (size_t)P * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return GORGO_ERR_CUDA;
     for (uint32_t p = 0; p < P; ++p) {
       double* par = parent.data() + (size_t)p * K;
-      double* lv = live.data() + (size_t)p * K;
+      double* lv = live + (size_t)p * K;
       bool accept = false;
       if (step == 0) {
         f_parent[p] = value[p];                             // the start weights themselves

@@ -163,7 +163,7 @@ struct WindowArgs {
   uint32_t window, hop, n_win;    // window j covers values [j*hop, j*hop + window)
   double* win_p95;                // [P*win_stride] window values (output, also input of the best)
   uint64_t win_stride;
-  double* best;                   // [P] smallest window value
+  double* best;                   // [P] smallest window value, or null
   uint32_t* best_win;             // [P] first window attaining it, or null
 };
 

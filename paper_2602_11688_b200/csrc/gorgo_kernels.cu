@@ -388,7 +388,7 @@ cudaError_t launch_window(const WindowArgs& a, uint32_t n_cand, cudaStream_t st)
     else if (wpad == 256) window_p95_select_kernel<8><<<grid, kWindowThreads, 0, st>>>(a);
     else window_p95_kernel<<<grid, kWindowThreads, smem, st>>>(a, wpad);
   }
-  window_best_kernel<<<n_cand, 256, 0, st>>>(a);
+  if (a.best) window_best_kernel<<<n_cand, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
