@@ -66,13 +66,14 @@ constexpr uint32_t kList = 64;        // requests whose lists the file warp hand
 constexpr uint32_t kInline = 3;       // list entries of a request handed over in shared memory
 constexpr uint32_t kMargin = 512;     // list victims once a cache is this close to full (blocks)
 constexpr uint32_t kHops = 4;         // occurrences looked at before the replica's next requests are asked
+constexpr uint32_t kNews = 4;         // requests after which a replica whose order ran out is looked at again
 constexpr uint32_t kFew = 8;          // requests of a launch up to which victims are not listed ahead
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
-// on the build.  want: the route warp waits for a victim of this replica (+ 1).
+// on the build.  committed: commits whose words are visible; decided: commits made; want: the route warp waits for a victim of this replica (+ 1).
 struct Control {
-  volatile uint32_t routed, timed, filed, listed, exp_ready, committed, want, want_timed, abort_flag;
+  volatile uint32_t routed, timed, filed, listed, exp_ready, committed, decided, want, want_timed, abort_flag;
   volatile int32_t status;
 };
 
@@ -635,9 +636,7 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
   while (true) {
     uint32_t avail = __shfl_sync(kFull, lds32(p_tail), 0) - head;
     if (avail == 0) {                               // the scout is behind: it lists this replica next
-      __threadfence_block();
       if (lane == 0) {
-        sts32(sb + offsetof(Control, committed), r);
         sts64(p_take, make_uint2(head, cons));
         sts32(sb + offsetof(Control, want), rep + 1u);
       }
@@ -858,7 +857,10 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (kExt) st_evict += need;
       held = C;
     }
-    if (lane == 0) sts32(p_occ, held);
+    if (lane == 0) {
+      sts32(p_occ, held);
+      sts32(sb + offsetof(Control, decided), q);
+    }
     PROF_LAP(3);
     // words are visible with `committed`; the fence waits for the reductions in flight, so it is made
     // only every kPublish requests
@@ -943,7 +945,7 @@ __device__ __forceinline__ void time_warp(const ReplayArgs& a, Shared<MaskT, kEx
   const uint32_t seg_mask = (1u << kTimeLanes) - 1u;
   // arrivals base .. base + 127 are in the ring for s in [base, base + 64)
   uint32_t base = a.first;
-  #pragma unroll 1
+#pragma unroll
   for (uint32_t t = lane; t < 2u * kNear; t += 32)
     sh.ts[(base + t) % (2u * kNear)] = base + t < end ? __dmul_rn(scale, __ldg(a.tr.ts + base + t)) : d_inf();
   __syncwarp();
@@ -1217,9 +1219,8 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
       const uint32_t timed = __shfl_sync(kFull, sh.c.timed, 0);
       smem_order();
       const uint32_t n = min(timed - filed, 32u);
-      // many at a time (a pass costs the same for one and for 32), unless the route warp waits for a
-      // victim among them
-      if (n >= kFiled || (n > 0 && (timed == end || __any_sync(kFull, sh.c.want != 0)))) {
+      // many at a time: a pass costs the same for one and for 32
+      if (n >= kFiled || (n > 0 && timed == end)) {
         uint32_t old = kNone, x = kNone;
         const uint32_t j = filed + lane;
         if (lane < n) {
@@ -1303,18 +1304,18 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
   const Touch* touch = a.tr.touch;
   // a launch of a few requests is over before lists made ahead are of use: only what is waited for
   const bool ahead = !a.scout_off && a.count > kFew;
-  uint32_t dry0 = kNone, dry1 = kNone;                 // requests known when the replica's order ran out
+  uint32_t dry0 = a.first - kNews, dry1 = dry0;        // requests known when the replica's order ran out
   uint32_t idle = 0;
+  const uint32_t ring = smem_addr(sh.route_ring);
   PROF_BEGIN();
   #pragma unroll 1
   while (true) {
-    // requests known: in the log, and committed (a touch that a later request touches
-    // again is still a victim of the commits in between)
+    // requests known: those whose commits are made (a touch that a later request touches again is
+    // still a victim of the commits in between).  Routes the file warp has not logged are in the ring.
     const uint32_t filed = __shfl_sync(kFull, sh.c.filed, 0);
-    const uint32_t done = __shfl_sync(kFull, sh.c.committed, 0);
-    const uint32_t seen = (int32_t)(filed - done) < 0 ? filed : done;
-    if (__any_sync(kFull, sh.c.abort_flag != 0 || (int32_t)(done - end) >= 0)) break;
-    const uint32_t want = sh.c.want;
+    const uint32_t seen = __shfl_sync(kFull, sh.c.decided, 0);
+    if (__any_sync(kFull, sh.c.abort_flag != 0 || (int32_t)(seen - end) >= 0)) break;
+    const uint32_t want = __shfl_sync(kFull, sh.c.want, 0);
     smem_order();
     uint32_t best = kNone;
 #pragma unroll
@@ -1322,7 +1323,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       const uint32_t i = lane + 32u * half;
       if (i < R && (want == i + 1u || (ahead && (uint64_t)*(volatile uint32_t*)&sh.occ[i] + kMargin >= a.m.C))) {
         const uint32_t fill = sh.ring_tail[i] - *(volatile uint32_t*)&sh.take[i].x;
-        if (fill * 2u <= a.ring_cap && (half ? dry1 : dry0) != seen) best = min(best, (fill << 8) | i);
+        const uint32_t news = seen - (half ? dry1 : dry0);
+        if (fill * 2u <= a.ring_cap && (news >= kNews || (news && want == i + 1u))) best = min(best, (want == i + 1u ? 0u : 1u << 16) | (fill << 8) | i);
       }
     }
     best = __reduce_min_sync(kFull, best);
@@ -1332,9 +1334,9 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       continue;
     }
     idle = 0;
-    const uint32_t i = best & 255u;
+    const uint32_t i = best & 255u;                    // (what is waited for, else the emptiest list)
     uint32_t tail = sh.ring_tail[i];
-    uint32_t room = a.ring_cap - 1u - (best >> 8);   // (the last victim taken stays readable)
+    uint32_t room = a.ring_cap - 1u - (best >> 8 & 255u);   // (the last victim taken stays readable)
     if (room > 32u) room = 32u;
     uint32_t pos = sh.scan_pos[i], vq = sh.scan_req[i];
     int32_t vk = sh.scan_k[i];
@@ -1344,14 +1346,15 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     const uint32_t budget = room - min(room, (uint32_t)(vk + 1));
     if (budget > 0 && pos < seen) {
       // (a word of four routes per lane and load; the loads of a stretch are in flight together)
-      const uint32_t mis = (uint32_t)(uintptr_t)cd.route_log & 3u, lo = pos + mis, hi = seen + mis, word0 = lo & ~3u;
+      const uint32_t mis = (uint32_t)(uintptr_t)cd.route_log & 3u, log_end = min(filed, seen);
+      const uint32_t lo = pos + mis, hi = max(lo, log_end + mis), word0 = lo & ~3u;
       auto routes = [&](uint32_t u) -> uint32_t {
         const uint32_t x = word0 + 128u * u + 4u * lane;
         return x < hi ? __ldcg(reinterpret_cast<const uint32_t*>(cd.route_log - mis + x)) : 0u;
       };
       uint32_t rt = routes(0), rt1 = routes(1), rt2 = routes(2), rt3 = routes(3);
       #pragma unroll 1
-      for (uint32_t u = 0; u < 4u && n_match < budget && stop < seen; ++u) {
+      for (uint32_t u = 0; u < 4u && n_match < budget && stop < log_end; ++u) {
         const uint32_t x = word0 + 128u * u + 4u * lane;
         uint32_t hit = x < hi ? __vcmpeq4(rt, i * 0x01010101u) : 0u;   // 0xFF in the bytes that are equal
         if (x < lo) hit &= kFull << (8u * (lo - x));
@@ -1372,8 +1375,19 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
           hit &= ~(0xFFu << (8u * b));
         }
         n_match += total;
-        stop = min(word0 + 128u * (u + 1u) - mis, seen);
+        stop = min(word0 + 128u * (u + 1u) - mis, log_end);
         rt = rt1; rt1 = rt2; rt2 = rt3;
+      }
+      #pragma unroll 1
+      while (stop >= log_end && stop < seen && n_match < budget) {
+        const uint32_t r = stop + lane, v = lds32(ring + (r % kRing) * 4u) & 0xFFu;
+        // (none of the entries has been written again: else all these are in the log by now)
+        if (__shfl_sync(kFull, sh.c.routed, 0) - stop >= kRing) break;
+        const unsigned bal = __ballot_sync(kFull, r < seen && v == i);
+        const uint32_t at = n_match + (uint32_t)__popc(bal & ((1u << lane) - 1u));
+        if ((bal >> lane & 1u) && at < kMatches) sh.scan_list[at] = r;
+        n_match += (uint32_t)__popc(bal);
+        stop = min(stop + 32u, seen);
       }
       __syncwarp();
       if (n_match > kMatches) { n_match = kMatches; stop = sh.scan_list[kMatches - 1] + 1u; }
@@ -1416,7 +1430,10 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     bool open = live && t.next != kNone && t.next_req < seen;
     auto step = [&]() {
       const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[t.next].next));
-      if ((uint32_t)__ldcg(cd.route_log + t.next_req) == i) live = open = false;
+      const uint32_t r = t.next_req;
+      uint32_t rt = lds32(ring + (r % kRing) * 4u) & 0xFFu;
+      if (r < filed || sh.c.routed - r >= kRing) rt = (uint32_t)__ldcg(cd.route_log + r);
+      if (rt == i) live = open = false;
       else { t.next = nx.x; t.next_req = nx.y; open = t.next != kNone && t.next_req < seen; }
     };
     if constexpr (sizeof(MaskT) == 4) {
@@ -1441,8 +1458,20 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
           if (other[u] == t.atom) live = open = false;
       }
     }
+    // The rest one by one.  If the route warp waits meanwhile, for what is found already or for another
+    // replica, the touches from the first undecided one on are looked at again next time.
     #pragma unroll 1
-    while (open) step();
+    while (const unsigned rest = __ballot_sync(kFull, open)) {
+      const uint32_t cut = (uint32_t)__ffs((int)rest) - 1u, w = __shfl_sync(kFull, sh.c.want, 0);
+      if (w != 0 && (w != i + 1u || (__ballot_sync(kFull, live) & low_bits(cut)))) {
+        live = live && lane < cut;
+        vq = __shfl_sync(kFull, my_q, cut);
+        vk = (int32_t)__shfl_sync(kFull, my_k, cut);
+        pos = vq + 1u;
+        break;
+      }
+      if (open) step();
+    }
     const unsigned lv = __ballot_sync(kFull, live);
     uint32_t cum = live ? len : 0u;
 #pragma unroll
@@ -1511,7 +1540,14 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   cd.params = a.params ? a.params + (size_t)p * K : a.inline_params;
   cd.scale = a.scales ? a.scales[p] : a.scale;
 
-  if (a.check_order && cd.hdr->processed != a.first) {   // uniform over the CTA
+  // (the first value of every table below: in flight together, a short launch is mostly such latencies)
+  const uint32_t tid = threadIdx.x;
+  const uint32_t processed = cd.hdr->processed;
+  const double w_net = cd.params[0], rtt_0 = tid < GR ? a.tr.rtt[tid] : 0.0, par_0 = tid < K ? cd.params[tid] : 0.0,
+               slot_0 = tid < RS && a.slots_in_smem ? g_slot[tid] : 0.0;
+  RepState rep_0 = {};
+  if (tid < R) rep_0 = cd.rep[tid];
+  if (a.check_order && processed != a.first) {   // uniform over the CTA
     if (threadIdx.x == 0) {
       cd.hdr->status = -8;
       if (a.status_out) a.status_out[p] = -8;
@@ -1519,15 +1555,15 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     return;
   }
 
-  const double w_net = cd.params[0];
-  for (uint32_t i = threadIdx.x; i < GR; i += blockDim.x) {
-    const double v = a.tr.rtt[i];
+  for (uint32_t i = tid; i < GR; i += blockDim.x) {
+    const double v = i == tid ? rtt_0 : a.tr.rtt[i];
     dy.rtt[i] = v;
     dy.wrtt[i] = __dmul_rn(w_net, v);                    // first product of the score
   }
-  for (uint32_t i = threadIdx.x; i < K; i += blockDim.x) sh.w[i] = cd.params[i];
-  for (uint32_t i = threadIdx.x; i < R; i += blockDim.x) {
-    const RepState rs = cd.rep[i];
+  if (tid < K) sh.w[tid] = par_0;                        // (K <= 67)
+  if (tid < R) {
+    const uint32_t i = tid;
+    const RepState rs = rep_0;
     sh.cur_req[i] = rs.cur_req; sh.cur_k[i] = rs.cur_k;
     sh.take[i] = make_uint2(0u, 0u); sh.ring_tail[i] = 0; sh.scan_cum[i] = 0;
     sh.scan_plen[i] = rs.part != kNone ? rs.part_len : 0u;
@@ -1537,7 +1573,7 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     sh.scan_k[i] = rs.cur_req == kNone ? -1 : rs.cur_k;
   }
   if (a.slots_in_smem)
-    for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) dy.free_at[x] = g_slot[x];
+    for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) dy.free_at[x] = x == threadIdx.x ? slot_0 : g_slot[x];
   for (uint32_t i = R + threadIdx.x; i < Shared<MaskT, kExt>::kR; i += blockDim.x) sh.part[i] = make_uint2(kNone, 0u);
   if (threadIdx.x < kRing) sh.near_head[threadIdx.x] = kNone;
   if (threadIdx.x < kStages) {                               // (stages are read before it is known that they are ready)
@@ -1548,7 +1584,7 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   if (threadIdx.x == 0) {
     sh.c.routed = a.first; sh.c.timed = a.first; sh.c.filed = a.first; sh.c.listed = a.first; sh.c.exp_ready = a.first;
     sh.c.abort_flag = 0; sh.c.status = 0;
-    sh.c.committed = a.first; sh.c.want = 0; sh.c.want_timed = a.first;
+    sh.c.committed = a.first; sh.c.decided = a.first; sh.c.want = 0; sh.c.want_timed = a.first;
 #pragma unroll
     for (uint32_t k = 0; k < kChunkRing / kChunkMin; ++k) mbar_init(sh.mbar + k);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -17,8 +17,8 @@ import json
 import numpy as np
 
 ROLES = {
-    "route": (0, ["wait until the request is ready, staged again", "score", "argmin, hand-over", "commit", "eviction",
-                  "publish, next request", None, "#requests not ready in advance",
+    "route": (0, ["commit and score", "argmin, eviction vote", "out of line: commit, eviction", "eviction",
+                  "decided again: waits, staging", "publish, hand-over", None, "#requests decided again",
                   "#requests staged again", "#evictions out of line"]),
     "time": (16, ["wait for a routed request", "times of a group"]),
     "expiry": (32, ["waits", "completions of one request"]),
