@@ -1444,8 +1444,9 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       #pragma unroll 1
       for (uint32_t hop = 0; hop < kHops; ++hop)
         if (open) step();
+      const uint32_t asked = __any_sync(kFull, open) ? n_match : 0u;
       #pragma unroll 1
-      for (uint32_t x = 0; x < n_match && __any_sync(kFull, open); x += 4) {
+      for (uint32_t x = 0; x < asked; x += 4) {
         uint32_t other[4];
 #pragma unroll
         for (uint32_t u = 0; u < 4; ++u) {
@@ -1456,6 +1457,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
 #pragma unroll
         for (uint32_t u = 0; u < 4; ++u)
           if (other[u] == t.atom) live = open = false;
+        if (!__any_sync(kFull, open)) break;
       }
     }
     // The rest one by one.  If the route warp waits meanwhile, for what is found already or for another
