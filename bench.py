@@ -106,7 +106,7 @@ NCU_TRAFFIC = {"longctx": {"bytes_per_candidate_request": (120_785_143_040 + 44_
 
 def kernel_sha16():
     import hashlib
-    src = os.path.join(ROOT, "paper_2602_11688_b200", "csrc", "gorgo_kernels.cu")
+    src = os.path.join(ROOT, "paper_2602_11688_b200", "csrc", "gorgo_replay.cu")
     try:
         return hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
     except OSError:
