@@ -178,7 +178,8 @@ StateLayout make_layout(const Model& m) {
   const uint64_t rs = (uint64_t)m.R * m.S;
   l.slot_off = o; o += rs * 8;
   l.slot_kv_off = o; o += rs * 8;
-  l.more_off = o = (o + 15u) & ~15ull; if (m.R > 32) o += (uint64_t)m.R * 16 * 16;   // (16 listed victims a replica)
+  l.more_off = o = (o + 15u) & ~15ull; if (m.R > 32) o += (uint64_t)m.R * listed_victims(m.R) * 16;
+  l.list_off = o; o += (uint64_t)m.R * (2 * listed_victims(m.R) + 1) * 16;
   l.bytes = align_up(o);
   return l;
 }
@@ -742,6 +743,7 @@ static int upload_impl(gorgo_sim_t* sim, uint64_t N, const double* ts_ms, const 
   tr.n_req = (uint32_t)N; tr.n_touch = (uint32_t)touch.size(); tr.n_atoms = A;
   tr.n_ids = (uint32_t)T; tr.n_distinct = D;
   tr.raw_off = reinterpret_cast<const uint32_t*>(sim->reg.extra);
+  tr.growing = 0;
   // chunks of static data: 16 requests unless these have many touches; room for the largest chunk, but
   // no more than 1.6 times the mean or 40 touches a request (what does not fit is read from global
   // memory)
@@ -841,6 +843,7 @@ static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, co
   const size_t Dn = tb.map.raw.size() - D0;
   tr.n_req = (uint32_t)N; tr.n_touch = (uint32_t)T; tr.n_atoms = (uint32_t)tb.map.raw.size();
   tr.n_ids = (uint32_t)T; tr.n_distinct = tr.n_atoms;
+  tr.growing = 1;
   tr.chunk_req = 4; tr.chunk_cap = 256;          // (a block of a growing trace is an atom: many touches)
 
   DeviceGuard guard(sim->device);

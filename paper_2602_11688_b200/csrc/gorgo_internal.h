@@ -40,7 +40,7 @@ struct __align__(32) RepState {
   int32_t cur_k;      //   next touch of that request to examine (counts down; <0: exhausted)
   uint32_t part;      // atom of which only a leading part is cached (kNone: none)
   uint32_t part_len;  //   blocks of it that are cached
-  uint32_t pad;
+  uint32_t listed;    // victims listed (see StateLayout)
 };
 static_assert(sizeof(RepState) == 32, "RepState layout");
 
@@ -70,6 +70,7 @@ struct TraceView {
   uint32_t n_req, n_touch, n_atoms;
   uint32_t n_ids, n_distinct;        // block ids in total, distinct ones
   // static staging of the replay: requests per chunk (a power of two), touches kept of a chunk
+  uint32_t growing;         // 1: requests can be appended
   uint32_t chunk_req, chunk_cap;
 };
 
@@ -87,8 +88,13 @@ struct StateLayout {
   uint64_t slot_off;       // double[R*S]: time each slot frees (finish of its newest request)
   uint64_t slot_kv_off;    // uint64[R*S]: KV tokens held by each slot's newest request
   uint64_t more_off;       // more than 32 replicas: what is rarely needed of the listed victims
+  uint64_t list_off;       // per replica: uint4 (where the scout stands), then two uint4 per listed victim
   uint64_t bytes;          // size of the block (multiple of 256)
 };
+
+// Victims listed ahead per replica (a power of two): enough for a few commits, no more, because an entry
+// listed long ago has more often been touched again.
+constexpr uint32_t listed_victims(uint32_t n_replicas) { return n_replicas <= 16 ? 32u : 16u; }
 
 // Everything one replay launch needs.  Candidate p of the launch uses element/byte strides.
 struct ReplayArgs {

@@ -49,7 +49,7 @@ __global__ void reset_states_kernel(unsigned char* states, StateLayout lay, uint
   RepState* rep = reinterpret_cast<RepState*>(st + lay.rep_off);
   for (uint32_t i = threadIdx.x; i < R; i += blockDim.x) {
     RepState rs;
-    rs.load = 0; rs.occ = 0; rs.cur_req = kNone; rs.cur_k = -1; rs.part = kNone; rs.part_len = 0; rs.pad = 0;
+    rs.load = 0; rs.occ = 0; rs.cur_req = kNone; rs.cur_k = -1; rs.part = kNone; rs.part_len = 0; rs.listed = 0;
     rep[i] = rs;
   }
   double* slot = reinterpret_cast<double*>(st + lay.slot_off);

@@ -88,7 +88,7 @@ struct Shared {
   // the blocks listed for the replica up to and with it (so that the victims of a commit are found by
   // one comparison per entry, without a scan over their lengths) and the request of the atom's first
   // occurrence after the listing.  The rest (that occurrence's touch, the victim's request, its index there,
-  // -) is read rarely; with 64 replicas it lies in memory, so that three candidates fit an SM.
+  // its touch) is read rarely; with 64 replicas it lies in memory, so that three candidates fit an SM.
   static constexpr uint32_t kVictims = sizeof(MaskT) == 8 ? 1024 : 512;
   static constexpr uint32_t kMore = sizeof(MaskT) == 8 ? 1 : kVictims;
   Control c;
@@ -605,11 +605,11 @@ __device__ __forceinline__ uint32_t dirty_from(const Touch* touch, uint32_t next
 // `next_req`: is its touch still the latest on replica `rep` as of the commit of request r there?
 // `dirty` gets what comes after r.
 __device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* route_log, uint32_t ring, uint32_t next,
-                                            uint32_t next_req, uint32_t r, uint32_t rep, uint32_t& dirty) {
+                                            uint32_t next_req, uint32_t r, uint32_t first, uint32_t rep, uint32_t& dirty) {
   #pragma unroll 1
   while (next != kNone && next_req <= r) {
     const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[next].next));
-    const uint32_t rt = next_req == r ? rep : r - next_req < kRecent ? (lds32(ring + (next_req % kRing) * 4u) & 0xFFu)
+    const uint32_t rt = next_req == r ? rep : r - next_req < kRecent && next_req >= first ? (lds32(ring + (next_req % kRing) * 4u) & 0xFFu)
                                                                      : (uint32_t)__ldcg(route_log + next_req);
     if (rt == rep) return false;
     next = nx.x; next_req = nx.y;
@@ -653,7 +653,7 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     uint32_t d = 0;
     if (listed && next_req < r + kStages) {         // it occurred again since it was listed, or will soon
       const uint32_t next = sizeof(MaskT) == 8 ? __ldcg(&more[e].x) : lds32(sb + (uint32_t)offsetof(Sh, victim_more) + e * 16u);
-      live = victim_live(a.tr.touch, route_log, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, rep, d);
+      live = victim_live(a.tr.touch, route_log, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, a.first, rep, d);
     }
     dirty |= __reduce_or_sync(kFull, d);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
@@ -1486,7 +1486,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       const uint32_t slot = i * a.ring_cap + ((tail + (uint32_t)__popc(lv & ((1u << lane) - 1u))) & (a.ring_cap - 1u));
       sh.victims[slot] = make_uint2(t.atom, cum);
       sh.victim_next[slot] = t.next == kNone ? kNone : t.next_req;
-      more[slot] = make_uint4(t.next, my_q, my_k, 0u);
+      more[slot] = make_uint4(t.next, my_q, my_k, my_off + my_k);
     }
     cum = __shfl_sync(kFull, cum, 31);
     // every lane's entries are stored before lane 0 publishes the new tail
@@ -1510,6 +1510,27 @@ enum Role : uint32_t { kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScou
 constexpr uint32_t kReplayThreads = 32 * kRoles;
 // Register cap: four candidates share an SM (80 registers a thread), three with more than 32 replicas.
 template <typename MaskT> constexpr int kReplayMinCtas = sizeof(MaskT) == 8 ? 3 : 4;
+
+// The lists of the launch before (the end of the kernel says why).  (Out of line: inlined it costs the
+// loops registers.)
+template <typename MaskT, bool kExt>
+__device__ __noinline__ void lists_in(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const uint4* listed, uint4* more) {
+  #pragma unroll 1
+  for (uint32_t x = threadIdx.x; x < a.m.R * a.ring_cap; x += blockDim.x) {
+    const uint32_t i = x / a.ring_cap, e = x % a.ring_cap;
+    if (e < sh.ring_tail[i]) {
+      const uint4* l = listed + (size_t)i * (2u * a.ring_cap + 1u) + 1u + 2u * e;
+      uint4 v = l[0], y = l[1];
+      if (y.x == kNone && a.tr.growing) {              // (it may have grown: any occurrence after the listed one will do)
+        const Touch t = a.tr.touch[y.w];
+        y.x = t.next; v.z = t.next_req;
+      }
+      sh.victims[x] = make_uint2(v.x, v.y);
+      sh.victim_next[x] = v.z;
+      more[x] = y;
+    }
+  }
+}
 
 template <typename MaskT, bool kExt>
 __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_kernel(const __grid_constant__ ReplayArgs a) {
@@ -1542,6 +1563,7 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   cd.params = a.params ? a.params + (size_t)p * K : a.inline_params;
   cd.scale = a.scales ? a.scales[p] : a.scale;
 
+  const uint4* listed = reinterpret_cast<const uint4*>(st + a.lay.list_off);
   // (the first value of every table below: in flight together, a short launch is mostly such latencies)
   const uint32_t tid = threadIdx.x;
   const uint32_t processed = cd.hdr->processed;
@@ -1573,6 +1595,11 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     sh.scan_pos[i] = rs.cur_req == kNone ? 0u : rs.cur_req + 1u;
     sh.scan_req[i] = rs.cur_req;
     sh.scan_k[i] = rs.cur_req == kNone ? -1 : rs.cur_k;
+    if (a.check_order && rs.listed) {                    // the list of the launch before, and where its scout stood
+      const uint4 g = listed[(size_t)i * (2u * a.ring_cap + 1u)];
+      sh.ring_tail[i] = rs.listed;
+      sh.scan_pos[i] = g.x; sh.scan_req[i] = g.y; sh.scan_k[i] = (int32_t)g.z; sh.scan_cum[i] = g.w;
+    }
   }
   if (a.slots_in_smem)
     for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) dy.free_at[x] = x == threadIdx.x ? slot_0 : g_slot[x];
@@ -1590,6 +1617,10 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
 #pragma unroll
     for (uint32_t k = 0; k < kChunkRing / kChunkMin; ++k) mbar_init(sh.mbar + k);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (a.check_order) {
+    __syncthreads();
+    lists_in<MaskT, kExt>(a, sh, listed, sizeof(MaskT) == 8 ? reinterpret_cast<uint4*>(st + a.lay.more_off) : sh.victim_more);
   }
   if (cd.finish_log) {
     // The trace may have grown since the last batch: requests that were to complete after its old
@@ -1634,29 +1665,54 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   else scout_warp<MaskT, kExt>(a, sh, cd, more, lane);
   __syncthreads();
 
+  // (pointers computed again: registers less in the loops)
+  unsigned char* st_end = a.states + (size_t)opaque(blockIdx.x) * a.lay.bytes;
+  RepState* rep_end = reinterpret_cast<RepState*>(st_end + a.lay.rep_off);
+  uint4* lists = reinterpret_cast<uint4*>(st_end + a.lay.list_off);
+  const uint4* more_end = sizeof(MaskT) == 8 ? reinterpret_cast<const uint4*>(st_end + a.lay.more_off) : sh.victim_more;
   // ---- write the small state back; the eviction cursor stands at the next listed touch, or behind
   //      the last one taken
   for (uint32_t i = threadIdx.x; i < R; i += blockDim.x) {
-    RepState s = {(long long)sh.rows[(a.first + a.count - 1u) % Shared<MaskT, kExt>::kRows][i], sh.occ[i], sh.cur_req[i], sh.cur_k[i], sh.part[i].x, sh.part[i].y, 0u};
-    const uint32_t head = sh.take[i].x, tail = sh.ring_tail[i], b = i * a.ring_cap, cap_mask = a.ring_cap - 1u;
+    const uint32_t head = sh.take[i].x, tail = sh.ring_tail[i];
+    RepState s = {(long long)sh.rows[(a.first + a.count - 1u) % Shared<MaskT, kExt>::kRows][i], sh.occ[i], sh.cur_req[i], sh.cur_k[i], sh.part[i].x, sh.part[i].y,
+                  a.check_order ? tail - head : 0u};
+    const uint32_t b = i * a.ring_cap, cap_mask = a.ring_cap - 1u;
     if (tail != head) {
-      const uint4 x = more[b + (head & cap_mask)];
+      const uint4 x = more_end[b + (head & cap_mask)];
       s.cur_req = x.y;
       s.cur_k = (int32_t)x.z;
     } else if (head != 0) {
       const uint32_t e = b + ((head - 1u) & cap_mask);
-      s.cur_req = more[e].y;
-      s.cur_k = (int32_t)more[e].z - 1;
+      s.cur_req = more_end[e].y;
+      s.cur_k = (int32_t)more_end[e].z - 1;
     }
-    cd.rep[i] = s;
+    rep_end[i] = s;
+    if (s.listed) lists[(size_t)i * (2u * a.ring_cap + 1u)] = make_uint4(sh.scan_pos[i], sh.scan_req[i], (uint32_t)sh.scan_k[i], sh.scan_cum[i] - sh.take[i].y);
+  }
+  // A state that goes on keeps the lists: short launches (a tuner's hop, a proxy's request) would else
+  // begin with a scout round per replica, most of it looking again at touches that are superseded.
+  // (Hops of 32 requests, two tuners: 13.4 -> 6.8 ms for 190 launches.)
+  if (a.check_order) {
+    #pragma unroll 1
+    for (uint32_t x = threadIdx.x; x < R * a.ring_cap; x += blockDim.x) {
+      const uint32_t i = x / a.ring_cap, e = x % a.ring_cap;
+      const uint2 tk = sh.take[i];
+      if (e < sh.ring_tail[i] - tk.x) {
+        const uint32_t slot = i * a.ring_cap + ((tk.x + e) & (a.ring_cap - 1u));
+        const uint2 v = sh.victims[slot];
+        uint4* l = lists + (size_t)i * (2u * a.ring_cap + 1u) + 1u + 2u * e;
+        l[0] = make_uint4(v.x, v.y - tk.y, sh.victim_next[slot], 0u);
+        l[1] = more_end[slot];
+      }
+    }
   }
   if (a.slots_in_smem)
-    for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) g_slot[x] = dy.free_at[x];
+    for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) reinterpret_cast<double*>(st_end + a.lay.slot_off)[x] = dy.free_at[x];
   if (threadIdx.x == 0) {
     const int32_t status = sh.c.status;
-    cd.hdr->processed = a.first + a.count;
-    if (status != 0) cd.hdr->status = status;
-    if (a.status_out && (status != 0 || !a.check_order)) a.status_out[p] = status;
+    reinterpret_cast<CandHeader*>(st_end)->processed = a.first + a.count;
+    if (status != 0) reinterpret_cast<CandHeader*>(st_end)->status = status;
+    if (a.status_out && (status != 0 || !a.check_order)) a.status_out[opaque(blockIdx.x)] = status;
   }
 }
 
@@ -1666,9 +1722,7 @@ constexpr size_t kSlotBytes = 40 * 1024;
 template <typename MaskT, bool kExt>
 size_t replay_smem_bytes(ReplayArgs& a) {
   a.slots_in_smem = (size_t)a.m.R * a.m.S * 8 <= kSlotBytes ? 1u : 0u;
-  // victims listed ahead per replica: enough for a few commits, no more, because an entry listed
-  // long ago has more often been touched again
-  a.ring_cap = a.m.R <= 16 ? 32u : 16u;
+  a.ring_cap = listed_victims(a.m.R);
   return shared_bytes<MaskT, kExt>(a.m, a.tr.chunk_req, a.tr.chunk_cap, a.slots_in_smem != 0);
 }
 
