@@ -451,7 +451,7 @@ int gorgo_debug_set(gorgo_sim_t *sim, uint32_t what, uint32_t value);
  * Limit: the scratch of ONE candidate, gorgo_workspace_bytes(sim, 1), must not exceed
  * GORGO_STATIC_SCRATCH_BYTES, else GORGO_ERR_STATIC_LIMIT and nothing runs; a population whose
  * candidates do not all fit at once is evaluated in waves.  (Per candidate the scratch is about
- * 41 bytes per request plus 1 to 8 bytes per distinct block id.)
+ * 37 bytes per request plus 4 or 8 bytes per distinct run of blocks that occur together.)
  * The first call on a device looks up the array's device address; make that first call outside
  * any stream capture.  All calls in a process share the one array per GPU and it keeps what the
  * previous call left there; each call clears what it needs to start from zero, but two calls
