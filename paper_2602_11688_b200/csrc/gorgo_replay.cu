@@ -1305,7 +1305,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
   // a launch of a few requests is over before lists made ahead are of use: only what is waited for
   const bool ahead = !a.scout_off && a.count > kFew;
   uint32_t dry0 = a.first - kNews, dry1 = dry0;        // requests known when the replica's order ran out
-  uint32_t idle = 0;
+  uint32_t idle = 0, idle_at = a.first;                // rounds without anything to do while this many requests were decided
   const uint32_t ring = smem_addr(sh.route_ring);
   PROF_BEGIN();
   #pragma unroll 1
@@ -1329,7 +1329,10 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     }
     best = __reduce_min_sync(kFull, best);
     if (best == kNone) {
-      if (++idle > (1u << 26)) break;                  // bounded wait
+      // The bound is on rounds in which the replay stands still, not on its length: caches may fill late,
+      // and victims have no other source.
+      if (seen != idle_at) { idle_at = seen; idle = 0; }
+      if (++idle > a.poll_limit) { sh.c.status = -6; sh.c.abort_flag = 1; break; }
       __nanosleep(100);
       continue;
     }
