@@ -416,9 +416,11 @@ int gorgo_measure_gather(int device, void *buffer, uint64_t buffer_bytes, uint64
  * decides (prefix hits are read ahead, eviction victims are listed ahead).  These switches let a
  * test take the other paths on purpose; none of them makes a kernel fault or hang.  They apply to
  * every later launch of `sim`.
- *   GORGO_DEBUG_POLL_LIMIT  polls after which a warp gives up waiting (default 2^24).  With 0 the
- *                           first wait that is not already satisfied gives up: the candidate
- *                           finishes with wrong results and status GORGO_ERR_DEVICE_LIMIT.
+ *   GORGO_DEBUG_POLL_LIMIT  polls after which a warp gives up waiting (default 2^24); a walk that
+ *                           another warp is on (over the log, occurrences of a block, a list of
+ *                           completions) does not count.  With 0 the first wait that is not
+ *                           already satisfied gives up: the candidate finishes with wrong results
+ *                           and status GORGO_ERR_DEVICE_LIMIT.
  *   GORGO_DEBUG_RING_POLLS  accepted, without effect (victims are always waited for).
  *   GORGO_DEBUG_PROBE_OFF   nonzero: requests are not staged several at once from words read ahead;
  *                           each is staged alone (results do not depend on it).

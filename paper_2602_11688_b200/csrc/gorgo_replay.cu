@@ -71,10 +71,14 @@ constexpr uint32_t kFew = 8;          // requests of a launch up to which victim
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
-// on the build.  committed: commits whose words are visible; decided: commits made; want: the route warp waits for a victim of this replica (+ 1).
+// on the build.  committed: commits whose words are visible; decided: commits made; want: the route warp
+// waits for a victim of this replica (+ 1); steps, walk, marks: see at_limit.
 struct Control {
   volatile uint32_t routed, timed, filed, listed, exp_ready, committed, decided, want, want_timed, abort_flag;
   volatile int32_t status;
+  volatile uint32_t steps, walk, marks[6];
+  uint32_t scan_pos[64], scan_req[64];   // scout, per replica: next request of the log, request it stands at,
+  int32_t scan_k[64];                    //   touch of it
 };
 
 // Shared memory of one candidate.  Everything with a fixed size comes first: its addresses are
@@ -117,8 +121,7 @@ struct Shared {
   uint32_t cur_req[kR];               // eviction cursor at the start
   int32_t cur_k[kR];
   volatile uint32_t ring_tail[kR];    // victims listed
-  uint32_t scan_pos[kR], scan_req[kR], scan_cum[kR], scan_plen[kR];   // scout: next request of the log, request it stands at,
-  int32_t scan_k[kR];                                        //   touch of it, blocks listed, blocks of a partly evicted touch
+  uint32_t scan_cum[kR], scan_plen[kR];   // scout: blocks listed, blocks of a partly evicted touch
   uint32_t scan_list[kMatches];       // requests found in the log in a pass
   ReqRec c_req[kChunkRing];           // static data of the requests
   uint32_t c_at[kChunkRing];          // index of a request's touches in c_touch (kNone: they are not all there)
@@ -189,10 +192,33 @@ __device__ __forceinline__ void sts32(uint32_t p, uint32_t v) {
   asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
 
+// A walk over the occurrences of an atom, over a replica's order or over a list of completions can be as long
+// as the trace: millions of steps behind a single request.  Those that wait meanwhile have to see that it
+// goes on: the route and expiry warps count their steps here, the scout leaves the number of its step in
+// `walk` and where it stands in scan_*.  (Every such walk is finite: its position only moves forward.)
+__device__ __forceinline__ void count_step(uint32_t sb) {
+  asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(sb + (uint32_t)offsetof(Control, steps)) : "memory");
+}
+// A wait has run into its limit.  It starts again if a decision or a walk has moved since this warp was here
+// before; else the candidate is marked failed, which ends every wait.  (Out of line, and only at the limit: the
+// same look in every poll cost four candidates an SM 8 %.)
+__device__ __noinline__ void at_limit(uint32_t sb) {
+  if ((threadIdx.x & 31u) != 0) return;
+  const uint32_t want = lds32(sb + (uint32_t)offsetof(Control, want)), mark = sb + (uint32_t)offsetof(Control, marks) + threadIdx.x / 32u * 4u;
+  uint32_t now = lds32(sb + (uint32_t)offsetof(Control, decided)) + lds32(sb + (uint32_t)offsetof(Control, steps)) + lds32(sb + (uint32_t)offsetof(Control, walk));
+  if (want != 0) {
+    const uint32_t i = sb + (want - 1u) * 4u;
+    now += 0x9E3779B9u * (lds32(i + (uint32_t)offsetof(Control, scan_pos)) + lds32(i + (uint32_t)offsetof(Control, scan_req)) -
+                          lds32(i + (uint32_t)offsetof(Control, scan_k)));
+  }
+  if (now == lds32(mark)) { sts32(sb + offsetof(Control, status), (uint32_t)-6); sts32(sb + offsetof(Control, abort_flag), 1u); }
+  sts32(mark, now);
+}
+
 // Polls the counter at shared address `p` until (int)(counter - want) >= 0, one lane for the warp.  If
-// the limit runs out (or another warp already gave up) the candidate is marked failed and every later
-// wait returns at once, so the CTA still terminates.  Called by converged warps; every lane gets the
-// same value.  (Out of line: one copy for all waits.)
+// the limit runs out while nothing moves (or another warp already gave up) the candidate is marked failed
+// and every later wait returns at once, so the CTA still terminates.  Called by converged warps; every lane
+// gets the same value.  (Out of line: one copy for all waits.)
 __device__ __noinline__ uint32_t wait_slow(uint32_t p, uint32_t want, uint32_t sb, uint32_t limit) {
   uint32_t v = 0;
   if ((threadIdx.x & 31u) == 0) {
@@ -200,7 +226,7 @@ __device__ __noinline__ uint32_t wait_slow(uint32_t p, uint32_t want, uint32_t s
     #pragma unroll 1
     for (uint32_t polls = 0; (int32_t)(v - want) < 0; ++polls) {
       if (lds32(sb + offsetof(Control, abort_flag))) break;
-      if (polls >= limit) { sts32(sb + offsetof(Control, status), (uint32_t)-6); sts32(sb + offsetof(Control, abort_flag), 1u); break; }
+      if (polls >= limit) { at_limit(sb); polls = 0; }
       if (polls > 4) __nanosleep(20);
       v = lds32(p);
     }
@@ -604,10 +630,11 @@ __device__ __forceinline__ uint32_t dirty_from(const Touch* touch, uint32_t next
 // A listed victim whose atom occurs again before r + kStages, first at touch `next` of request
 // `next_req`: is its touch still the latest on replica `rep` as of the commit of request r there?
 // `dirty` gets what comes after r.
-__device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* route_log, uint32_t ring, uint32_t next,
+__device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* route_log, uint32_t sb, uint32_t ring, uint32_t next,
                                             uint32_t next_req, uint32_t r, uint32_t first, uint32_t rep, uint32_t& dirty) {
   #pragma unroll 1
   while (next != kNone && next_req <= r) {
+    count_step(sb);
     const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[next].next));
     const uint32_t rt = next_req == r ? rep : r - next_req < kRecent && next_req >= first ? (lds32(ring + (next_req % kRing) * 4u) & 0xFFu)
                                                                      : (uint32_t)__ldcg(route_log + next_req);
@@ -653,7 +680,7 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     uint32_t d = 0;
     if (listed && next_req < r + kStages) {         // it occurred again since it was listed, or will soon
       const uint32_t next = sizeof(MaskT) == 8 ? __ldcg(&more[e].x) : lds32(sb + (uint32_t)offsetof(Sh, victim_more) + e * 16u);
-      live = victim_live(a.tr.touch, route_log, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, a.first, rep, d);
+      live = victim_live(a.tr.touch, route_log, sb, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, a.first, rep, d);
     }
     dirty |= __reduce_or_sync(kFull, d);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
@@ -1149,6 +1176,7 @@ __device__ __forceinline__ void expiry_warp(const ReplayArgs& a, Shared<MaskT, k
     uint32_t e = hd.x;
     #pragma unroll 1
     for (uint32_t guard = 0; e != kNone && guard < a.tr.n_req; ++guard) {   // (rarely: more than kInline entries)
+      if (lane == 0) count_step(sb);
       const uint4 rec = __ldcg(exp_rec + e);
       take(make_uint2(rec.y, rec.z));
       e = rec.x;
@@ -1285,11 +1313,34 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
     if (progress) idle = 0;
     else {
       if (__any_sync(kFull, sh.c.abort_flag != 0)) break;
-      if (++idle > a.poll_limit) { sh.c.status = -6; sh.c.abort_flag = 1; break; }
+      // (whom it waits for is at work or in a wait of its own; 2^31 rounds are longer than any walk)
+      if (++idle >> 31) break;
       __nanosleep(100);
     }
   }
   PROF_END(48);
+}
+
+// Asks the replica's next requests (one per lane, `n` of them: number, first touch, touches) for the atom that
+// this lane's touch, the my_k-th of request my_q, holds (kNone: nothing to ask).  True if one has it at the same index.
+__device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
+                                              uint32_t m, uint32_t n) {
+  bool again = false;
+  #pragma unroll 1
+  for (uint32_t x = 0; x < n; x += 4) {
+    uint32_t other[4];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) {
+      const uint32_t y = min(x + u, n - 1u);
+      const uint32_t o = __shfl_sync(kFull, off, y), mm = __shfl_sync(kFull, m, y), qq = __shfl_sync(kFull, rq, y);
+      other[u] = atom != kNone && qq > my_q && my_k < mm ? __ldg(&touch[o + my_k].atom) : kNone - 1u;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u) again = again || other[u] == atom;
+    if (again) atom = kNone;
+    if (!__any_sync(kFull, atom != kNone)) break;
+  }
+  return again;
 }
 
 // ------------------------------------------------------------------------------ scout warp
@@ -1305,8 +1356,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
   // a launch of a few requests is over before lists made ahead are of use: only what is waited for
   const bool ahead = !a.scout_off && a.count > kFew;
   uint32_t dry0 = a.first - kNews, dry1 = dry0;        // requests known when the replica's order ran out
-  uint32_t idle = 0, idle_at = a.first;                // rounds without anything to do while this many requests were decided
-  const uint32_t ring = smem_addr(sh.route_ring);
+  uint32_t idle = 0;
+  const uint32_t sb = smem_addr(&sh), ring = smem_addr(sh.route_ring);
   PROF_BEGIN();
   #pragma unroll 1
   while (true) {
@@ -1329,10 +1380,10 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     }
     best = __reduce_min_sync(kFull, best);
     if (best == kNone) {
-      // The bound is on rounds in which the replay stands still, not on its length: caches may fill late,
-      // and victims have no other source.
-      if (seen != idle_at) { idle_at = seen; idle = 0; }
-      if (++idle > a.poll_limit) { sh.c.status = -6; sh.c.abort_flag = 1; break; }
+      // Only rounds in which the route warp waits for a victim count: a launch may go on for long before a cache
+      // fills, and it ends this warp when it ends.  (The route warp's own limit reports the failure.)
+      idle += want != 0 ? 1u : 0u;
+      if (idle > a.poll_limit) break;
       __nanosleep(100);
       continue;
     }
@@ -1341,8 +1392,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     uint32_t tail = sh.ring_tail[i];
     uint32_t room = a.ring_cap - 1u - (best >> 8 & 255u);   // (the last victim taken stays readable)
     if (room > 32u) room = 32u;
-    uint32_t pos = sh.scan_pos[i], vq = sh.scan_req[i];
-    int32_t vk = sh.scan_k[i];
+    uint32_t pos = sh.c.scan_pos[i], vq = sh.c.scan_req[i];
+    int32_t vk = sh.c.scan_k[i];
     // ---- requests of the replica in the next stretch of the log, in order (the first kMatches)
     uint32_t n_match = 0, off = 0, m = 0, rq = 0;
     uint32_t stop = pos;                               // requests < stop are looked at in this pass
@@ -1439,45 +1490,40 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (rt == i) live = open = false;
       else { t.next = nx.x; t.next_req = nx.y; open = t.next != kNone && t.next_req < seen; }
     };
-    // An atom that occurs in request after request (a prompt many share) would take about R steps.  The
-    // replica's next requests, found above, usually have it at the same index: they are asked first.
-    // (Shared prompts: 8 replicas, 64 candidates 0.99 us per request with the walk alone, 0.78 with this;
-    // 56 replicas, 241 candidates 4.9 and 3.7.)
+    // One occurrence after the other.  An atom that occurs in request after request (a prompt many share) would
+    // take about R steps.  The replica's next requests, found above, usually have it at the same index: they are
+    // asked after the first kHops.  (Shared prompts: 8 replicas, 64 candidates 1.04 us per request with the walk
+    // alone, 0.80 with this; 56 replicas, 241 candidates 5.2 and 3.9.)
+    //   If the route warp waits meanwhile, for what is found already or for another replica, the touches from the
+    // first undecided one on are looked at again next time.  (Found already: the first lane that is live is decided.)
+    //   (One copy of the step for both phases: with two, the loops of all warps are 3 % slower at four candidates an SM.)
     #pragma unroll 1
-    for (uint32_t hop = 0; hop < kHops && __any_sync(kFull, open); ++hop)
-      if (open) step();
-    const uint32_t asked = __any_sync(kFull, open) ? n_match : 0u;
-    #pragma unroll 1
-    for (uint32_t x = 0; x < asked; x += 4) {
-      uint32_t other[4];
-#pragma unroll
-      for (uint32_t u = 0; u < 4; ++u) {
-        const uint32_t y = min(x + u, n_match - 1u);
-        const uint32_t o = __shfl_sync(kFull, off, y), mm = __shfl_sync(kFull, m, y), qq = __shfl_sync(kFull, rq, y);
-        other[u] = open && qq > my_q && my_k < mm ? __ldg(&touch[o + my_k].atom) : kNone;
-      }
-#pragma unroll
-      for (uint32_t u = 0; u < 4; ++u)
-        if (other[u] == t.atom) live = open = false;
-      if (!__any_sync(kFull, open)) break;
-    }
-    // The rest one by one.  If the route warp waits meanwhile, for what is found already or for another
-    // replica, the touches from the first undecided one on are looked at again next time.
-    #pragma unroll 1
-    while (const unsigned rest = __ballot_sync(kFull, open)) {
-      const uint32_t cut = (uint32_t)__ffs((int)rest) - 1u, w = __shfl_sync(kFull, sh.c.want, 0);
-      if (w != 0 && (w != i + 1u || (__ballot_sync(kFull, live) & low_bits(cut)))) {
-        live = live && lane < cut;
-        vq = __shfl_sync(kFull, my_q, cut);
-        vk = (int32_t)__shfl_sync(kFull, my_k, cut);
-        pos = vq + 1u;
-        break;
+    for (uint32_t hop = 0;; ++hop) {
+      unsigned rest = __ballot_sync(kFull, open);
+      if (!rest) break;
+      if (hop >= kHops) {
+        if (hop == kHops && n_match) {
+          if (touched_again(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
+          rest = __ballot_sync(kFull, open);
+          if (!rest) break;
+        }
+        const uint32_t w = __shfl_sync(kFull, sh.c.want, 0);
+        const unsigned found = __ballot_sync(kFull, live);
+        if (w != 0 && (w != i + 1u || !(found & (0u - found) & rest))) {
+          const uint32_t cut = (uint32_t)__ffs((int)rest) - 1u;
+          live = live && lane < cut;
+          vq = __shfl_sync(kFull, my_q, cut);
+          vk = (int32_t)__shfl_sync(kFull, my_k, cut);
+          pos = vq + 1u;
+          break;
+        }
+        sts32(sb + (uint32_t)offsetof(Control, walk), hop);
       }
       if (open) step();
     }
     const unsigned lv = __ballot_sync(kFull, live);
     uint32_t cum = live ? len : 0u;
-#pragma unroll
+    #pragma unroll 1
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t up = __shfl_up_sync(kFull, cum, d);
       if (lane >= (uint32_t)d) cum += up;
@@ -1495,7 +1541,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     __syncwarp();
     smem_order();
     if (lane == 0) {
-      sh.scan_pos[i] = pos; sh.scan_req[i] = vq; sh.scan_k[i] = vk; sh.scan_cum[i] = cum;
+      sh.c.scan_pos[i] = pos; sh.c.scan_req[i] = vq; sh.c.scan_k[i] = vk; sh.scan_cum[i] = cum;
       sh.ring_tail[i] = tail + (uint32_t)__popc(lv);
     }
     if (used == 0 && pos == seen) {                    // the order ran out
@@ -1593,19 +1639,20 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
     sh.take[i] = make_uint2(0u, 0u); sh.ring_tail[i] = 0; sh.scan_cum[i] = 0;
     sh.scan_plen[i] = rs.part != kNone ? rs.part_len : 0u;
     sh.part[i] = make_uint2(rs.part, rs.part_len); sh.occ[i] = rs.occ;
-    sh.scan_pos[i] = rs.cur_req == kNone ? 0u : rs.cur_req + 1u;
-    sh.scan_req[i] = rs.cur_req;
-    sh.scan_k[i] = rs.cur_req == kNone ? -1 : rs.cur_k;
+    sh.c.scan_pos[i] = rs.cur_req == kNone ? 0u : rs.cur_req + 1u;
+    sh.c.scan_req[i] = rs.cur_req;
+    sh.c.scan_k[i] = rs.cur_req == kNone ? -1 : rs.cur_k;
     if (a.check_order && rs.listed) {                    // the list of the launch before, and where its scout stood
       const uint4 g = listed[(size_t)i * (2u * a.ring_cap + 1u)];
       sh.ring_tail[i] = rs.listed;
-      sh.scan_pos[i] = g.x; sh.scan_req[i] = g.y; sh.scan_k[i] = (int32_t)g.z; sh.scan_cum[i] = g.w;
+      sh.c.scan_pos[i] = g.x; sh.c.scan_req[i] = g.y; sh.c.scan_k[i] = (int32_t)g.z; sh.scan_cum[i] = g.w;
     }
   }
   if (a.slots_in_smem)
     for (uint32_t x = threadIdx.x; x < RS; x += blockDim.x) dy.free_at[x] = x == threadIdx.x ? slot_0 : g_slot[x];
   for (uint32_t i = R + threadIdx.x; i < Shared<MaskT, kExt>::kR; i += blockDim.x) sh.part[i] = make_uint2(kNone, 0u);
   if (threadIdx.x < kRing) sh.near_head[threadIdx.x] = kNone;
+  if (threadIdx.x < 6u) sh.c.marks[threadIdx.x] = 0u;
   if (threadIdx.x < kStages) {                               // (stages are read before it is known that they are ready)
     sh.tag[threadIdx.x] = 0u;
     sh.facts[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
@@ -1613,7 +1660,7 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   }
   if (threadIdx.x == 0) {
     sh.c.routed = a.first; sh.c.timed = a.first; sh.c.filed = a.first; sh.c.listed = a.first; sh.c.exp_ready = a.first;
-    sh.c.abort_flag = 0; sh.c.status = 0;
+    sh.c.abort_flag = 0; sh.c.status = 0; sh.c.steps = 0; sh.c.walk = 0;
     sh.c.committed = a.first; sh.c.decided = a.first; sh.c.want = 0; sh.c.want_timed = a.first;
 #pragma unroll
     for (uint32_t k = 0; k < kChunkRing / kChunkMin; ++k) mbar_init(sh.mbar + k);
@@ -1688,7 +1735,7 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
       s.cur_k = (int32_t)more_end[e].z - 1;
     }
     rep_end[i] = s;
-    if (s.listed) lists[(size_t)i * (2u * a.ring_cap + 1u)] = make_uint4(sh.scan_pos[i], sh.scan_req[i], (uint32_t)sh.scan_k[i], sh.scan_cum[i] - sh.take[i].y);
+    if (s.listed) lists[(size_t)i * (2u * a.ring_cap + 1u)] = make_uint4(sh.c.scan_pos[i], sh.c.scan_req[i], (uint32_t)sh.c.scan_k[i], sh.scan_cum[i] - sh.take[i].y);
   }
   // A state that goes on keeps the lists: short launches (a tuner's hop, a proxy's request) would else
   // begin with a scout round per replica, most of it looking again at touches that are superseded.

@@ -28,3 +28,49 @@ def test_caches_that_fill_late():
     w = W.handmade([10.0], reqs, slots=4, cache_blocks=54_000, params=[(1.0, 1.0, 1.0)])
     refs = exact_with_few_polls(w)
     assert int(refs[0][4][3]) == N - 54_000           # evictions begin with request 54,000
+
+
+LONG = 60_000            # requests behind one step of another warp
+
+
+def fleet_of_two(reqs, cache_blocks):
+    """Requests (replica, output tokens, block ids): the network term alone decides, by the origin."""
+    t = [(2.0 * k, 512 * len(ids), out, ids) for k, (_, out, ids) in enumerate(reqs)]
+    return W.handmade([[10.0, 90.0], [90.0, 10.0]], t, slots=4, cache_blocks=cache_blocks, n_regions=2,
+                      origin=[x[0] for x in reqs], params=[(1.0, 0.0, 0.0)])
+
+
+def test_first_eviction_behind_a_long_order():
+    """The cache is far from full until one prompt needs all of it: the whole order of the replica, most
+    of it superseded, is walked while that one commit waits."""
+    reqs = [(2.0 * k, 512, 1, [1]) for k in range(LONG)]
+    reqs += [(2.0 * (LONG + k), 512 * 2_000, 1, list(range(10_000 * (k + 1), 10_000 * (k + 1) + 2_000))) for k in range(3)]
+    w = W.handmade([10.0], reqs, slots=4, cache_blocks=2_000, params=[(1.0, 1.0, 1.0)])
+    assert int(exact_with_few_polls(w)[0][4][3]) == 1 + 2 * 2_000
+
+
+@pytest.mark.parametrize("cache_blocks", [2_000, 8])
+def test_victim_whose_block_occurs_in_every_request(cache_blocks):
+    """Replica 1 sees a block once, replica 0 after that in every request; then replica 1 has to evict it.
+    2,000 blocks: nothing is listed ahead and the scout walks all occurrences; 8: the block is listed at
+    once and the commit walks what occurred since."""
+    reqs = [(1, 1, [7])] + [(0, 1, [7])] * LONG
+    reqs += [(1, 1, list(range(10_000 * (k + 1), 10_000 * (k + 1) + cache_blocks))) for k in range(3)]
+    refs = exact_with_few_polls(fleet_of_two(reqs, cache_blocks))
+    assert int(refs[0][4][3]) == 1 + 2 * cache_blocks
+
+
+def test_replica_with_few_requests_in_a_long_log():
+    """Nearly all requests go to replica 0; the order of replica 1 lies thousands of log words apart."""
+    reqs = [((1 if k % 20_000 == 5 else 0), 1, [1 + k % 3]) for k in range(4 * LONG)]
+    reqs += [(1, 1, list(range(10_000 * (k + 1), 10_000 * (k + 1) + 2_000))) for k in range(3)]
+    exact_with_few_polls(fleet_of_two(reqs, 2_000))
+
+
+def test_completions_of_all_requests_seen_by_one():
+    """All requests are in flight at once and done before the next arrival: their completions are one
+    list of that request."""
+    reqs = [(0.001 * k, 512, 1, [k % 5]) for k in range(LONG)]
+    reqs += [(1e9 + 100.0 * k, 512, 3, [k % 7]) for k in range(300)]
+    w = W.handmade([10.0, 11.0, 12.0], reqs, slots=16, cache_blocks=4, params=[(1.0, 1.0, 1.0)])
+    exact_with_few_polls(w)
