@@ -1343,6 +1343,15 @@ __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom,
   return again;
 }
 
+// With more than 32 replicas it is called, not inlined: where prompts are not shared it is not reached, and inside
+// the scout's loop its code alone cost 64 replicas with 400 candidates 3 % and a small cache with 444 candidates 5 %
+// (1.81 -> 1.66 and 2.35 -> 2.05 us per request out of line; 1.76 and 2.24 without it, where shared prompts
+// take 5.2 instead of 3.9).  Up to 32 replicas the call costs shared prompts 7 % at four candidates an SM.
+__device__ __noinline__ bool touched_again_called(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
+                                                  uint32_t m, uint32_t n) {
+  return touched_again(touch, atom, my_q, my_k, rq, off, m, n);
+}
+
 // ------------------------------------------------------------------------------ scout warp
 // Lists coming victims: for the active replica with the emptiest ring it walks the recency order
 // (the requests of the route log with that replica, deepest touch first) from where it stopped, up to
@@ -1503,7 +1512,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (!rest) break;
       if (hop >= kHops) {
         if (hop == kHops && n_match) {
-          if (touched_again(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
+          if (sizeof(MaskT) == 8 ? touched_again_called(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)
+                                 : touched_again(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
           rest = __ballot_sync(kFull, open);
           if (!rest) break;
         }
