@@ -373,11 +373,11 @@ int eval_impl(gorgo_sim* sim, uint32_t P, const double* params, double scale, vo
     }
     a.first = 0; a.count = (uint32_t)N; a.check_order = 0;
     a.params = wave_params;
-    if (route) a.route_log = route + (size_t)p0 * N;
     a.queue_in_requests = pol && pol->queue_in_requests ? 1u : 0u;
     a.forced_route = pol ? pol->forced_route : nullptr;
     if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
-    a.route_out = nullptr;
+    // (the replay reads its log in words: it is the workspace's, aligned and padded, never the caller's array)
+    a.route_out = route ? route + (size_t)p0 * N : nullptr;
     a.hit_out = hit ? hit + (size_t)p0 * N : nullptr;
     a.ttft_out = reinterpret_cast<double*>(base + w.ttft);
     a.e2e_out = reinterpret_cast<double*>(base + w.e2e);
@@ -1180,8 +1180,8 @@ int gorgo_tune_online(gorgo_sim_t* sim, const gorgo_online_config_t* cfg, uint32
     a.scale = cfg->time_scale;
     a.first = (uint32_t)done; a.count = (uint32_t)count; a.check_order = 1;
     a.params = pin.p ? live : d_params;
-    if (route) a.route_log = route;
     if (attach_speeds(sim, base, w, st, &a) != GORGO_OK) return GORGO_ERR_CUDA;
+    a.route_out = route ? route + done : nullptr;
     a.ttft_out = d_ttft + done; a.e2e_out = d_e2e + done; a.out_stride = N;   // request r at [p*N + r]
     a.status_out = d_status;
     if (launch_replay(a, P, st) != cudaSuccess) return GORGO_ERR_CUDA;

@@ -119,7 +119,8 @@ struct ReplayArgs {
   uint32_t* exp_head;             // [r]: first entry of the list of requests whose completion the
                                   //   proxy sees when request r arrives (kNone: none)
   uint4* exp_rec;                 // [j]: (next entry of j's list, input tokens of j, replica of j, list of late completions)
-  uint8_t* route_log;             // chosen replica of every request replayed so far
+  uint8_t* route_log;             // chosen replica of every request replayed so far; read in words of four: the
+                                  //   array begins 4-byte aligned and is padded to a multiple of 4 bytes
   uint64_t route_log_stride;      // elements between candidates
   // baseline policies: queue signal counted in requests instead of tokens; one fixed route per
   // request of the trace (shared by the candidates of the launch) or null
