@@ -1494,8 +1494,13 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     auto step = [&]() {
       const uint2 nx = __ldg(reinterpret_cast<const uint2*>(&touch[t.next].next));
       const uint32_t r = t.next_req;
-      uint32_t rt = lds32(ring + (r % kRing) * 4u) & 0xFFu;
-      if (r < filed || sh.c.routed - r >= kRing) rt = (uint32_t)__ldcg(cd.route_log + r);
+      bool logged = r < filed;
+      uint32_t rt = 0;
+      if (!logged) {
+        rt = lds32(ring + (r % kRing) * 4u) & 0xFFu;
+        logged = sh.c.routed - r >= kRing;
+      }
+      if (logged) rt = (uint32_t)__ldcg(cd.route_log + r);
       if (rt == i) live = open = false;
       else { t.next = nx.x; t.next_req = nx.y; open = t.next != kNone && t.next_req < seen; }
     };
@@ -1533,7 +1538,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     }
     const unsigned lv = __ballot_sync(kFull, live);
     uint32_t cum = live ? len : 0u;
-    #pragma unroll 1
+#pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t up = __shfl_up_sync(kFull, cum, d);
       if (lane >= (uint32_t)d) cum += up;
