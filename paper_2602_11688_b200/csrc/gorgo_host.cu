@@ -18,9 +18,6 @@
 
 using namespace gorgo;
 
-// 64-bit id -> dense number: open addressing, one 8-byte slot per entry (upper half of the hash,
-// dense number + 1; 0 = empty), so that a lookup costs one cache miss.  The caller's ids by dense
-// number are kept beside it (`raw`) and decide when the upper halves agree.
 // Large host arrays lie on huge pages where the system allows it: the tables of an upload are filled once
 // in random order, and with 4 KB pages their first touches and TLB misses are a third of its time.
 template <typename T>
@@ -46,11 +43,14 @@ struct HugePages {
 };
 template <typename T> using HugeVector = std::vector<T, HugePages<T>>;
 
+// 64-bit id -> dense number: open addressing, one 8-byte slot per entry (upper half of the hash,
+// dense number + 1; 0 = empty), so that a lookup costs one cache miss.  The caller's ids by dense
+// number are kept beside it (`raw`) and decide when the upper halves agree.
 struct IdMap {
   HugeVector<uint64_t> slot;
   HugeVector<uint64_t> raw;
   uint64_t mask = 0;
-  static uint64_t hash(uint64_t z) {
+  static uint64_t hash(uint64_t z) {               // 64-bit finaliser of MurmurHash3 (A. Appleby)
     z ^= z >> 33; z *= 0xff51afd7ed558ccdULL; z ^= z >> 33; z *= 0xc4ceb9fe1a85ec53ULL;
     return z ^ (z >> 33);
   }
@@ -90,7 +90,7 @@ struct IdMap {
 // its own: requests to come may share any part of what is known so far.
 struct TraceBuilder {
   IdMap map{1ull << 12};
-  std::vector<uint32_t> last_g, last_r;   // per dense id: touch and request of its last occurrence
+  std::vector<uint32_t> last_g;           // per dense id: touch of its last occurrence
   std::vector<double> ts;                 // arrival times so far
   uint64_t T = 0;                         // block ids so far
   uint64_t grid_cursor = 0;               // first request not yet behind the last grid edge
@@ -284,13 +284,13 @@ bool all_finite(const double* v, uint64_t n) {
 
 bool finite_nonneg(double v) { return std::isfinite(v) && v >= 0.0; }
 
-// Rolling-window objective asked for with an evaluation (all pointers DEVICE).
 // Baseline policy asked for with an evaluation.
 struct PolicySpec {
   bool queue_in_requests;
   const uint8_t* forced_route;   // DEVICE [N] or null
 };
 
+// Rolling-window objective asked for with an evaluation (all pointers DEVICE).
 struct WindowSpec {
   uint32_t window, hop;
   double* win_p95;      // [P * n_windows] or null
@@ -572,7 +572,7 @@ static int check_requests(const Model& m, uint64_t n, double prev_t, const doubl
     if (g >= m.G) return GORGO_ERR_BAD_TRACE;
     ReqRec& q = req[k];
     q.ts_ms = t; q.off = 0; q.in_tok = input_tokens[k]; q.out_tok = output_tokens[k];
-    q.m = 0; q.origin = g; q.prev_share = kNone; q.nblk = (uint32_t)nb;
+    q.m = 0; q.origin = g; q.pad = 0; q.nblk = (uint32_t)nb;
   }
   return GORGO_OK;
 }
@@ -721,7 +721,6 @@ static int upload_impl(gorgo_sim_t* sim, uint64_t N, const double* ts_ms, const 
   std::vector<Around> last(A, Around{kNone, kNone});   // touch and request of an atom's last occurrence
   for (uint64_t r = 0; r < N; ++r) {
     req[r].off = (uint32_t)touch.size();
-    uint32_t latest = 0;                         // latest earlier request (+1) that shares an atom
     for (uint64_t g = hash_off[r]; g < hash_off[r + 1];) {
       const uint32_t at = atom_at[dense[g]];
       const uint32_t len = head[at + 1] - head[at];
@@ -730,14 +729,12 @@ static int upload_impl(gorgo_sim_t* sim, uint64_t N, const double* ts_ms, const 
       if (la.pred != kNone) {
         if (la.succ == (uint32_t)r) return GORGO_ERR_BAD_TRACE;   // an id twice in one request
         touch[la.pred].next = here; touch[la.pred].next_req = (uint32_t)r;
-        if (la.succ + 1 > latest) latest = la.succ + 1;
       }
       la.pred = here; la.succ = (uint32_t)r;
       touch.push_back({at, len | (uint32_t)(g - hash_off[r]) << 16, kNone, kNone});
       g += len;
     }
     req[r].m = (uint16_t)(touch.size() - req[r].off);
-    req[r].prev_share = latest ? latest - 1 : kNone;
   }
   TraceView& tr = sim->tr;
   tr.n_req = (uint32_t)N; tr.n_touch = (uint32_t)touch.size(); tr.n_atoms = A;
@@ -818,22 +815,19 @@ static int append_impl(gorgo_sim_t* sim, uint64_t n_new, const double* ts_ms, co
     const uint32_t r = (uint32_t)(N0 + k);
     req[k].off = (uint32_t)(T0 + hash_off[k]);
     req[k].m = (uint16_t)req[k].nblk;
-    uint32_t latest = 0;
     for (uint64_t gl = hash_off[k]; gl < hash_off[k + 1]; ++gl) {
       const uint32_t d = tb.map.get_or_add(hash_ids[gl]);
       const uint32_t g = (uint32_t)(T0 + gl);
       touch[gl] = {d, 1u | (uint32_t)(gl - hash_off[k]) << 16, kNone, kNone};
       if (d == tb.last_g.size()) {
-        tb.last_g.push_back(g); tb.last_r.push_back(r);
+        tb.last_g.push_back(g);
         continue;
       }
       const uint32_t pg = tb.last_g[d];
-      if (tb.last_r[d] + 1 > latest) latest = tb.last_r[d] + 1;
       if (pg >= T0) { touch[pg - T0].next = g; touch[pg - T0].next_req = r; }
       else { prev[gl] = pg; ++n_links; }
-      tb.last_g[d] = g; tb.last_r[d] = r;
+      tb.last_g[d] = g;
     }
-    req[k].prev_share = latest ? latest - 1 : kNone;
   }
   tb.ts.insert(tb.ts.end(), ts_ms, ts_ms + n_new);
   tb.T = T;

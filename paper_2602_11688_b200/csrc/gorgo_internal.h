@@ -15,7 +15,7 @@ struct __align__(32) ReqRec {
   uint32_t out_tok;     // output tokens
   uint16_t m;           // touches (atoms) of the request
   uint16_t origin;      // origin region
-  uint32_t prev_share;  // latest earlier request that shares a block with this one (kNone: none)
+  uint32_t pad;
   uint32_t nblk;        // blocks of the request
 };
 static_assert(sizeof(ReqRec) == 32, "ReqRec must be one sector");
@@ -195,12 +195,9 @@ cudaError_t launch_policy_routes(const TraceView& tr, uint32_t R, bool affinity,
                                  const uint32_t* draws, uint8_t* route, cudaStream_t st);
 #ifdef GORGO_PROF
 // Cycle accounting build only: 16 accumulators per role (route 0, time 16, expiry 32, file 48,
-// scout 64, stage 80, commit 96).
+// scout 64, stage 80; 96 to 111 stay 0).
 cudaError_t prof_read(unsigned long long* out112, bool reset);
 #endif
-// After requests [first_new, first_new + n_new) were appended to a growing trace: every block of
-// theirs that occurred before gets its previous occurrence (`prev[i]` of the i-th new touch)
-// linked to it.
 // What a small append writes, carried by the launch itself: runs of words for up to five places, then the
 // triples (touch of an earlier batch, its new successor, the successor's request).
 struct AppendPayload {
@@ -212,6 +209,9 @@ struct AppendPayload {
   uint32_t words[kWords];
 };
 cudaError_t launch_append(const AppendPayload& a, cudaStream_t st);
+// After requests [first_new, first_new + n_new) were appended to a growing trace: every block of
+// theirs that occurred before gets its previous occurrence (`prev[i]` of the i-th new touch)
+// linked to it.
 cudaError_t launch_link_occurrences(const TraceView& tr, uint32_t first_new, uint32_t n_new,
                                     const uint32_t* prev, Touch* touch, cudaStream_t st);
 cudaError_t launch_gather(const void* buf, uint64_t n_sectors, uint32_t per_thread, uint32_t blocks,

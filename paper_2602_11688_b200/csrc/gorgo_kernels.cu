@@ -6,8 +6,8 @@ namespace gorgo {
 
 namespace {
 
-// ------------------------------------------------------------------------------- reset
-// One thread per appended touch: a block whose previous occurrence belongs to an earlier batch
+// ------------------------------------------------------------------------- growing trace
+// One warp per appended request: a block whose previous occurrence belongs to an earlier batch
 // becomes that occurrence's successor.
 __global__ void link_occurrences_kernel(TraceView tr, uint32_t first_new, uint32_t n_new, const uint32_t* prev,
                                         Touch* touch) {
@@ -37,6 +37,7 @@ __global__ void append_kernel(const __grid_constant__ AppendPayload a) {
   }
 }
 
+// ------------------------------------------------------------------------------- reset
 __global__ void reset_states_kernel(unsigned char* states, StateLayout lay, uint32_t R, uint32_t S,
                                     uint32_t n_cand) {
   const uint32_t p = blockIdx.x;
