@@ -27,8 +27,10 @@
 // Measured with straight-line loops on eight warps, an SM runs at full rate up to about 28 KB of code
 // and fetches about one instruction per cycle beyond.  Splitting the route warp further (argmin and
 // commits apart, two commit warps) gave 1.07 us per request at one candidate per SM and 1.8 at two;
-// this split gives 0.73 and 0.78, and 1.35 at four (long-context trace, 16 replicas, 20,000 requests; the
-// twelve-warp kernel on blocks before it 1.1, 1.35 and 2.7).
+// this split gives 0.73, 0.84, 1.09 and 1.32 at one to four (long-context trace, 16 replicas, 20,000 requests,
+// 4,000 blocks a cache; the twelve-warp kernel on blocks before it 1.09, 1.39, 2.65 and 2.77).  The loops are
+// still over the cache: with three or four candidates an SM 128 bytes more in one of them cost about 3 %,
+// so what is rare is out of line, and loops that could share a body do.
 #include "gorgo_device.cuh"
 
 namespace gorgo {
@@ -64,11 +66,25 @@ constexpr uint32_t kNear = 64;        // completions within fewer than this many
 constexpr uint32_t kFiled = 16;      // requests the file warp waits for
 constexpr uint32_t kList = 64;        // requests whose lists the file warp hands over ahead
 constexpr uint32_t kInline = 3;       // list entries of a request handed over in shared memory
-constexpr uint32_t kMargin = 512;     // list victims once a cache is this close to full (blocks)
-constexpr uint32_t kHops = 4;         // occurrences looked at before the replica's next requests are asked
-constexpr uint32_t kNews = 4;         // requests after which a replica whose order ran out is looked at again
-constexpr uint32_t kFew = 8;          // requests of a launch up to which victims are not listed ahead
-constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round
+// (Rules of the scout.  The times are us per request on reduced cases unless they say otherwise.)
+// List victims once a cache is this close to full (blocks).  64, 512 and 2,048 give the same times everywhere
+// (within 1 %): a cache passes the margin once, and a list holds 16 or 32 entries.  A few prompts' worth.
+constexpr uint32_t kMargin = 512;
+// Occurrences looked at before the replica's next requests are asked.  2 / 4 / 8 / 16, shared prompts: 8 replicas
+// 0.96 / 0.80 / 0.77 / 0.82, and with a cache of one long prompt 0.77 / 0.79 / 0.83 / 0.88; 32 replicas 2.1 / 2.13 /
+// 2.28 / 2.60; 56 replicas 3.87 / 3.90 / 4.04 / 4.47.  Prompts that are not shared: no difference.
+constexpr uint32_t kHops = 4;
+// Requests after which a replica whose order ran out is looked at again.  1 / 4 / 16, a cache of one long prompt:
+// 1 replica 1.00 / 1.18 / 1.51, 2 replicas 0.93 / 0.96 / 1.35, 16 replicas 0.99 / 0.95 / 0.95, 64 replicas 1.32 / 1.27 /
+// 1.23; larger caches run out of nothing.
+constexpr uint32_t kNews = 4;
+// Requests of a launch up to which victims are listed only when a commit waits for one.  A proxy waits for every
+// launch, and the round the scout is in when the last request is done is part of that: appended and routed one by
+// one 39 us (regions) and 45 us (long context), with lists made ahead 44 and 50; two at a time 41 and 48 (regions);
+// four to eight within 5 % either way; at 16 the lists win, 91 and 84.  Launches of an uploaded trace that follow one
+// another without a wait would take them from two requests on: 8 requests 26.5 and 21.8 us.
+constexpr uint32_t kFew = 8;
+constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round: one per lane
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
 // on the build.  committed: commits whose words are visible; decided: commits made; want: the route warp
@@ -1362,7 +1378,6 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
                                            uint32_t lane) {
   const uint32_t R = a.m.R, end = a.first + a.count;
   const Touch* touch = a.tr.touch;
-  // a launch of a few requests is over before lists made ahead are of use: only what is waited for
   const bool ahead = !a.scout_off && a.count > kFew;
   uint32_t dry0 = a.first - kNews, dry1 = dry0;        // requests known when the replica's order ran out
   uint32_t idle = 0;
@@ -1506,11 +1521,11 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
     };
     // One occurrence after the other.  An atom that occurs in request after request (a prompt many share) would
     // take about R steps.  The replica's next requests, found above, usually have it at the same index: they are
-    // asked after the first kHops.  (Shared prompts: 8 replicas, 64 candidates 1.04 us per request with the walk
-    // alone, 0.80 with this; 56 replicas, 241 candidates 5.2 and 3.9.)
+    // asked after the first kHops.  (Shared prompts: 8 replicas, 64 candidates 1.09 us per request with the walk
+    // alone, 0.80 with this; 32 replicas 3.85 and 2.13; 56 replicas, 241 candidates 5.2 and 3.9.)
     //   If the route warp waits meanwhile, for what is found already or for another replica, the touches from the
     // first undecided one on are looked at again next time.  (Found already: the first lane that is live is decided.)
-    //   (One copy of the step for both phases: with two, the loops of all warps are 3 % slower at four candidates an SM.)
+    //   (One copy of the step for both phases: with two, four candidates an SM take 1.41 instead of 1.33 us.)
     #pragma unroll 1
     for (uint32_t hop = 0;; ++hop) {
       unsigned rest = __ballot_sync(kFull, open);

@@ -1,8 +1,8 @@
 """GPU parity on the paths of the replay kernel that ordinary traces rarely or never take:
-prompts longer than a shared-memory stage, replays without the helper warps (the probe warps
-that stage prefix hits ahead, the scout warps that pre-validate eviction victims), a wait that
-runs out, and the hand-worked timing cases.  Everything goes through the C ABI; results are
-compared bit for bit with the CPU oracle."""
+prompts longer than a shared-memory stage, replays in which nothing is prepared ahead (every request
+staged alone, every victim listed only when a commit waits for it), a wait that runs out, and the
+hand-worked timing cases.  Everything goes through the C ABI; results are compared bit for bit with
+the CPU oracle."""
 import numpy as np
 import pytest
 
@@ -49,34 +49,38 @@ def test_prompts_longer_than_a_stage(R, max_blocks, C):
     assert max(int(r[0].hit.max()) for r in refs) > min(128, max_blocks // 2)   # long prefix hits
 
 
-def _switches(gb, probe_off, scout_off, ring_polls):
-    d = {gb.GORGO_DEBUG_PROBE_OFF: int(probe_off), gb.GORGO_DEBUG_SCOUT_OFF: int(scout_off)}
-    if ring_polls is not None:
-        d[gb.GORGO_DEBUG_RING_POLLS] = ring_polls
-    return d
+def _switches(gb, probe_off, scout_off):
+    return {gb.GORGO_DEBUG_PROBE_OFF: int(probe_off), gb.GORGO_DEBUG_SCOUT_OFF: int(scout_off)}
 
 
-@pytest.mark.parametrize("probe_off,scout_off,ring_polls", [(1, 0, None), (0, 1, 0), (1, 1, 0),
-                                                            (0, 0, 0)])
+@pytest.mark.parametrize("probe_off,scout_off", [(1, 0), (0, 1), (1, 1), (0, 0)])
 @pytest.mark.parametrize("R,structured", [(3, True), (9, False), (17, True), (33, False), (64, True)])
-def test_small_traces_without_the_helper_warps(R, structured, probe_off, scout_off, ring_polls):
-    """The probe and scout warps only prepare work ahead of time: without them (every request
-    probed by the gate warp, every victim found by the commit warps themselves) the bits are the
-    same."""
+def test_small_traces_with_nothing_prepared_ahead(R, structured, probe_off, scout_off):
+    """What the stage and scout warps prepare ahead of time only takes work off the commits.  Without
+    it (requests staged one at a time with the words as they are then, victims listed by the scout only
+    when the route warp waits for one) the bits are the same."""
     from paper_2602_11688_b200 import binding as gb
     rng = np.random.default_rng(R)
     reqs = small_trace(R + 3, n_req=400, structured=structured)
     params = rng.normal(1.0, 0.3, size=(4, 3))
     w = W.handmade(rng.uniform(5, 60, size=R), reqs, slots=2, cache_blocks=9, params=params)
-    check_population(w, scale=1.0, debug=_switches(gb, probe_off, scout_off, ring_polls))
+    check_population(w, scale=1.0, debug=_switches(gb, probe_off, scout_off))
 
 
-@pytest.mark.parametrize("probe_off,scout_off,ring_polls", [(1, 0, None), (0, 1, 0), (1, 1, 0)])
-def test_longctx_reduced_without_the_helper_warps(probe_off, scout_off, ring_polls):
+@pytest.mark.parametrize("probe_off,scout_off", [(1, 0), (0, 1), (1, 1)])
+def test_longctx_reduced_with_nothing_prepared_ahead(probe_off, scout_off):
     from paper_2602_11688_b200 import binding as gb
     w = W.make_workload("longctx", n_requests=12_000, cache_blocks=3_000, population=6)
-    gpu, refs = check_population(w, debug=_switches(gb, probe_off, scout_off, ring_polls))
+    gpu, refs = check_population(w, debug=_switches(gb, probe_off, scout_off))
     assert sum(int(r[4][3]) for r in refs) > 0
+
+
+def test_the_switch_without_effect_is_accepted():
+    """GORGO_DEBUG_RING_POLLS selected a path that no longer exists: any value is taken and changes nothing."""
+    from paper_2602_11688_b200 import binding as gb
+    w = W.make_workload("tiny", n_requests=400, cache_blocks=150, population=3)
+    for value in (0, 1, 2 ** 32 - 1):
+        check_population(w, debug={gb.GORGO_DEBUG_RING_POLLS: value})
 
 
 def test_a_wait_that_runs_out_is_reported_and_nothing_hangs():
