@@ -418,7 +418,8 @@ int gorgo_measure_gather(int device, void *buffer, uint64_t buffer_bytes, uint64
  * every later launch of `sim`.
  *   GORGO_DEBUG_POLL_LIMIT  polls after which a warp gives up waiting (default 2^24); a walk that
  *                           another warp is on (over the log, occurrences of a block, a list of
- *                           completions) does not count.  With 0 the first wait that is not
+ *                           completions) does not count, and under a KV budget S*S/4 polls are
+ *                           added for its rounds over the S slots.  With 0 the first wait that is not
  *                           already satisfied gives up: the candidate finishes with wrong results
  *                           and status GORGO_ERR_DEVICE_LIMIT.
  *   GORGO_DEBUG_RING_POLLS  accepted, without effect (victims are always waited for).

@@ -230,7 +230,10 @@ uint64_t reset_bytes(const gorgo_sim* sim, const WsLayout& w) { return sim->prox
 ReplayArgs base_args(const gorgo_sim* sim, unsigned char* base, const WsLayout& w) {
   ReplayArgs a = {};
   a.m = sim->m; a.tr = sim->tr;
-  a.poll_limit = sim->poll_limit;
+  // Under a KV budget one request may be moved past the finish of every other slot, each time with a look at
+  // all slots: S * S / 8 reads behind one wait of another warp, a poll each two at most.
+  const uint64_t rounds = sim->kv_budget ? (uint64_t)sim->m.S * sim->m.S / 4 : 0;
+  a.poll_limit = (uint32_t)std::min<uint64_t>(sim->poll_limit + rounds, 0xFFFFFFFFu);
   a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
   a.masks = base + w.masks; a.mask_stride = w.mask_stride; a.index_off = w.index_off;
   a.states = base + w.states; a.lay = w.st;

@@ -74,3 +74,23 @@ def test_completions_of_all_requests_seen_by_one():
     reqs += [(1e9 + 100.0 * k, 512, 3, [k % 7]) for k in range(300)]
     w = W.handmade([10.0, 11.0, 12.0], reqs, slots=16, cache_blocks=4, params=[(1.0, 1.0, 1.0)])
     exact_with_few_polls(w)
+
+
+def test_admission_that_waits_for_hundreds_of_slots():
+    """A KV budget of one request and thousands of slots: every request moves past the finish of all before
+    it, and each of these rounds looks at all slots."""
+    from paper_2602_11688_b200 import binding as gb
+    from oracle import gorgo_oracle as O
+    import torch
+    N = 300
+    reqs = [(0.01 * k, 512, 3, [k]) for k in range(N)]
+    w = W.handmade([10.0], reqs, slots=2_048, cache_blocks=64, params=[(1.0, 1.0, 1.0)])
+    sim = gb.GorgoSim(w)
+    assert gb.gorgo_sim_set_service_model(sim.h, 0.0, 515) == gb.GORGO_OK
+    assert gb.gorgo_debug_set(sim.h, gb.GORGO_DEBUG_POLL_LIMIT, POLLS) == gb.GORGO_OK
+    out = sim.eval_population(w.params, 1.0, want_route=True)
+    torch.cuda.synchronize()
+    assert int(out["status"].item()) == 0
+    _, p95_ttft, p95_e2e, _, _ = O.replay(w, w.params[0], 1.0, kv_budget_tokens=515)
+    assert float(out["p95_ttft"].item()) == p95_ttft and float(out["p95_e2e"].item()) == p95_e2e
+    sim.close()
