@@ -451,10 +451,13 @@ int gorgo_debug_set(gorgo_sim_t *sim, uint32_t what, uint32_t value);
  * each), `route` DEVICE P*N bytes or NULL, `hit_blocks` DEVICE P*N uint16 or NULL, `cand_status`
  * DEVICE P int32 or NULL: 0, or GORGO_ERR_DEVICE_LIMIT for a candidate whose replay gave up on a
  * bounded wait (its outputs are then meaningless; read it after synchronising the stream).
- * Limit: the scratch of ONE candidate, gorgo_workspace_bytes(sim, 1), must not exceed
- * GORGO_STATIC_SCRATCH_BYTES, else GORGO_ERR_STATIC_LIMIT and nothing runs; a population whose
- * candidates do not all fit at once is evaluated in waves.  (Per candidate the scratch is about
- * 37 bytes per request plus 4 or 8 bytes per distinct run of blocks that occur together.)
+ * Limit: the scratch of ONE candidate must not exceed GORGO_STATIC_SCRATCH_BYTES, else
+ * GORGO_ERR_STATIC_LIMIT and nothing runs; a population whose candidates do not all fit at once is
+ * evaluated in waves.  That scratch is gorgo_workspace_bytes(sim, 1), less the words of the proxy
+ * index while that is off (so a trace for which gorgo_workspace_bytes(sim, 1) fits always runs):
+ * 37 bytes per request and candidate and 5 per request beside them, 4 or 8 bytes (up to 32 replicas,
+ * or more) per distinct run of blocks that occur together, and per replica 1,072 bytes (560 above 16
+ * replicas, 816 above 32) and 16 per slot.
  * The first call on a device looks up the array's device address; make that first call outside
  * any stream capture.  All calls in a process share the one array per GPU and it keeps what the
  * previous call left there; each call clears what it needs to start from zero, but two calls

@@ -130,7 +130,7 @@ def test_static_scratch_entry_point_runs_in_waves_when_the_population_does_not_f
 def test_static_scratch_entry_point_refuses_a_trace_beyond_its_limit():
     import torch
     from paper_2602_11688_b200 import binding as gb
-    N = 2_200_000                                            # ~41 bytes of scratch per request
+    N = 2_200_000                                            # 42 bytes of scratch per request
     spec = W.WorkloadSpec(name="too-long", seed=0, n_replicas=2, n_regions=1, n_requests=N,
                           n_sessions=1, cache_blocks=8, slots=2, population=1)
     w = W.Workload(spec=spec, rtt_ms=np.array([[10.0, 20.0]]),
