@@ -1339,22 +1339,33 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
 
 // Asks the replica's next requests (one per lane, `n` of them: number, first touch, touches) for the atom that
 // this lane's touch, the my_k-th of request my_q, holds (kNone: nothing to ask).  True if one has it at the same index.
+//   Usually a few lanes ask and twenty or thirty requests are asked, so the requests go by lane and the askers one
+// after the other (kAsk of them with their loads in flight together): one memory latency per asker.  (The askers by lane
+// and the requests one after the other, four at a time: shared prompts, 8 replicas, 64 candidates 0.81 us per request,
+// with this 0.78.  More than one asker in flight is no faster there, and its code in the scout's loop costs four candidates an SM
+// 2 % (two) to 5 % (four); with more than 32 replicas, where the function is called, 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
+template <uint32_t kAsk>
 __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
                                               uint32_t m, uint32_t n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  unsigned open = __ballot_sync(kFull, atom != kNone);
   bool again = false;
   #pragma unroll 1
-  for (uint32_t x = 0; x < n; x += 4) {
-    uint32_t other[4];
+  while (open) {
+    uint32_t got[kAsk], want[kAsk], src[kAsk];
 #pragma unroll
-    for (uint32_t u = 0; u < 4; ++u) {
-      const uint32_t y = min(x + u, n - 1u);
-      const uint32_t o = __shfl_sync(kFull, off, y), mm = __shfl_sync(kFull, m, y), qq = __shfl_sync(kFull, rq, y);
-      other[u] = atom != kNone && qq > my_q && my_k < mm ? __ldg(&touch[o + my_k].atom) : kNone - 1u;
+    for (uint32_t u = 0; u < kAsk; ++u) {
+      src[u] = open ? (uint32_t)__ffs((int)open) - 1u : 32u;
+      open &= open - 1u;
+      const uint32_t from = src[u] & 31u, q = __shfl_sync(kFull, my_q, from), k = __shfl_sync(kFull, my_k, from);
+      want[u] = __shfl_sync(kFull, atom, from);
+      got[u] = src[u] < 32u && lane < n && rq > q && k < m ? __ldg(&touch[off + k].atom) : kNone;
     }
 #pragma unroll
-    for (uint32_t u = 0; u < 4; ++u) again = again || other[u] == atom;
-    if (again) atom = kNone;
-    if (!__any_sync(kFull, atom != kNone)) break;
+    for (uint32_t u = 0; u < kAsk; ++u) {
+      const bool has = __any_sync(kFull, got[u] == want[u] && got[u] != kNone);
+      again = again || (lane == src[u] && has);
+    }
   }
   return again;
 }
@@ -1365,7 +1376,7 @@ __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom,
 // take 5.2 instead of 3.9).  Up to 32 replicas the call costs shared prompts 7 % at four candidates an SM.
 __device__ __noinline__ bool touched_again_called(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
                                                   uint32_t m, uint32_t n) {
-  return touched_again(touch, atom, my_q, my_k, rq, off, m, n);
+  return touched_again<4>(touch, atom, my_q, my_k, rq, off, m, n);
 }
 
 // ------------------------------------------------------------------------------ scout warp
@@ -1533,7 +1544,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (hop >= kHops) {
         if (hop == kHops && n_match) {
           if (sizeof(MaskT) == 8 ? touched_again_called(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)
-                                 : touched_again(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
+                                 : touched_again<1>(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
           rest = __ballot_sync(kFull, open);
           if (!rest) break;
         }
