@@ -74,6 +74,13 @@ constexpr uint32_t kMargin = 512;
 // 0.96 / 0.80 / 0.77 / 0.82, and with a cache of one long prompt 0.77 / 0.79 / 0.83 / 0.88; 32 replicas 2.1 / 2.13 /
 // 2.28 / 2.60; 56 replicas 3.87 / 3.90 / 4.04 / 4.47.  Prompts that are not shared: no difference.
 constexpr uint32_t kHops = 4;
+// Quarters of a list up to which it is filled again.  A commit that takes more victims than are listed waits for a
+// scout round, 5,000 to 10,000 ticks.  Filled again from half a list down, that was 7 commits in 100 on small caches (lists
+// of 16, found with 10 entries, 14 taken) and 2 with shared prompts; the scout idles for two thirds of the time.
+// Half / 5 eighths / 3 quarters / 7 eighths: 32 replicas, 148 candidates 1.18 / 1.13 / 1.11 / 1.11 us per request, 480 candidates
+// 1.64 / 1.59 / 1.57 / 1.57; 64 replicas, 60 candidates 1.25 / 1.20 / 1.19 / 1.19; 16 replicas 0.79 / 0.78 / 0.78 / 0.78, four an
+// SM 1.46 / 1.46 / 1.47 / 1.47; shared prompts 0.81 / 0.81 / 0.82 / 0.82, four an SM 1.38 / 1.35 / 1.34 / 1.35.
+constexpr uint32_t kRefill = 3;
 // Requests after which a replica whose order ran out is looked at again.  1 / 4 / 16, a cache of one long prompt:
 // 1 replica 1.00 / 1.18 / 1.51, 2 replicas 0.93 / 0.96 / 1.35, 16 replicas 0.99 / 0.95 / 0.95, 64 replicas 1.32 / 1.27 /
 // 1.23; larger caches run out of nothing.
@@ -1410,7 +1417,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (i < R && (want == i + 1u || (ahead && (uint64_t)*(volatile uint32_t*)&sh.occ[i] + kMargin >= a.m.C))) {
         const uint32_t fill = sh.ring_tail[i] - *(volatile uint32_t*)&sh.take[i].x;
         const uint32_t news = seen - (half ? dry1 : dry0);
-        if (fill * 2u <= a.ring_cap && (news >= kNews || (news && want == i + 1u))) best = min(best, (want == i + 1u ? 0u : 1u << 16) | (fill << 8) | i);
+        if (fill * 4u <= a.ring_cap * kRefill && (news >= kNews || (news && want == i + 1u))) best = min(best, (want == i + 1u ? 0u : 1u << 16) | (fill << 8) | i);
       }
     }
     best = __reduce_min_sync(kFull, best);
