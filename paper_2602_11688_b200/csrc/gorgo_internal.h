@@ -108,6 +108,7 @@ struct ReplayArgs {
   uint32_t probe_off, scout_off;  // test switches: no mask words read ahead / no victims listed ahead
   uint32_t slots_in_smem;         // set by the launcher: per-slot state fits in shared memory
   uint32_t ring_cap;              // set by the launcher: listed victims kept per replica (a power of two)
+  uint32_t roles;                 // set by the launcher: role of each warp, four bits each
   const double* params;           // [P*K] device, or null: `inline_params` (one candidate)
   double inline_params[67];
   unsigned char* masks;           // [P * mask_stride] bytes: cached-on-replica words, one per atom

@@ -672,7 +672,12 @@ __device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* r
 // lists them, one entry per lane; waits for the scout where its list is too short.  Returns the
 // requests that are dirty now (see route_warp).  (Out of line: the route warp handles the usual case
 // itself.)
-template <typename MaskT, bool kExt>
+//   The list usually holds more than the commit takes.  The entries behind the first that is enough if all before it are
+// victims are left for another round of the loop: the walks of 32 lanes over later occurrences take as long as the
+// longest.  (One candidate an SM, half-full lists against full ones: 16 replicas, 639 blocks a cache 1.69 -> 1.49 us per request,
+// 64 replicas 1.35 -> 1.31.  Not in the dense build, whose loops are larger than the instruction cache: the few
+// instructions cost three and four candidates an SM 4 to 5 %.)
+template <typename MaskT, bool kExt, bool kDense>
 __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, kExt>& sh, MaskT* mask,
                                             const uint8_t* route_log, const uint4* more, uint32_t rep, uint32_t r, uint32_t need) {
   using Sh = Shared<MaskT, kExt>;
@@ -697,8 +702,12 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     const uint32_t e = rep * a.ring_cap + ((head + lane) & cap_mask);
     const uint2 v = lds64(sb + (uint32_t)offsetof(Sh, victims) + e * 8u);
     const uint32_t next_req = lds32(sb + (uint32_t)offsetof(Sh, victim_next) + e * 4u);
-    const bool listed = lane < avail;
     const uint32_t upto = v.y - cons;               // blocks gone with this entry
+    if (!kDense) {
+      const uint32_t most = __ballot_sync(kFull, lane < avail && upto >= need);
+      if (most) avail = min(avail, (uint32_t)__ffs((int)most));
+    }
+    const bool listed = lane < avail;
     bool live = listed;
     uint32_t d = 0;
     if (listed && next_req < r + kStages) {         // it occurred again since it was listed, or will soon
@@ -708,10 +717,12 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     dirty |= __reduce_or_sync(kFull, d);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
     uint32_t dead = listed && !live ? upto - (lane ? prev : 0u) : 0u;   // blocks that are no victims
-    #pragma unroll 1
-    for (uint32_t w = 1; w < 32u; w <<= 1) {
-      const uint32_t below = __shfl_up_sync(kFull, dead, w);
-      if (lane >= w) dead += below;
+    if (kDense || __any_sync(kFull, dead != 0u)) {
+      #pragma unroll 1
+      for (uint32_t w = 1; w < 32u; w <<= 1) {
+        const uint32_t below = __shfl_up_sync(kFull, dead, w);
+        if (lane >= w) dead += below;
+      }
     }
     const uint32_t freed = upto - dead;             // blocks that are freed up to this entry
     const uint32_t enough = __ballot_sync(kFull, live && freed >= need);
@@ -778,7 +789,7 @@ __device__ __noinline__ uint32_t commit_slow(const ReplayArgs& a, Shared<MaskT, 
 // reductions interleaved, before it is known whether q is ready and its stage up to date; if not
 // (about 1.5 requests in 100), q is decided once more with nothing to commit.  Everything unusual is out of line
 // behind one vote.  (Commit after score: 0.85 us per request at one candidate per SM; side by side 0.73.)
-template <typename MaskT, bool kExt>
+template <typename MaskT, bool kExt, bool kDense>
 __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, uint32_t sb, const Dyn& dy,
                                            const StageArgs<MaskT>& sa, const uint8_t* route_log, const uint4* more, const RepState* rep,
                                            uint32_t p, uint32_t lane) {
@@ -888,7 +899,7 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
       }
       if (need != 0u && (again || enough == 0u || __any_sync(kFull, soon))) {
         PROF_ADD(9, 1);
-        dirty |= evict_slow<MaskT, kExt>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
+        dirty |= evict_slow<MaskT, kExt, kDense>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
         if (kExt) st_evict += need;
         need = 0u;
         held = C;
@@ -1349,8 +1360,9 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
 //   Usually a few lanes ask and twenty or thirty requests are asked, so the requests go by lane and the askers one
 // after the other (kAsk of them with their loads in flight together): one memory latency per asker.  (The askers by lane
 // and the requests one after the other, four at a time: shared prompts, 8 replicas, 64 candidates 0.81 us per request,
-// with this 0.78.  More than one asker in flight is no faster there, and its code in the scout's loop costs four candidates an SM
-// 2 % (two) to 5 % (four); with more than 32 replicas, where the function is called, 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
+// with this 0.78.  In the dense build the code of more than one asker in flight, inside the scout's loop, costs four
+// candidates an SM 2 % (two) to 5 % (four); with more than 32 replicas, where it is called there, and with up to two
+// candidates an SM four are in flight: with 64 replicas 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
 template <uint32_t kAsk>
 __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
                                               uint32_t m, uint32_t n) {
@@ -1391,7 +1403,7 @@ __device__ __noinline__ bool touched_again_called(const Touch* touch, uint32_t a
 // (the requests of the route log with that replica, deepest touch first) from where it stopped, up to
 // 32 touches per round, one per lane, and appends those that are still the latest touch of their
 // atom.  The route warp checks again what occurs between the listing and the eviction.
-template <typename MaskT, bool kExt>
+template <typename MaskT, bool kExt, bool kDense>
 __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const Cand<MaskT>& cd, uint4* more,
                                            uint32_t lane) {
   const uint32_t R = a.m.R, end = a.first + a.count;
@@ -1550,8 +1562,10 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (!rest) break;
       if (hop >= kHops) {
         if (hop == kHops && n_match) {
-          if (sizeof(MaskT) == 8 ? touched_again_called(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)
-                                 : touched_again<1>(touch, open ? t.atom : kNone, my_q, my_k, rq, off, m, n_match)) live = open = false;
+          const uint32_t asked = open ? t.atom : kNone;
+          if (!kDense ? touched_again<4>(touch, asked, my_q, my_k, rq, off, m, n_match)
+              : sizeof(MaskT) == 8 ? touched_again_called(touch, asked, my_q, my_k, rq, off, m, n_match)
+                                   : touched_again<1>(touch, asked, my_q, my_k, rq, off, m, n_match)) live = open = false;
           rest = __ballot_sync(kFull, open);
           if (!rest) break;
         }
@@ -1603,8 +1617,18 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
 
 enum Role : uint32_t { kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScout, kRoleFile, kRoles };
 constexpr uint32_t kReplayThreads = 32 * kRoles;
-// Register cap: four candidates share an SM (80 registers a thread), three with more than 32 replicas.
-template <typename MaskT> constexpr int kReplayMinCtas = sizeof(MaskT) == 8 ? 3 : 4;
+// The dense build's register cap: four candidates share an SM (80 registers a thread), three with more than 32 replicas.
+// The other build is for launches of at most two candidates an SM, where a replay is bound by its chain and not by
+// instruction fetch: registers without spills, and code that only pays there.
+template <typename MaskT, bool kDense> constexpr int kReplayMinCtas = !kDense ? 2 : sizeof(MaskT) == 8 ? 3 : 4;
+// Roles by warp, four bits each.  The hardware gives an SM's four schedulers a block's warps in turn, so the third and
+// fourth of six have a scheduler alone.  With one candidate an SM the route warp is the third: 2 to 3 % faster
+// than next to the scout.  With a second candidate all schedulers hold three warps, and the other order is 6 % faster.
+constexpr uint32_t role_order(Role w0, Role w1, Role w2, Role w3, Role w4, Role w5) {
+  return w0 | w1 << 4 | w2 << 8 | w3 << 12 | w4 << 16 | w5 << 20;
+}
+constexpr uint32_t kOrderAlone = role_order(kRoleScout, kRoleStage, kRoleRoute, kRoleExpiry, kRoleTime, kRoleFile);
+constexpr uint32_t kOrderShared = role_order(kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScout, kRoleFile);
 
 // The lists of the launch before (the end of the kernel says why).  (Out of line: inlined it costs the
 // loops registers.)
@@ -1627,11 +1651,12 @@ __device__ __noinline__ void lists_in(const ReplayArgs& a, Shared<MaskT, kExt>& 
   }
 }
 
-template <typename MaskT, bool kExt>
-__global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_kernel(const __grid_constant__ ReplayArgs a) {
+template <typename MaskT, bool kExt, bool kDense>
+__global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kDense>)) replay_kernel(const __grid_constant__ ReplayArgs a) {
   const uint32_t p = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warp = __shfl_sync(kFull, threadIdx.x >> 5, 0);   // (known to be the same for all lanes)
+  const uint32_t w_id = __shfl_sync(kFull, threadIdx.x >> 5, 0);   // (known to be the same for all lanes)
+  const uint32_t warp = kDense ? w_id : a.roles >> (4u * w_id) & 15u;
   const uint32_t R = a.m.R, K = a.m.K, GR = a.m.G * a.m.R, RS = a.m.R * a.m.S;
   const uint32_t N = a.tr.n_req;
 
@@ -1753,12 +1778,12 @@ __global__ void __launch_bounds__(kReplayThreads, kReplayMinCtas<MaskT>) replay_
   const uint32_t sb = smem_addr(smem_raw);
   const StageArgs<MaskT> sa = {cd.mask, cd.index, cd.scale};
   uint4* more = sizeof(MaskT) == 8 ? reinterpret_cast<uint4*>(st + a.lay.more_off) : sh.victim_more;
-  if (warp == kRoleRoute) route_warp<MaskT, kExt>(a, sh, sb, dy, sa, cd.route_log, more, cd.rep, p, lane);
+  if (warp == kRoleRoute) route_warp<MaskT, kExt, kDense>(a, sh, sb, dy, sa, cd.route_log, more, cd.rep, p, lane);
   else if (warp == kRoleStage) stage_warp<MaskT, kExt>(a, sh, sb, sa, lane);
   else if (warp == kRoleTime) time_warp<MaskT, kExt>(a, sh, sb, dy, cd.slot_kv, cd.scale, lane);
   else if (warp == kRoleExpiry) expiry_warp<MaskT, kExt>(a, sh, sb, cd.exp_rec, cd.scale, lane);
   else if (warp == kRoleFile) file_warp<MaskT, kExt>(a, sh, cd, p, lane);
-  else scout_warp<MaskT, kExt>(a, sh, cd, more, lane);
+  else scout_warp<MaskT, kExt, kDense>(a, sh, cd, more, lane);
   __syncthreads();
 
   // (pointers computed again: registers less in the loops)
@@ -1822,30 +1847,44 @@ size_t replay_smem_bytes(ReplayArgs& a) {
   return shared_bytes<MaskT, kExt>(a.m, a.tr.chunk_req, a.tr.chunk_cap, a.slots_in_smem != 0);
 }
 
-template <typename MaskT, bool kExt>
+template <typename MaskT, bool kExt, bool kDense>
 cudaError_t prepare_replay(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(replay_kernel<MaskT, kExt>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // several candidates share an SM: the per-CTA footprint, not the default carve-out, decides
-  return cudaFuncSetAttribute(replay_kernel<MaskT, kExt>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kDense>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared);
 }
 
-template <typename MaskT, bool kExt>
+template <typename MaskT, bool kExt, bool kDense>
 cudaError_t launch_replay_t(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
   const size_t smem = replay_smem_bytes<MaskT, kExt>(a);
-  cudaError_t e = prepare_replay<MaskT, kExt>(smem);
+  cudaError_t e = prepare_replay<MaskT, kExt, kDense>(smem);
   if (e != cudaSuccess) return e;
-  replay_kernel<MaskT, kExt><<<n_cand, kReplayThreads, smem, st>>>(a);
+  replay_kernel<MaskT, kExt, kDense><<<n_cand, kReplayThreads, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+// Up to two candidates an SM take the build without a register cap.  (us per request, this build against the dense
+// one: 16 replicas, one an SM 0.73 and 0.78, two 0.82 and 0.85; with its registers only two fit an SM, so three would take
+// two waves: 1.6 and 1.2.)  The second candidate comes to an SM when every SM has one.
+template <typename MaskT, bool kExt>
+cudaError_t launch_replay_n(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  a.roles = n_cand <= (uint32_t)sms ? kOrderAlone : kOrderShared;
+  return n_cand <= 2u * (uint32_t)sms ? launch_replay_t<MaskT, kExt, false>(a, n_cand, st)
+                                      : launch_replay_t<MaskT, kExt, true>(a, n_cand, st);
 }
 
 template <typename MaskT>
 int replay_occupancy_t(ReplayArgs& a, size_t* smem_out) {
   *smem_out = replay_smem_bytes<MaskT, false>(a);
   int n = 0;
-  if (prepare_replay<MaskT, false>(*smem_out) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false>, (int)kReplayThreads,
+  if (prepare_replay<MaskT, false, true>(*smem_out) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false, true>, (int)kReplayThreads,
                                                     *smem_out) != cudaSuccess) {
     cudaGetLastError();
     return -1;
@@ -1871,9 +1910,9 @@ cudaError_t launch_replay(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st)
   // the plain cost-model replay carries none of the optional model parts
   const bool ext = a.queue_in_requests || a.forced_route || a.rep_prefill_ms || a.rep_tpot_ms ||
                    a.decode_slowdown > 0.0 || a.kv_budget > 0 || a.rtt_ewma || a.proxy_index || a.stats;
-  if (a.m.R <= 32) return ext ? launch_replay_t<uint32_t, true>(a, n_cand, st) : launch_replay_t<uint32_t, false>(a, n_cand, st);
-  return ext ? launch_replay_t<unsigned long long, true>(a, n_cand, st)
-             : launch_replay_t<unsigned long long, false>(a, n_cand, st);
+  if (a.m.R <= 32) return ext ? launch_replay_n<uint32_t, true>(a, n_cand, st) : launch_replay_n<uint32_t, false>(a, n_cand, st);
+  return ext ? launch_replay_n<unsigned long long, true>(a, n_cand, st)
+             : launch_replay_n<unsigned long long, false>(a, n_cand, st);
 }
 
 #ifdef GORGO_PROF

@@ -1,0 +1,43 @@
+"""GPU parity at the edges of the rule that picks the replay kernel's build: up to one candidate an SM, up
+to two, more.  Traces that make the rare paths of the eviction common: a prompt that many share, caches of a few
+prompts, victims that occur again between their listing and their eviction."""
+import numpy as np
+import pytest
+
+from paper_2602_11688_b200 import workloads as W
+from tests.util import assert_candidate_matches, gpu_eval, oracle_eval, small_trace
+
+pytestmark = pytest.mark.gpu
+
+
+def _sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def shared_prompt_trace(seed, n_req, B=512):
+    """Sessions that all begin with one of two prompts of two blocks."""
+    reqs = []
+    for t, in_tok, out, ids in small_trace(seed, n_req=n_req, n_sessions=20, max_blocks=9):
+        reqs.append((t, in_tok + 2 * B, out, ([1, 2] if ids[0] % 3 else [3, 4]) + list(ids)))
+    return reqs
+
+
+@pytest.mark.parametrize("per_sm,extra", [(0, 3), (1, 0), (1, 1), (2, 0), (2, 1), (4, 5)])
+@pytest.mark.parametrize("R,C,stats", [(2, 24, False), (8, 17, True), (32, 40, False), (33, 13, True), (64, 30, False)])
+def test_every_build_matches_the_oracle(per_sm, extra, R, C, stats):
+    rng = np.random.default_rng(R)
+    base = rng.normal(1.0, 0.3, size=(3, 3))
+    base[0] = (0.0, 1.0, 0.0)                         # follow the cache
+    base[1] = (0.0, 0.0, 1.0)                         # spread out: evictions everywhere
+    w = W.handmade(rng.uniform(5, 60, size=R), shared_prompt_trace(R, 400), slots=2, cache_blocks=C, params=base)
+    P = per_sm * _sms() + extra
+    params = np.tile(base, (P // 3 + 1, 1))[:P]
+    gpu = gpu_eval(w, params, 1.0, stats=stats)
+    refs = oracle_eval(w, base, 1.0)
+    for p in sorted({0, 1, 2, P - 3, P - 2, P - 1}):
+        assert_candidate_matches(gpu, p, refs[p % 3])
+    for key in ("route", "hit", "p95_ttft", "p95_e2e"):   # equal weights, equal results
+        for k in range(3):
+            assert (gpu[key][k::3] == gpu[key][k]).all(), (key, k)
+    assert sum(int(r[4][3]) for r in refs) > 0        # evictions happened
