@@ -91,6 +91,13 @@ constexpr uint32_t kNews = 4;
 // four to eight within 5 % either way; at 16 the lists win, 91 and 84.  Launches of an uploaded trace that follow one
 // another without a wait would take them from two requests on: 8 requests 26.5 and 21.8 us.
 constexpr uint32_t kFew = 8;
+// Sleeps of the waits, of the idle file and scout warps.  With three and four candidates an SM instruction fetch is what
+// the warps share, and polls take part of it.  Waits 20, file and scout 100 / 40 and 500 / 100 and 300 ns: 16 replicas
+// three an SM 1.171 / 1.156 / 1.157 us per request, four 1.453 / 1.429 / 1.429; 32 replicas, 480 candidates 1.563 / 1.545 / 1.544; 64
+// replicas, 400 candidates 1.938 / 1.924 / 1.925.  One candidate an SM: no difference, but a launch of one request ends when
+// the file warp has seen it, so there that sleep stays short.
+constexpr uint32_t kWaitNs = 40;
+template <bool kDense> constexpr uint32_t kIdleNs = kDense ? 500 : 100;
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round: one per lane
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
@@ -250,7 +257,7 @@ __device__ __noinline__ uint32_t wait_slow(uint32_t p, uint32_t want, uint32_t s
     for (uint32_t polls = 0; (int32_t)(v - want) < 0; ++polls) {
       if (lds32(sb + offsetof(Control, abort_flag))) break;
       if (polls >= limit) { at_limit(sb); polls = 0; }
-      if (polls > 4) __nanosleep(20);
+      if (polls > 4) __nanosleep(kWaitNs);
       v = lds32(p);
     }
   }
@@ -1230,7 +1237,7 @@ __device__ __forceinline__ void expiry_warp(const ReplayArgs& a, Shared<MaskT, k
 // (found through the time grid over the arrivals, then a short scan), and the hand-over of finished
 // lists to the expiry warp.  The list of request r gains entries only from requests <= r - kNear, so
 // it is final once the file warp has passed r - kNear.
-template <typename MaskT, bool kExt>
+template <typename MaskT, bool kExt, bool kDense>
 __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const Cand<MaskT>& cd, uint32_t p,
                                           uint32_t lane) {
   const uint32_t end = a.first + a.count, N = a.tr.n_req;
@@ -1349,7 +1356,7 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
       if (__any_sync(kFull, sh.c.abort_flag != 0)) break;
       // (whom it waits for is at work or in a wait of its own; 2^31 rounds are longer than any walk)
       if (++idle >> 31) break;
-      __nanosleep(100);
+      __nanosleep(kIdleNs<kDense>);
     }
   }
   PROF_END(48);
@@ -1438,7 +1445,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       // fills, and it ends this warp when it ends.  (The route warp's own limit reports the failure.)
       idle += want != 0 ? 1u : 0u;
       if (idle > a.poll_limit) break;
-      __nanosleep(100);
+      __nanosleep(kIdleNs<kDense>);
       continue;
     }
     idle = 0;
@@ -1782,7 +1789,7 @@ __global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kDense>
   else if (warp == kRoleStage) stage_warp<MaskT, kExt>(a, sh, sb, sa, lane);
   else if (warp == kRoleTime) time_warp<MaskT, kExt>(a, sh, sb, dy, cd.slot_kv, cd.scale, lane);
   else if (warp == kRoleExpiry) expiry_warp<MaskT, kExt>(a, sh, sb, cd.exp_rec, cd.scale, lane);
-  else if (warp == kRoleFile) file_warp<MaskT, kExt>(a, sh, cd, p, lane);
+  else if (warp == kRoleFile) file_warp<MaskT, kExt, kDense>(a, sh, cd, p, lane);
   else scout_warp<MaskT, kExt, kDense>(a, sh, cd, more, lane);
   __syncthreads();
 
