@@ -41,3 +41,29 @@ def test_every_build_matches_the_oracle(per_sm, extra, R, C, stats):
         for k in range(3):
             assert (gpu[key][k::3] == gpu[key][k]).all(), (key, k)
     assert sum(int(r[4][3]) for r in refs) > 0        # evictions happened
+
+
+@pytest.mark.parametrize("lam,steps,resident", [(1, 2, 1), (5, 3, 1), (5, 3, 5), (5, 3, 6), (4, 0, 4)])
+def test_the_parent_is_evaluated_with_the_first_offspring(lam, steps, resident):
+    """Workspaces that hold the first population and the parent, the population alone, or one candidate."""
+    from oracle import gorgo_oracle as O
+    from oracle import gorgo_tuning as T
+    from paper_2602_11688_b200 import binding as gb
+    rng = np.random.default_rng(lam)
+    w = W.handmade(rng.uniform(5, 60, size=4), small_trace(3, n_req=300), slots=2, cache_blocks=15,
+                   params=[(0.5, 1.0, 0.1)])
+    z = rng.standard_normal((steps, lam, 2))
+    es = dict(tuned=np.array([0, 2], np.uint32), lo=np.array([0.05, 0.05]), hi=np.array([2.0, 0.5]))
+    sim = gb.GorgoSim(w)
+    try:
+        sim.ensure_workspace(resident)
+        rc, x, f, sigma, hist = gb.gorgo_es_run(sim.h, x0=w.params[0], z=z, sigma0=0.5, sigma_up=1.5, n_steps=steps, lam=lam,
+                                                workspace=sim.workspace, stream=sim.stream, time_scale=1.0, **es)
+        assert rc == gb.GORGO_OK
+    finally:
+        sim.close()
+    rx, rf, rsigma, rhist = T.es_run(lambda v: O.replay(w, np.array(v), 1.0)[1], w.params[0].tolist(), es["tuned"].tolist(),
+                                     es["lo"].tolist(), es["hi"].tolist(), 0.5, 1.5, z.tolist())
+    assert x.tolist() == rx and f == rf and sigma == rsigma
+    for t, h in enumerate(rhist):
+        assert hist[t, 0] == h[0] and bool(hist[t, 1]) == h[1] and hist[t, 3] == h[3], t
