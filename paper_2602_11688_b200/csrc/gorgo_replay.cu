@@ -30,7 +30,9 @@
 // this split gives 0.73, 0.84, 1.09 and 1.32 at one to four (long-context trace, 16 replicas, 20,000 requests,
 // 4,000 blocks a cache; the twelve-warp kernel on blocks before it 1.09, 1.39, 2.65 and 2.77).  The loops are
 // still over the cache: with three or four candidates an SM 128 bytes more in one of them cost about 3 %,
-// so what is rare is out of line, and loops that could share a body do.
+// so what is rare is out of line, and loops that could share a body do.  Two builds share this source (kDense): up to two
+// candidates an SM, and more; on another trace of 15,000 and 20,000 requests 0.79, 0.84, 1.20 and 1.46 us at one to four an SM
+// with one build, 0.73, 0.83, 1.16 and 1.43 with two.
 #include "gorgo_device.cuh"
 
 namespace gorgo {
