@@ -426,12 +426,17 @@ int gorgo_measure_gather(int device, void *buffer, uint64_t buffer_bytes, uint64
  *   GORGO_DEBUG_PROBE_OFF   nonzero: requests are not staged several at once from words read ahead;
  *                           each is staged alone (results do not depend on it).
  *   GORGO_DEBUG_SCOUT_OFF   nonzero: victims are listed only when a commit asks for one (results do
- *                           not depend on it). */
+ *                           not depend on it).
+ *   GORGO_DEBUG_BUILD       build of the replay kernel: 0 (default) chosen by the candidates of each
+ *                           launch, 1 the one for up to two candidates an SM, 2 the one for more
+ *                           (results do not depend on it).  gorgo_replay_occupancy then reports that
+ *                           build. */
 enum {
   GORGO_DEBUG_POLL_LIMIT = 0,
   GORGO_DEBUG_RING_POLLS = 1,
   GORGO_DEBUG_PROBE_OFF = 2,
-  GORGO_DEBUG_SCOUT_OFF = 3
+  GORGO_DEBUG_SCOUT_OFF = 3,
+  GORGO_DEBUG_BUILD = 4
 };
 int gorgo_debug_set(gorgo_sim_t *sim, uint32_t what, uint32_t value);
 

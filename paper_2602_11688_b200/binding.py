@@ -39,6 +39,7 @@ EXPORTS = [
     "gorgo_trace_begin", "gorgo_trace_append",
 ]
 GORGO_DEBUG_POLL_LIMIT, GORGO_DEBUG_RING_POLLS, GORGO_DEBUG_PROBE_OFF, GORGO_DEBUG_SCOUT_OFF = 0, 1, 2, 3
+GORGO_DEBUG_BUILD = 4
 
 
 class gorgo_config_t(C.Structure):

@@ -123,7 +123,7 @@ struct gorgo_sim {
   bool has_trace = false;
   TraceView tr = {};
   uint32_t poll_limit = 1u << 24;   // bound of the device-side waits of one warp for another
-  uint32_t probe_off = 0, scout_off = 0;   // test switches (gorgo_debug_set)
+  uint32_t probe_off = 0, scout_off = 0, build = 0;   // test switches (gorgo_debug_set)
   // optional CUDA-event timing of the replay kernel (one pair per wave of the last evaluation)
   bool profiling = false;
   std::vector<cudaEvent_t> ev;    // pairs around the replay launches
@@ -234,7 +234,7 @@ ReplayArgs base_args(const gorgo_sim* sim, unsigned char* base, const WsLayout& 
   // all slots: S * S / 8 reads behind one wait of another warp, a poll each two at most.
   const uint64_t rounds = sim->kv_budget ? (uint64_t)sim->m.S * sim->m.S / 4 : 0;
   a.poll_limit = (uint32_t)std::min<uint64_t>(sim->poll_limit + rounds, 0xFFFFFFFFu);
-  a.probe_off = sim->probe_off; a.scout_off = sim->scout_off;
+  a.probe_off = sim->probe_off; a.scout_off = sim->scout_off; a.build = sim->build;
   a.masks = base + w.masks; a.mask_stride = w.mask_stride; a.index_off = w.index_off;
   a.states = base + w.states; a.lay = w.st;
   a.exp_head = reinterpret_cast<uint32_t*>(base + w.exp_head);
@@ -1356,7 +1356,7 @@ int gorgo_replay_occupancy(gorgo_sim_t* sim, int32_t* ctas_per_sm, uint64_t* sme
   if (!sim || !ctas_per_sm) return GORGO_ERR_INVALID_ARG;
   DeviceGuard guard(sim->device);
   if (!guard.ok) return GORGO_ERR_CUDA;
-  const int n = replay_occupancy(sim->m, sim->tr, smem_bytes_per_cta);
+  const int n = replay_occupancy(sim->m, sim->tr, sim->build, smem_bytes_per_cta);
   if (n < 0) return GORGO_ERR_CUDA;
   *ctas_per_sm = n;
   return GORGO_OK;
@@ -1406,6 +1406,10 @@ int gorgo_debug_set(gorgo_sim_t* sim, uint32_t what, uint32_t value) {
     case GORGO_DEBUG_RING_POLLS: break;
     case GORGO_DEBUG_PROBE_OFF: sim->probe_off = value ? 1u : 0u; break;
     case GORGO_DEBUG_SCOUT_OFF: sim->scout_off = value ? 1u : 0u; break;
+    case GORGO_DEBUG_BUILD:
+      if (value > kReplayBuilds) return GORGO_ERR_INVALID_ARG;
+      sim->build = value;
+      break;
     default: return GORGO_ERR_INVALID_ARG;
   }
   return GORGO_OK;

@@ -96,6 +96,9 @@ struct StateLayout {
 // listed long ago has more often been touched again.
 constexpr uint32_t listed_victims(uint32_t n_replicas) { return n_replicas <= 16 ? 32u : 16u; }
 
+// Builds of the replay kernel per mask width, plain or extended.
+constexpr uint32_t kReplayBuilds = 2;
+
 // Everything one replay launch needs.  Candidate p of the launch uses element/byte strides.
 struct ReplayArgs {
   Model m;
@@ -109,6 +112,7 @@ struct ReplayArgs {
   uint32_t slots_in_smem;         // set by the launcher: per-slot state fits in shared memory
   uint32_t ring_cap;              // set by the launcher: listed victims kept per replica (a power of two)
   uint32_t roles;                 // set by the launcher: role of each warp, four bits each
+  uint32_t build;                 // test switch: 0, or the build of the kernel that is launched (1 to kReplayBuilds)
   const double* params;           // [P*K] device, or null: `inline_params` (one candidate)
   double inline_params[67];
   unsigned char* masks;           // [P * mask_stride] bytes: cached-on-replica words, one per atom
@@ -220,7 +224,7 @@ cudaError_t launch_gather(const void* buf, uint64_t n_sectors, uint32_t per_thre
 uint32_t window_max();          // largest window the window kernel handles
 uint32_t mask_bytes_for(uint32_t n_replicas);
 // CTAs of the replay kernel that fit one SM for this model (-1: query failed), and the dynamic
-// shared memory one CTA asks for.
-int replay_occupancy(const Model& m, const TraceView& tr, uint64_t* smem_bytes);
+// shared memory one CTA asks for.  `build` as in ReplayArgs; 0: the one for many candidates.
+int replay_occupancy(const Model& m, const TraceView& tr, uint32_t build, uint64_t* smem_bytes);
 
 }  // namespace gorgo

@@ -1884,16 +1884,16 @@ cudaError_t launch_replay_n(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   a.roles = n_cand <= (uint32_t)sms ? kOrderAlone : kOrderShared;
-  return n_cand <= 2u * (uint32_t)sms ? launch_replay_t<MaskT, kExt, false>(a, n_cand, st)
-                                      : launch_replay_t<MaskT, kExt, true>(a, n_cand, st);
+  const bool dense = a.build ? a.build == 2u : n_cand > 2u * (uint32_t)sms;
+  return dense ? launch_replay_t<MaskT, kExt, true>(a, n_cand, st) : launch_replay_t<MaskT, kExt, false>(a, n_cand, st);
 }
 
-template <typename MaskT>
+template <typename MaskT, bool kDense>
 int replay_occupancy_t(ReplayArgs& a, size_t* smem_out) {
   *smem_out = replay_smem_bytes<MaskT, false>(a);
   int n = 0;
-  if (prepare_replay<MaskT, false, true>(*smem_out) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false, true>, (int)kReplayThreads,
+  if (prepare_replay<MaskT, false, kDense>(*smem_out) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false, kDense>, (int)kReplayThreads,
                                                     *smem_out) != cudaSuccess) {
     cudaGetLastError();
     return -1;
@@ -1903,12 +1903,14 @@ int replay_occupancy_t(ReplayArgs& a, size_t* smem_out) {
 
 }  // namespace
 
-int replay_occupancy(const Model& m, const TraceView& tr, uint64_t* smem_bytes) {
+int replay_occupancy(const Model& m, const TraceView& tr, uint32_t build, uint64_t* smem_bytes) {
   ReplayArgs a = {};
   a.m = m;
   a.tr = tr;
   size_t smem = 0;
-  const int n = m.R <= 32 ? replay_occupancy_t<uint32_t>(a, &smem) : replay_occupancy_t<unsigned long long>(a, &smem);
+  const int n = m.R <= 32 ? (build == 1 ? replay_occupancy_t<uint32_t, false>(a, &smem) : replay_occupancy_t<uint32_t, true>(a, &smem))
+                : build == 1 ? replay_occupancy_t<unsigned long long, false>(a, &smem)
+                             : replay_occupancy_t<unsigned long long, true>(a, &smem);
   if (smem_bytes) *smem_bytes = smem;
   return n;
 }
