@@ -1369,9 +1369,9 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
 //   Usually a few lanes ask and twenty or thirty requests are asked, so the requests go by lane and the askers one
 // after the other (kAsk of them with their loads in flight together): one memory latency per asker.  (The askers by lane
 // and the requests one after the other, four at a time: shared prompts, 8 replicas, 64 candidates 0.81 us per request,
-// with this 0.78.  In the dense build the code of more than one asker in flight, inside the scout's loop, costs four
-// candidates an SM 2 % (two) to 5 % (four); with more than 32 replicas, where it is called there, and with up to two
-// candidates an SM four are in flight: with 64 replicas 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
+// with this 0.78.  Inlined, one asker is in flight: the code of four inside the scout's loop costs four candidates an
+// SM 5 %, two 1 to 3 % and with 64 replicas 7 to 9 % (1.79 -> 1.95 us), and gains 1 % with one candidate an SM and
+// shared prompts.  With more than 32 replicas it is called, with four: 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
 template <uint32_t kAsk>
 __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
                                               uint32_t m, uint32_t n) {
@@ -1572,9 +1572,8 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       if (hop >= kHops) {
         if (hop == kHops && n_match) {
           const uint32_t asked = open ? t.atom : kNone;
-          if (!kDense ? touched_again<4>(touch, asked, my_q, my_k, rq, off, m, n_match)
-              : sizeof(MaskT) == 8 ? touched_again_called(touch, asked, my_q, my_k, rq, off, m, n_match)
-                                   : touched_again<1>(touch, asked, my_q, my_k, rq, off, m, n_match)) live = open = false;
+          if (sizeof(MaskT) == 8 ? touched_again_called(touch, asked, my_q, my_k, rq, off, m, n_match)
+                                : touched_again<1>(touch, asked, my_q, my_k, rq, off, m, n_match)) live = open = false;
           rest = __ballot_sync(kFull, open);
           if (!rest) break;
         }
