@@ -388,7 +388,9 @@ int gorgo_tune_online(gorgo_sim_t *sim, const gorgo_online_config_t *cfg, uint32
 
 /* Measurement aid (no counterpart in the paper): how many candidates (CTAs of the replay kernel)
  * one SM holds at once for this configuration, and the shared memory each takes.  A population
- * larger than SMs x that number is replayed in successive rounds of CTAs. */
+ * larger than SMs x that number is replayed in successive rounds of CTAs.  (The number is the same for
+ * every launch of more than a quarter as many candidates as the GPU has SMs; smaller launches take a
+ * build of which an SM may hold one less.) */
 int gorgo_replay_occupancy(gorgo_sim_t *sim, int32_t *ctas_per_sm, uint64_t *smem_bytes_per_cta);
 /* Measurement aid (no counterpart in the paper).  With profiling enabled, gorgo_eval_population
  * records a CUDA event on `cuda_stream` directly before and after each launch of the replay
@@ -428,9 +430,9 @@ int gorgo_measure_gather(int device, void *buffer, uint64_t buffer_bytes, uint64
  *   GORGO_DEBUG_SCOUT_OFF   nonzero: victims are listed only when a commit asks for one (results do
  *                           not depend on it).
  *   GORGO_DEBUG_BUILD       build of the replay kernel: 0 (default) chosen by the candidates of each
- *                           launch, 1 the one for up to two candidates an SM, 2 the one for more
- *                           (results do not depend on it).  gorgo_replay_occupancy then reports that
- *                           build. */
+ *                           launch, 1 the one for at most a quarter as many candidates as the GPU has
+ *                           SMs, 2 the one for up to two an SM, 3 the one for more (results do not
+ *                           depend on it).  gorgo_replay_occupancy then reports that build. */
 enum {
   GORGO_DEBUG_POLL_LIMIT = 0,
   GORGO_DEBUG_RING_POLLS = 1,

@@ -97,7 +97,7 @@ struct StateLayout {
 constexpr uint32_t listed_victims(uint32_t n_replicas) { return n_replicas <= 16 ? 32u : 16u; }
 
 // Builds of the replay kernel per mask width, plain or extended.
-constexpr uint32_t kReplayBuilds = 2;
+constexpr uint32_t kReplayBuilds = 3;
 
 // Everything one replay launch needs.  Candidate p of the launch uses element/byte strides.
 struct ReplayArgs {
@@ -111,7 +111,6 @@ struct ReplayArgs {
   uint32_t probe_off, scout_off;  // test switches: no mask words read ahead / no victims listed ahead
   uint32_t slots_in_smem;         // set by the launcher: per-slot state fits in shared memory
   uint32_t ring_cap;              // set by the launcher: listed victims kept per replica (a power of two)
-  uint32_t roles;                 // set by the launcher: role of each warp, four bits each
   uint32_t build;                 // test switch: 0, or the build of the kernel that is launched (1 to kReplayBuilds)
   const double* params;           // [P*K] device, or null: `inline_params` (one candidate)
   double inline_params[67];

@@ -30,9 +30,11 @@
 // this split gives 0.73, 0.84, 1.09 and 1.32 at one to four (long-context trace, 16 replicas, 20,000 requests,
 // 4,000 blocks a cache; the twelve-warp kernel on blocks before it 1.09, 1.39, 2.65 and 2.77).  The loops are
 // still over the cache: with three or four candidates an SM 128 bytes more in one of them cost about 3 %,
-// so what is rare is out of line, and loops that could share a body do.  Two builds share this source (kDense): up to two
-// candidates an SM, and more; on another trace of 15,000 and 20,000 requests 0.79, 0.84, 1.20 and 1.46 us at one to four an SM
-// with one build, 0.73, 0.83, 1.16 and 1.43 with two.
+// so what is rare is out of line, and loops that could share a body do.  Three builds share this source
+// (launch_replay_n says which a launch takes).  16 / 148 / 256 / 444 / 592 candidates, long contexts (8,000 requests, 2,000
+// blocks a cache) with the dense build 0.87 / 0.89 / 0.96 / 1.35 / 1.64 us per request, with the three 0.80 / 0.85 / 0.94 / 1.35 /
+// 1.64; shared prompts 0.76 / 0.80 / 0.85 / 1.05 / 1.22 and 0.74 / 0.79 / 0.85 / 1.05 / 1.22; 64 replicas (6,000
+// requests) 1.32 / 1.51 / 1.68 / 2.36 / 3.91 and 1.29 / 1.43 / 1.62 / 2.36 / 3.91.
 #include "gorgo_device.cuh"
 
 namespace gorgo {
@@ -53,6 +55,9 @@ __device__ unsigned long long g_prof[112];
 #define PROF_ADD(k, v) do {} while (0)
 #define PROF_END(base) do {} while (0)
 #endif
+
+// Builds of the kernel that share this source (launch_replay_n says which a launch takes).
+enum Build : uint32_t { kSparse = 1, kPaired = 2, kDense = 3 };
 
 constexpr uint32_t kStages = 16;      // requests staged ahead of the commits
 constexpr uint32_t kPublish = 8;      // commits are published that many at a time
@@ -99,7 +104,7 @@ constexpr uint32_t kFew = 8;
 // replicas, 400 candidates 1.938 / 1.924 / 1.925.  One candidate an SM: no difference, but a launch of one request ends when
 // the file warp has seen it, so there that sleep stays short.
 constexpr uint32_t kWaitNs = 40;
-template <bool kDense> constexpr uint32_t kIdleNs = kDense ? 500 : 100;
+template <uint32_t kBuild> constexpr uint32_t kIdleNs = kBuild == kSparse ? 100 : 500;
 constexpr uint32_t kMatches = 32;     // requests of a replica looked at per scout round: one per lane
 
 // Counters the warps hand work over with; first in shared memory, so that their addresses do not depend
@@ -684,9 +689,10 @@ __device__ __forceinline__ bool victim_live(const Touch* touch, const uint8_t* r
 //   The list usually holds more than the commit takes.  The entries behind the first that is enough if all before it are
 // victims are left for another round of the loop: the walks of 32 lanes over later occurrences take as long as the
 // longest.  (One candidate an SM, half-full lists against full ones: 16 replicas, 639 blocks a cache 1.69 -> 1.49 us per request,
-// 64 replicas 1.35 -> 1.31.  Not in the dense build, whose loops are larger than the instruction cache: the few
-// instructions cost three and four candidates an SM 4 to 5 %.)
-template <typename MaskT, bool kExt, bool kDense>
+// 64 replicas 1.35 -> 1.31; without the limit and otherwise the same, 148 candidates 0.88 -> 0.85 and, 64 replicas, 1.51 -> 1.43.
+// Not in the dense build: with three and four candidates an SM the loops are larger than the instruction cache, and the
+// few instructions cost 1 to 2 %, 592 candidates with 64 replicas 5 %.)
+template <typename MaskT, bool kExt, uint32_t kBuild>
 __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, kExt>& sh, MaskT* mask,
                                             const uint8_t* route_log, const uint4* more, uint32_t rep, uint32_t r, uint32_t need) {
   using Sh = Shared<MaskT, kExt>;
@@ -712,7 +718,7 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     const uint2 v = lds64(sb + (uint32_t)offsetof(Sh, victims) + e * 8u);
     const uint32_t next_req = lds32(sb + (uint32_t)offsetof(Sh, victim_next) + e * 4u);
     const uint32_t upto = v.y - cons;               // blocks gone with this entry
-    if (!kDense) {
+    if (kBuild != kDense) {
       const uint32_t most = __ballot_sync(kFull, lane < avail && upto >= need);
       if (most) avail = min(avail, (uint32_t)__ffs((int)most));
     }
@@ -726,7 +732,7 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     dirty |= __reduce_or_sync(kFull, d);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
     uint32_t dead = listed && !live ? upto - (lane ? prev : 0u) : 0u;   // blocks that are no victims
-    if (kDense || __any_sync(kFull, dead != 0u)) {
+    if (kBuild == kDense || __any_sync(kFull, dead != 0u)) {
       #pragma unroll 1
       for (uint32_t w = 1; w < 32u; w <<= 1) {
         const uint32_t below = __shfl_up_sync(kFull, dead, w);
@@ -798,7 +804,7 @@ __device__ __noinline__ uint32_t commit_slow(const ReplayArgs& a, Shared<MaskT, 
 // reductions interleaved, before it is known whether q is ready and its stage up to date; if not
 // (about 1.5 requests in 100), q is decided once more with nothing to commit.  Everything unusual is out of line
 // behind one vote.  (Commit after score: 0.85 us per request at one candidate per SM; side by side 0.73.)
-template <typename MaskT, bool kExt, bool kDense>
+template <typename MaskT, bool kExt, uint32_t kBuild>
 __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, uint32_t sb, const Dyn& dy,
                                            const StageArgs<MaskT>& sa, const uint8_t* route_log, const uint4* more, const RepState* rep,
                                            uint32_t p, uint32_t lane) {
@@ -908,7 +914,7 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
       }
       if (need != 0u && (again || enough == 0u || __any_sync(kFull, soon))) {
         PROF_ADD(9, 1);
-        dirty |= evict_slow<MaskT, kExt, kDense>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
+        dirty |= evict_slow<MaskT, kExt, kBuild>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
         if (kExt) st_evict += need;
         need = 0u;
         held = C;
@@ -1239,7 +1245,7 @@ __device__ __forceinline__ void expiry_warp(const ReplayArgs& a, Shared<MaskT, k
 // (found through the time grid over the arrivals, then a short scan), and the hand-over of finished
 // lists to the expiry warp.  The list of request r gains entries only from requests <= r - kNear, so
 // it is final once the file warp has passed r - kNear.
-template <typename MaskT, bool kExt, bool kDense>
+template <typename MaskT, bool kExt, uint32_t kBuild>
 __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const Cand<MaskT>& cd, uint32_t p,
                                           uint32_t lane) {
   const uint32_t end = a.first + a.count, N = a.tr.n_req;
@@ -1358,7 +1364,7 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
       if (__any_sync(kFull, sh.c.abort_flag != 0)) break;
       // (whom it waits for is at work or in a wait of its own; 2^31 rounds are longer than any walk)
       if (++idle >> 31) break;
-      __nanosleep(kIdleNs<kDense>);
+      __nanosleep(kIdleNs<kBuild>);
     }
   }
   PROF_END(48);
@@ -1412,7 +1418,7 @@ __device__ __noinline__ bool touched_again_called(const Touch* touch, uint32_t a
 // (the requests of the route log with that replica, deepest touch first) from where it stopped, up to
 // 32 touches per round, one per lane, and appends those that are still the latest touch of their
 // atom.  The route warp checks again what occurs between the listing and the eviction.
-template <typename MaskT, bool kExt, bool kDense>
+template <typename MaskT, bool kExt, uint32_t kBuild>
 __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kExt>& sh, const Cand<MaskT>& cd, uint4* more,
                                            uint32_t lane) {
   const uint32_t R = a.m.R, end = a.first + a.count;
@@ -1447,7 +1453,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
       // fills, and it ends this warp when it ends.  (The route warp's own limit reports the failure.)
       idle += want != 0 ? 1u : 0u;
       if (idle > a.poll_limit) break;
-      __nanosleep(kIdleNs<kDense>);
+      __nanosleep(kIdleNs<kBuild>);
       continue;
     }
     idle = 0;
@@ -1625,18 +1631,21 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
 
 enum Role : uint32_t { kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScout, kRoleFile, kRoles };
 constexpr uint32_t kReplayThreads = 32 * kRoles;
-// The dense build's register cap: four candidates share an SM (80 registers a thread), three with more than 32 replicas.
-// The other build is for launches of at most two candidates an SM, where a replay is bound by its chain and not by
-// instruction fetch: registers without spills, and code that only pays there.
-template <typename MaskT, bool kDense> constexpr int kReplayMinCtas = !kDense ? 2 : sizeof(MaskT) == 8 ? 3 : 4;
+// Candidates an SM holds, which caps the registers: four (80 registers a thread), three with more than 32 replicas (96).
+// A launch does not see what other streams run on the GPU, so a build that large launches take leaves room for as
+// many: with two an SM (98 registers, no spills; 3 to 6 % faster alone) three populations of 148 on three streams took
+// 1.91 us per request instead of 1.45 (16 replicas), 1.69 instead of 1.14 (shared prompts) and 2.40 instead of 1.75 (32
+// replicas), and two of 256 1.96 instead of 1.62.  The build for few candidates has at most 96 registers.  Three of its
+// blocks fit an SM only if their warps begin on alternate schedulers, as the blocks of one launch do; those of
+// several launches do not always (three streams of 148 took two turns with 96 registers too), but two always fit.
+template <typename MaskT, uint32_t kBuild> constexpr int kReplayMinCtas = kBuild == kSparse || sizeof(MaskT) == 8 ? 3 : 4;
 // Roles by warp, four bits each.  The hardware gives an SM's four schedulers a block's warps in turn, so the third and
 // fourth of six have a scheduler alone.  With one candidate an SM the route warp is the third: 2 to 3 % faster
-// than next to the scout.  With a second candidate all schedulers hold three warps, and the other order is 6 % faster.
+// than next to the scout.  With a second candidate all schedulers hold three warps, and the order of Role is 6 % faster.
 constexpr uint32_t role_order(Role w0, Role w1, Role w2, Role w3, Role w4, Role w5) {
   return w0 | w1 << 4 | w2 << 8 | w3 << 12 | w4 << 16 | w5 << 20;
 }
-constexpr uint32_t kOrderAlone = role_order(kRoleScout, kRoleStage, kRoleRoute, kRoleExpiry, kRoleTime, kRoleFile);
-constexpr uint32_t kOrderShared = role_order(kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScout, kRoleFile);
+constexpr uint32_t kOrderSparse = role_order(kRoleScout, kRoleStage, kRoleRoute, kRoleExpiry, kRoleTime, kRoleFile);
 
 // The lists of the launch before (the end of the kernel says why).  (Out of line: inlined it costs the
 // loops registers.)
@@ -1659,12 +1668,12 @@ __device__ __noinline__ void lists_in(const ReplayArgs& a, Shared<MaskT, kExt>& 
   }
 }
 
-template <typename MaskT, bool kExt, bool kDense>
-__global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kDense>)) replay_kernel(const __grid_constant__ ReplayArgs a) {
+template <typename MaskT, bool kExt, uint32_t kBuild>
+__global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kBuild>)) replay_kernel(const __grid_constant__ ReplayArgs a) {
   const uint32_t p = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t w_id = __shfl_sync(kFull, threadIdx.x >> 5, 0);   // (known to be the same for all lanes)
-  const uint32_t warp = kDense ? w_id : a.roles >> (4u * w_id) & 15u;
+  const uint32_t warp = kBuild == kSparse ? kOrderSparse >> (4u * w_id) & 15u : w_id;
   const uint32_t R = a.m.R, K = a.m.K, GR = a.m.G * a.m.R, RS = a.m.R * a.m.S;
   const uint32_t N = a.tr.n_req;
 
@@ -1786,12 +1795,12 @@ __global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kDense>
   const uint32_t sb = smem_addr(smem_raw);
   const StageArgs<MaskT> sa = {cd.mask, cd.index, cd.scale};
   uint4* more = sizeof(MaskT) == 8 ? reinterpret_cast<uint4*>(st + a.lay.more_off) : sh.victim_more;
-  if (warp == kRoleRoute) route_warp<MaskT, kExt, kDense>(a, sh, sb, dy, sa, cd.route_log, more, cd.rep, p, lane);
+  if (warp == kRoleRoute) route_warp<MaskT, kExt, kBuild>(a, sh, sb, dy, sa, cd.route_log, more, cd.rep, p, lane);
   else if (warp == kRoleStage) stage_warp<MaskT, kExt>(a, sh, sb, sa, lane);
   else if (warp == kRoleTime) time_warp<MaskT, kExt>(a, sh, sb, dy, cd.slot_kv, cd.scale, lane);
   else if (warp == kRoleExpiry) expiry_warp<MaskT, kExt>(a, sh, sb, cd.exp_rec, cd.scale, lane);
-  else if (warp == kRoleFile) file_warp<MaskT, kExt, kDense>(a, sh, cd, p, lane);
-  else scout_warp<MaskT, kExt, kDense>(a, sh, cd, more, lane);
+  else if (warp == kRoleFile) file_warp<MaskT, kExt, kBuild>(a, sh, cd, p, lane);
+  else scout_warp<MaskT, kExt, kBuild>(a, sh, cd, more, lane);
   __syncthreads();
 
   // (pointers computed again: registers less in the loops)
@@ -1855,49 +1864,59 @@ size_t replay_smem_bytes(ReplayArgs& a) {
   return shared_bytes<MaskT, kExt>(a.m, a.tr.chunk_req, a.tr.chunk_cap, a.slots_in_smem != 0);
 }
 
-template <typename MaskT, bool kExt, bool kDense>
+template <typename MaskT, bool kExt, uint32_t kBuild>
 cudaError_t prepare_replay(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kDense>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kBuild>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // several candidates share an SM: the per-CTA footprint, not the default carve-out, decides
-  return cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kDense>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  return cudaFuncSetAttribute(replay_kernel<MaskT, kExt, kBuild>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared);
 }
 
-template <typename MaskT, bool kExt, bool kDense>
+template <typename MaskT, bool kExt, uint32_t kBuild>
 cudaError_t launch_replay_t(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
   const size_t smem = replay_smem_bytes<MaskT, kExt>(a);
-  cudaError_t e = prepare_replay<MaskT, kExt, kDense>(smem);
+  cudaError_t e = prepare_replay<MaskT, kExt, kBuild>(smem);
   if (e != cudaSuccess) return e;
-  replay_kernel<MaskT, kExt, kDense><<<n_cand, kReplayThreads, smem, st>>>(a);
+  replay_kernel<MaskT, kExt, kBuild><<<n_cand, kReplayThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
-// Up to two candidates an SM take the build without a register cap.  (us per request, this build against the dense
-// one: 16 replicas, one an SM 0.73 and 0.78, two 0.82 and 0.85; with its registers only two fit an SM, so three would take
-// two waves: 1.6 and 1.2.)  The second candidate comes to an SM when every SM has one.
+// The build of a launch.  Up to a quarter of the SMs: the one for few candidates, 3 to 6 % faster than the next (16
+// candidates, long contexts 0.80 and 0.84 us per request, shared prompts 0.74 and 0.76, 64 replicas 1.29 and 1.33).  A GPU
+// takes launches of eight streams at once unless it is told otherwise, so even then no SM has more than two of these, and
+// two fit (eight populations of 37 at once: 1.07 us per request).  Up to half of the SMs, six populations of 74
+// would take 1.85 instead of 1.55.  Up to two candidates an SM: the build with the limited
+// eviction (see evict_slow).  More: the dense one.  Around the line, 296 candidates 1.05 and 1.05, 32 replicas 1.23 and 1.24,
+// 64 replicas 1.77 and 1.82; 444 candidates 1.37 and 1.35, 32 replicas 1.61 and 1.59, 64 replicas 2.33 and 2.35.
 template <typename MaskT, bool kExt>
-cudaError_t launch_replay_n(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
+cudaError_t launch_replay_n(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  a.roles = n_cand <= (uint32_t)sms ? kOrderAlone : kOrderShared;
-  const bool dense = a.build ? a.build == 2u : n_cand > 2u * (uint32_t)sms;
-  return dense ? launch_replay_t<MaskT, kExt, true>(a, n_cand, st) : launch_replay_t<MaskT, kExt, false>(a, n_cand, st);
+  const uint32_t build = a.build ? a.build : n_cand <= (uint32_t)sms / 4u ? kSparse : n_cand <= 2u * (uint32_t)sms ? kPaired : kDense;
+  return build == kSparse ? launch_replay_t<MaskT, kExt, kSparse>(a, n_cand, st)
+         : build == kPaired ? launch_replay_t<MaskT, kExt, kPaired>(a, n_cand, st)
+                            : launch_replay_t<MaskT, kExt, kDense>(a, n_cand, st);
 }
 
-template <typename MaskT, bool kDense>
+template <typename MaskT, uint32_t kBuild>
 int replay_occupancy_t(ReplayArgs& a, size_t* smem_out) {
   *smem_out = replay_smem_bytes<MaskT, false>(a);
   int n = 0;
-  if (prepare_replay<MaskT, false, kDense>(*smem_out) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false, kDense>, (int)kReplayThreads,
+  if (prepare_replay<MaskT, false, kBuild>(*smem_out) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, replay_kernel<MaskT, false, kBuild>, (int)kReplayThreads,
                                                     *smem_out) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }
   return n;
+}
+template <typename MaskT>
+int replay_occupancy_n(ReplayArgs& a, size_t* smem_out) {
+  return a.build == kSparse ? replay_occupancy_t<MaskT, kSparse>(a, smem_out)
+         : a.build == kPaired ? replay_occupancy_t<MaskT, kPaired>(a, smem_out) : replay_occupancy_t<MaskT, kDense>(a, smem_out);
 }
 
 }  // namespace
@@ -1906,10 +1925,9 @@ int replay_occupancy(const Model& m, const TraceView& tr, uint32_t build, uint64
   ReplayArgs a = {};
   a.m = m;
   a.tr = tr;
+  a.build = build;
   size_t smem = 0;
-  const int n = m.R <= 32 ? (build == 1 ? replay_occupancy_t<uint32_t, false>(a, &smem) : replay_occupancy_t<uint32_t, true>(a, &smem))
-                : build == 1 ? replay_occupancy_t<unsigned long long, false>(a, &smem)
-                             : replay_occupancy_t<unsigned long long, true>(a, &smem);
+  const int n = m.R <= 32 ? replay_occupancy_n<uint32_t>(a, &smem) : replay_occupancy_n<unsigned long long>(a, &smem);
   if (smem_bytes) *smem_bytes = smem;
   return n;
 }

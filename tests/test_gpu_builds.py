@@ -1,5 +1,5 @@
-"""GPU parity at the edges of the rule that picks the replay kernel's build: up to one candidate an SM, up
-to two, more.  Traces that make the rare paths of the eviction common: a prompt that many share, caches of a few
+"""GPU parity at the edges of the rule that picks the replay kernel's build: up to a quarter of the SMs, up to
+two candidates an SM, more.  Traces that make the rare paths of the eviction common: a prompt that many share, caches of a few
 prompts, victims that occur again between their listing and their eviction."""
 import numpy as np
 import pytest
@@ -41,6 +41,12 @@ def test_every_build_matches_the_oracle(per_sm, extra, R, C, stats):
         for k in range(3):
             assert (gpu[key][k::3] == gpu[key][k]).all(), (key, k)
     assert sum(int(r[4][3]) for r in refs) > 0        # evictions happened
+
+
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("R,C,stats", [(8, 17, True), (32, 40, False), (64, 30, False)])
+def test_the_last_population_of_the_build_for_few_and_the_next(over, R, C, stats):
+    test_every_build_matches_the_oracle(0, _sms() // 4 + over, R, C, stats)
 
 
 @pytest.mark.parametrize("lam,steps,resident", [(1, 2, 1), (5, 3, 1), (5, 3, 5), (5, 3, 6), (4, 0, 4)])
