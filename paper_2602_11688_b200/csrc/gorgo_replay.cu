@@ -1889,6 +1889,9 @@ cudaError_t launch_replay_t(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
 // would take 1.85 instead of 1.55.  Up to two candidates an SM: the build with the limited
 // eviction (see evict_slow).  More: the dense one.  Around the line, 296 candidates 1.05 and 1.05, 32 replicas 1.23 and 1.24,
 // 64 replicas 1.77 and 1.82; 444 candidates 1.37 and 1.35, 32 replicas 1.61 and 1.59, 64 replicas 2.33 and 2.35.
+// Where shared memory lets only two an SM fit, the line could lie elsewhere, but does not matter: 600 candidates on a
+// grown trace 4.86 and 4.87 (shared prompts), 15.9 and 16.4 (long contexts), with 38 KB of slots 2.83 and 2.84, 32
+// replicas 3.35 and 3.27, 64 replicas 4.29 and 4.19.
 template <typename MaskT, bool kExt>
 cudaError_t launch_replay_n(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st) {
   int dev = 0, sms = 0;
