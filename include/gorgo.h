@@ -322,8 +322,8 @@ int gorgo_eval_population_windows(gorgo_sim_t *sim, uint32_t n_candidates, const
  * n_tuned + k] perturbs tuned parameter k of offspring l in step t.  Parameters not listed in
  * `tuned` keep their value from x0.  The arithmetic of Eq. 4 is done on the host in double
  * precision with the C library's exp and log; the sum ln x + sigma*z is two rounded operations.
- * All pointers are HOST except `workspace` (DEVICE, as for gorgo_eval_population).  The call
- * synchronises `cuda_stream` once per step.  `history`, if not NULL, receives per step
+ * All pointers are HOST except `workspace` (DEVICE, as for gorgo_eval_population: at least
+ * gorgo_workspace_bytes(sim, 1), also with n_steps = 0).  The call synchronises `cuda_stream` once per step.  `history`, if not NULL, receives per step
  * 4 + n_tuned doubles: objective of the best offspring, 1.0 if it was accepted else 0.0, sigma
  * after the step, objective of the parent after the step, tuned values of the parent after the
  * step.  Errors: GORGO_ERR_INVALID_ARG (NULL, lambda = 0, n_tuned = 0 or > K, an index >= K,

@@ -1060,6 +1060,11 @@ int gorgo_es_run(gorgo_sim_t* sim, const gorgo_es_config_t* cfg, const double* x
       return GORGO_ERR_INVALID_ARG;
     if (!(x0[cfg->tuned[k]] > 0.0)) return GORGO_ERR_INVALID_ARG;   // ln(x) of Eq. 4
   }
+  // The evaluations below lay the workspace out without the words of a proxy index that is off, so that one for L candidates
+  // holds the parent too; what is asked of the caller is gorgo_workspace_bytes(sim, 1), whatever the steps.
+  if (!finite_nonneg(cfg->time_scale)) return GORGO_ERR_NONFINITE_PARAM;
+  if ((uintptr_t)workspace % kAlign) return GORGO_ERR_INVALID_ARG;
+  if (make_ws(sim, 1, true).total > workspace_bytes) return GORGO_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   std::vector<double> parent(x0, x0 + K), pop(((size_t)L + 1) * K), pt((size_t)L + 1), pe((size_t)L + 1);
   const std::vector<double>& f = cfg->objective == 0 ? pt : pe;

@@ -73,3 +73,26 @@ def test_the_parent_is_evaluated_with_the_first_offspring(lam, steps, resident):
     assert x.tolist() == rx and f == rf and sigma == rsigma
     for t, h in enumerate(rhist):
         assert hist[t, 0] == h[0] and bool(hist[t, 1]) == h[1] and hist[t, 3] == h[3], t
+
+
+@pytest.mark.parametrize("steps,lam", [(0, 3), (1, 1), (2, 3)])
+@pytest.mark.parametrize("R", [4, 40])
+def test_the_strategy_asks_for_the_workspace_of_one_candidate(R, steps, lam):
+    """The same with and without steps; one byte less is refused and nothing is written."""
+    import torch
+    from paper_2602_11688_b200 import binding as gb
+    w = W.handmade(np.linspace(5.0, 60.0, R), small_trace(3, n_req=200), slots=2, cache_blocks=15, params=[(0.5, 1.0, 0.1)])
+    z = np.random.default_rng(1).standard_normal((steps, lam, 2))
+    sim = gb.GorgoSim(w)
+    try:
+        rc, need = gb.gorgo_workspace_bytes(sim.h, 1)
+        room = torch.zeros(need, dtype=torch.uint8, device="cuda")
+        kw = dict(x0=w.params[0], z=z, tuned=[0, 2], lo=[0.05, 0.05], hi=[2.0, 0.5], sigma0=0.5, sigma_up=1.5, n_steps=steps,
+                  lam=lam, stream=sim.stream, time_scale=1.0)
+        assert gb.gorgo_es_run(sim.h, workspace=room[:need - 1], **kw)[0] == gb.GORGO_ERR_WORKSPACE_TOO_SMALL
+        torch.cuda.synchronize()
+        assert int(room.count_nonzero()) == 0
+        assert gb.gorgo_es_run(sim.h, workspace=room, **{**kw, "time_scale": -1.0})[0] == gb.GORGO_ERR_NONFINITE_PARAM
+        assert gb.gorgo_es_run(sim.h, workspace=room, **kw)[0] == gb.GORGO_OK
+    finally:
+        sim.close()
