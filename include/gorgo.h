@@ -465,7 +465,8 @@ int gorgo_debug_set(gorgo_sim_t *sim, uint32_t what, uint32_t value);
  * 37 bytes per request and candidate and 5 per request beside them, 4 or 8 bytes (up to 32 replicas,
  * or more) per distinct run of blocks that occur together, and per replica 1,072 bytes (560 above 16
  * replicas, 816 above 32) and 16 per slot.
- * The first call on a device looks up the array's device address; make that first call outside
+ * The first call on a device looks up the array's device address and loads every kernel that a later
+ * call can launch (any population, number of replicas and model parts); make that first call outside
  * any stream capture.  All calls in a process share the one array per GPU and it keeps what the
  * previous call left there; each call clears what it needs to start from zero, but two calls
  * whose GPU work overlaps (different streams, different handles, different threads) race on it:

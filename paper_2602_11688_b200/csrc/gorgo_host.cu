@@ -1498,13 +1498,15 @@ constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
 void* g_scratch_ptr[kMaxDevices] = {};
 
-// Device address of the built-in scratch on the CURRENT device (looked up on first use).
+// Device address of the built-in scratch on the CURRENT device (looked up on first use).  The same first call loads every
+// kernel that a later one can launch, whatever its candidates, replicas and model parts.
 int static_scratch_address(int device, void** out) {
   if (device < 0 || device >= kMaxDevices) return GORGO_ERR_INVALID_ARG;
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
   if (!g_scratch_ptr[device]) {
     void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) {
+    if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p || load_replay() != cudaSuccess ||
+        load_population_kernels() != cudaSuccess) {
       cudaGetLastError();
       return GORGO_ERR_CUDA;
     }

@@ -220,6 +220,10 @@ cudaError_t launch_link_occurrences(const TraceView& tr, uint32_t first_new, uin
                                     const uint32_t* prev, Touch* touch, cudaStream_t st);
 cudaError_t launch_gather(const void* buf, uint64_t n_sectors, uint32_t per_thread, uint32_t blocks,
                           uint32_t* sink, cudaStream_t st);
+// Loads what a population evaluation can launch on the current device (kernels are else loaded at their first
+// launch, which may allocate device memory).
+cudaError_t load_replay();
+cudaError_t load_population_kernels();
 uint32_t window_max();          // largest window the window kernel handles
 uint32_t mask_bytes_for(uint32_t n_replicas);
 // CTAs of the replay kernel that fit one SM for this model (-1: query failed), and the dynamic

@@ -323,6 +323,12 @@ cudaError_t launch_link_occurrences(const TraceView& tr, uint32_t first_new, uin
   return cudaGetLastError();
 }
 
+cudaError_t load_population_kernels() {
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, reset_states_kernel);
+  return e != cudaSuccess ? e : cudaFuncGetAttributes(&fa, select_p95_kernel);
+}
+
 cudaError_t launch_select(const SelectArgs& a, uint32_t n_cand, cudaStream_t st) {
   select_p95_kernel<<<dim3(n_cand, 2), kSelectThreads, 0, st>>>(a);
   return cudaGetLastError();

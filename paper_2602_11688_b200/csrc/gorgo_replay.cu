@@ -1935,6 +1935,19 @@ int replay_occupancy(const Model& m, const TraceView& tr, uint32_t build, uint64
   return n;
 }
 
+cudaError_t load_replay() {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaSuccess;
+  const auto load = [&](auto kernel) { if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel); };
+  load(replay_kernel<uint32_t, false, kSparse>); load(replay_kernel<uint32_t, true, kSparse>);
+  load(replay_kernel<uint32_t, false, kPaired>); load(replay_kernel<uint32_t, true, kPaired>);
+  load(replay_kernel<uint32_t, false, kDense>); load(replay_kernel<uint32_t, true, kDense>);
+  load(replay_kernel<unsigned long long, false, kSparse>); load(replay_kernel<unsigned long long, true, kSparse>);
+  load(replay_kernel<unsigned long long, false, kPaired>); load(replay_kernel<unsigned long long, true, kPaired>);
+  load(replay_kernel<unsigned long long, false, kDense>); load(replay_kernel<unsigned long long, true, kDense>);
+  return e;
+}
+
 uint32_t mask_bytes_for(uint32_t n_replicas) { return n_replicas <= 32 ? 4u : 8u; }
 
 cudaError_t launch_replay(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st) {

@@ -150,3 +150,46 @@ def test_static_scratch_entry_point_refuses_a_trace_beyond_its_limit():
     torch.cuda.synchronize()
     assert a.item() == -1.0 and b.item() == -1.0             # nothing ran
     sim.close()
+
+
+CHILD = """
+import numpy as np, torch
+from paper_2602_11688_b200 import binding as gb
+from paper_2602_11688_b200 import workloads as W
+few, many = torch.cuda.get_device_properties(0).multi_processor_count // 8, 5 * torch.cuda.get_device_properties(0).multi_processor_count
+sims = []
+for base, speeds in (("tiny", False), ("tiny", True), ("largest", False), ("largest", True)):
+    w = W.make_workload(base, n_requests=300, cache_blocks=300, population=many)
+    sim = gb.GorgoSim(w)
+    if speeds:
+        assert gb.gorgo_sim_set_replica_speeds(sim.h, np.full(sim.R, 0.05), None) == gb.GORGO_OK
+    sims.append((sim, torch.from_numpy(np.ascontiguousarray(w.params)).cuda()))
+a = torch.empty(many, dtype=torch.float64, device="cuda")
+b = torch.empty(many, dtype=torch.float64, device="cuda")
+status = torch.zeros(many, dtype=torch.int32, device="cuda")
+
+def run(k, P):
+    sim, params = sims[k]
+    assert gb.gorgo_eval_population_static(sim.h, P, params, 1.0, sim.stream, a, b, None, None, status) == gb.GORGO_OK
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+free = run(0, few)
+for k in range(4):
+    for P in (few, 2 * few + 1, many // 5, many // 2, many):
+        now = run(k, P)
+        assert now == free, (k, P, free - now)
+assert int(status.abs().sum()) == 0
+print("same free memory")
+"""
+
+
+def test_only_the_first_call_of_a_process_loads_anything():
+    """In a fresh process: after one small population of the plain model, larger populations (other builds of the
+    replay kernel, waves among them), more than 32 replicas and optional model parts take no device memory."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", CHILD], cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0 and "same free memory" in out.stdout, out.stderr[-2000:]
