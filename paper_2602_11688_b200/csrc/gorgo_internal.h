@@ -111,6 +111,7 @@ struct ReplayArgs {
   uint32_t probe_off, scout_off;  // test switches: no mask words read ahead / no victims listed ahead
   uint32_t slots_in_smem;         // set by the launcher: per-slot state fits in shared memory
   uint32_t ring_cap;              // set by the launcher: listed victims kept per replica (a power of two)
+  uint32_t alone;                 // set by the launcher: at most one candidate an SM
   uint32_t build;                 // test switch: 0, or the build of the kernel that is launched (1 to kReplayBuilds)
   const double* params;           // [P*K] device, or null: `inline_params` (one candidate)
   double inline_params[67];

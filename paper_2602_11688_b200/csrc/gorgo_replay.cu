@@ -1639,14 +1639,6 @@ constexpr uint32_t kReplayThreads = 32 * kRoles;
 // blocks fit an SM only if their warps begin on alternate schedulers, as the blocks of one launch do; those of
 // several launches do not always (three streams of 148 took two turns with 96 registers too), but two always fit.
 template <typename MaskT, uint32_t kBuild> constexpr int kReplayMinCtas = kBuild == kSparse || sizeof(MaskT) == 8 ? 3 : 4;
-// Roles by warp, four bits each.  The hardware gives an SM's four schedulers a block's warps in turn, so the third and
-// fourth of six have a scheduler alone.  With one candidate an SM the route warp is the third: 2 to 3 % faster
-// than next to the scout.  With a second candidate all schedulers hold three warps, and the order of Role is 6 % faster.
-constexpr uint32_t role_order(Role w0, Role w1, Role w2, Role w3, Role w4, Role w5) {
-  return w0 | w1 << 4 | w2 << 8 | w3 << 12 | w4 << 16 | w5 << 20;
-}
-constexpr uint32_t kOrderSparse = role_order(kRoleScout, kRoleStage, kRoleRoute, kRoleExpiry, kRoleTime, kRoleFile);
-
 // The lists of the launch before (the end of the kernel says why).  (Out of line: inlined it costs the
 // loops registers.)
 template <typename MaskT, bool kExt>
@@ -1673,7 +1665,17 @@ __global__ void __launch_bounds__(kReplayThreads, (kReplayMinCtas<MaskT, kBuild>
   const uint32_t p = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t w_id = __shfl_sync(kFull, threadIdx.x >> 5, 0);   // (known to be the same for all lanes)
-  const uint32_t warp = kBuild == kSparse ? kOrderSparse >> (4u * w_id) & 15u : w_id;
+  // Role of the warp.  The hardware gives an SM's four schedulers a block's warps in turn, so the third and fourth of six
+  // have a scheduler alone.  In a launch of at most one candidate an SM the order is scout, stage, route, expiry, time,
+  // file: with the route warp alone 148 candidates take 0.844 us per request instead of 0.863, 32 replicas 1.07 instead
+  // of 1.09, 64 replicas 1.40 instead of 1.43.  Two an SM put three warps on every scheduler, and the order of Role is
+  // the faster one (256 candidates 0.94, in the other order 0.98).  (The form matters more than its few instructions: as
+  // a table or a select, which move the roles' code, 256 candidates took 0.97 and 0.98 in the order of Role too.)
+  uint32_t warp = w_id;
+  if (kBuild != kDense && (kBuild == kSparse || a.alone) && !(w_id & 1u)) {
+    warp += 4u;
+    if (warp >= kRoles) warp -= kRoles;
+  }
   const uint32_t R = a.m.R, K = a.m.K, GR = a.m.G * a.m.R, RS = a.m.R * a.m.S;
   const uint32_t N = a.tr.n_req;
 
@@ -1893,11 +1895,12 @@ cudaError_t launch_replay_t(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
 // grown trace 4.86 and 4.87 (shared prompts), 15.9 and 16.4 (long contexts), with 38 KB of slots 2.83 and 2.84, 32
 // replicas 3.35 and 3.27, 64 replicas 4.29 and 4.19.
 template <typename MaskT, bool kExt>
-cudaError_t launch_replay_n(const ReplayArgs& a, uint32_t n_cand, cudaStream_t st) {
+cudaError_t launch_replay_n(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
+  a.alone = n_cand <= (uint32_t)sms ? 1u : 0u;
   const uint32_t build = a.build ? a.build : n_cand <= (uint32_t)sms / 4u ? kSparse : n_cand <= 2u * (uint32_t)sms ? kPaired : kDense;
   return build == kSparse ? launch_replay_t<MaskT, kExt, kSparse>(a, n_cand, st)
          : build == kPaired ? launch_replay_t<MaskT, kExt, kPaired>(a, n_cand, st)
