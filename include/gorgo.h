@@ -390,7 +390,7 @@ int gorgo_tune_online(gorgo_sim_t *sim, const gorgo_online_config_t *cfg, uint32
  * one SM holds at once for this configuration, and the shared memory each takes.  A population
  * larger than SMs x that number is replayed in successive rounds of CTAs.  (The number is the same for
  * every launch of more than a quarter as many candidates as the GPU has SMs; smaller launches take a
- * build of which an SM may hold one less.) */
+ * build of which an SM may hold only two.) */
 int gorgo_replay_occupancy(gorgo_sim_t *sim, int32_t *ctas_per_sm, uint64_t *smem_bytes_per_cta);
 /* Measurement aid (no counterpart in the paper).  With profiling enabled, gorgo_eval_population
  * records a CUDA event on `cuda_stream` directly before and after each launch of the replay

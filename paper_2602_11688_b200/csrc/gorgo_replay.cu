@@ -32,9 +32,9 @@
 // still over the cache: with three or four candidates an SM 128 bytes more in one of them cost about 3 %,
 // so what is rare is out of line, and loops that could share a body do.  Three builds share this source
 // (launch_replay_n says which a launch takes).  16 / 148 / 256 / 444 / 592 candidates, long contexts (8,000 requests, 2,000
-// blocks a cache) with the dense build 0.87 / 0.89 / 0.96 / 1.35 / 1.64 us per request, with the three 0.80 / 0.85 / 0.94 / 1.35 /
-// 1.64; shared prompts 0.76 / 0.80 / 0.85 / 1.05 / 1.22 and 0.74 / 0.79 / 0.85 / 1.05 / 1.22; 64 replicas (6,000
-// requests) 1.32 / 1.51 / 1.68 / 2.36 / 3.91 and 1.29 / 1.43 / 1.62 / 2.36 / 3.91.
+// blocks a cache) with the dense build 0.87 / 0.89 / 0.96 / 1.35 / 1.64 us per request, with the three 0.79 / 0.84 / 0.94 / 1.35 /
+// 1.64; shared prompts 0.76 / 0.80 / 0.85 / 1.05 / 1.22 and 0.74 / 0.78 / 0.85 / 1.05 / 1.22; 64 replicas (6,000
+// requests) 1.32 / 1.51 / 1.68 / 2.36 / 3.91 and 1.29 / 1.40 / 1.61 / 2.36 / 3.91.
 #include "gorgo_device.cuh"
 
 namespace gorgo {
@@ -1633,12 +1633,12 @@ enum Role : uint32_t { kRoleRoute, kRoleStage, kRoleTime, kRoleExpiry, kRoleScou
 constexpr uint32_t kReplayThreads = 32 * kRoles;
 // Candidates an SM holds, which caps the registers: four (80 registers a thread), three with more than 32 replicas (96).
 // A launch does not see what other streams run on the GPU, so a build that large launches take leaves room for as
-// many: with two an SM (98 registers, no spills; 3 to 6 % faster alone) three populations of 148 on three streams took
-// 1.91 us per request instead of 1.45 (16 replicas), 1.69 instead of 1.14 (shared prompts) and 2.40 instead of 1.75 (32
-// replicas), and two of 256 1.96 instead of 1.62.  The build for few candidates has at most 96 registers.  Three of its
-// blocks fit an SM only if their warps begin on alternate schedulers, as the blocks of one launch do; those of
-// several launches do not always (three streams of 148 took two turns with 96 registers too), but two always fit.
-template <typename MaskT, uint32_t kBuild> constexpr int kReplayMinCtas = kBuild == kSparse || sizeof(MaskT) == 8 ? 3 : 4;
+// many: with two an SM (98 registers, no spills; 1 to 4 % faster alone) three populations of 148 on three streams took
+// 1.91 us per request instead of 1.41 (16 replicas), 1.69 instead of 1.10 (shared prompts) and 2.40 instead of 1.68 (32
+// replicas), and two of 256 1.96 instead of 1.62.  The build for few candidates has room for two
+// (three with more than 32 replicas, where two gain nothing).  With 96 registers three would fit, 1 % slower, but only if
+// their warps begin on alternate schedulers, as those of one launch do; three streams of 148 took two turns all the same.
+template <typename MaskT, uint32_t kBuild> constexpr int kReplayMinCtas = sizeof(MaskT) == 8 ? 3 : kBuild == kSparse ? 2 : 4;
 // The lists of the launch before (the end of the kernel says why).  (Out of line: inlined it costs the
 // loops registers.)
 template <typename MaskT, bool kExt>
@@ -1884,10 +1884,10 @@ cudaError_t launch_replay_t(ReplayArgs a, uint32_t n_cand, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// The build of a launch.  Up to a quarter of the SMs: the one for few candidates, 3 to 6 % faster than the next (16
-// candidates, long contexts 0.80 and 0.84 us per request, shared prompts 0.74 and 0.76, 64 replicas 1.29 and 1.33).  A GPU
-// takes launches of eight streams at once unless it is told otherwise, so even then no SM has more than two of these, and
-// two fit (eight populations of 37 at once: 1.07 us per request).  Up to half of the SMs, six populations of 74
+// The build of a launch.  Up to a quarter of the SMs: the one for few candidates, 1 to 4 % faster than the next (16
+// candidates, long contexts 0.79 and 0.82 us per request, shared prompts 0.74 and 0.75, 32 replicas 1.02 and 1.05).  A GPU
+// takes launches of eight streams at once unless it is told otherwise: even then there are at most two of these an SM, and
+// two fit (eight populations of 37 at once: 1.09 us per request).  Up to half of the SMs, six populations of 74
 // would take 1.85 instead of 1.55.  Up to two candidates an SM: the build with the limited
 // eviction (see evict_slow).  More: the dense one.  Around the line, 296 candidates 1.05 and 1.05, 32 replicas 1.23 and 1.24,
 // 64 replicas 1.77 and 1.82; 444 candidates 1.37 and 1.35, 32 replicas 1.61 and 1.59, 64 replicas 2.33 and 2.35.
