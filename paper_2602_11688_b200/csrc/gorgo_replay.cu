@@ -1376,8 +1376,9 @@ __device__ __forceinline__ void file_warp(const ReplayArgs& a, Shared<MaskT, kEx
 // after the other (kAsk of them with their loads in flight together): one memory latency per asker.  (The askers by lane
 // and the requests one after the other, four at a time: shared prompts, 8 replicas, 64 candidates 0.81 us per request,
 // with this 0.78.  Inlined, one asker is in flight: the code of four inside the scout's loop costs four candidates an
-// SM 5 %, two 1 to 3 % and with 64 replicas 7 to 9 % (1.79 -> 1.95 us), and gains 1 % with one candidate an SM and
-// shared prompts.  With more than 32 replicas it is called, with four: 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
+// SM 5 %, two 1 to 3 % and with 64 replicas 7 to 9 % (1.79 -> 1.95 us).  With one candidate an SM and shared prompts four
+// gain 1 % (8 replicas, 16 candidates 0.738 -> 0.729), so the build for few candidates has four.  With more than 32
+// replicas it is called, with four: 1, 2, 4 and 8 take 2.02, 1.98, 1.97 and 2.05 us.)
 template <uint32_t kAsk>
 __device__ __forceinline__ bool touched_again(const Touch* touch, uint32_t atom, uint32_t my_q, uint32_t my_k, uint32_t rq, uint32_t off,
                                               uint32_t m, uint32_t n) {
@@ -1579,7 +1580,7 @@ __device__ __forceinline__ void scout_warp(const ReplayArgs& a, Shared<MaskT, kE
         if (hop == kHops && n_match) {
           const uint32_t asked = open ? t.atom : kNone;
           if (sizeof(MaskT) == 8 ? touched_again_called(touch, asked, my_q, my_k, rq, off, m, n_match)
-                                : touched_again<1>(touch, asked, my_q, my_k, rq, off, m, n_match)) live = open = false;
+                                : touched_again<kBuild == kSparse ? 4 : 1>(touch, asked, my_q, my_k, rq, off, m, n_match)) live = open = false;
           rest = __ballot_sync(kFull, open);
           if (!rest) break;
         }
