@@ -200,7 +200,7 @@ cudaError_t launch_policy_routes(const TraceView& tr, uint32_t R, bool affinity,
                                  const uint32_t* draws, uint8_t* route, cudaStream_t st);
 #ifdef GORGO_PROF
 // Cycle accounting build only: 16 accumulators per role (route 0, time 16, expiry 32, file 48,
-// scout 64, stage 80; 96 to 111 stay 0).
+// scout 64, stage 80; 96: the eviction out of line).
 cudaError_t prof_read(unsigned long long* out112, bool reset);
 #endif
 // What a small append writes, carried by the launch itself: runs of words for up to five places, then the

@@ -42,17 +42,24 @@ namespace {
 
 // Cycle accounting of the warps (built only with -DGORGO_PROF; the normal library carries none of
 // it).  Every lap adds the SM clock ticks since the previous lap of the same warp to one of 16
-// accumulators per role; the totals of all candidates end up in g_prof.
+// accumulators per role; the totals of all candidates end up in g_prof.  What functions out of line spend
+// is added by themselves, from 96 on.
 #ifdef GORGO_PROF
 __device__ unsigned long long g_prof[112];
 #define PROF_BEGIN() unsigned long long pf[16] = {}; long long pf_t = clock64()
 #define PROF_LAP(k) do { const long long pf_n = clock64(); pf[k] += (unsigned long long)(pf_n - pf_t); pf_t = pf_n; } while (0)
 #define PROF_ADD(k, v) pf[k] += (unsigned long long)(v)
+#define PROF_MARK(t) const long long t = clock64()
+#define PROF_SINCE(k, t) do { if ((threadIdx.x & 31u) == 0) atomicAdd(&g_prof[k], (unsigned long long)(clock64() - t)); } while (0)
+#define PROF_COUNT(k) do { if ((threadIdx.x & 31u) == 0) atomicAdd(&g_prof[k], 1ull); } while (0)
 #define PROF_END(base) do { if (lane == 0) { _Pragma("unroll") for (int pf_i = 0; pf_i < 16; ++pf_i) atomicAdd(&g_prof[(base) + pf_i], pf[pf_i]); } } while (0)
 #else
 #define PROF_BEGIN() do {} while (0)
 #define PROF_LAP(k) do {} while (0)
 #define PROF_ADD(k, v) do {} while (0)
+#define PROF_MARK(t) do {} while (0)
+#define PROF_SINCE(k, t) do {} while (0)
+#define PROF_COUNT(k) do {} while (0)
 #define PROF_END(base) do {} while (0)
 #endif
 
@@ -710,7 +717,10 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
         sts64(p_take, make_uint2(head, cons));
         sts32(sb + offsetof(Control, want), rep + 1u);
       }
+      PROF_MARK(waited);
       avail = wait_slow(p_tail, head + 1u, sb, a.poll_limit) - head;
+      PROF_SINCE(96, waited);
+      PROF_COUNT(97);
       if (lane == 0) sts32(sb + offsetof(Control, want), 0u);
       if ((int32_t)avail <= 0) break;               // gave up
     }
@@ -725,11 +735,14 @@ __device__ __noinline__ uint32_t evict_slow(const ReplayArgs& a, Shared<MaskT, k
     const bool listed = lane < avail;
     bool live = listed;
     uint32_t d = 0;
+    PROF_MARK(walked);
     if (listed && next_req < r + kStages) {         // it occurred again since it was listed, or will soon
       const uint32_t next = sizeof(MaskT) == 8 ? __ldcg(&more[e].x) : lds32(sb + (uint32_t)offsetof(Sh, victim_more) + e * 16u);
       live = victim_live(a.tr.touch, route_log, sb, sb + (uint32_t)offsetof(Sh, route_ring), next, next_req, r, a.first, rep, d);
     }
     dirty |= __reduce_or_sync(kFull, d);
+    PROF_SINCE(98, walked);
+    PROF_COUNT(99);
     const uint32_t prev = __shfl_up_sync(kFull, upto, 1);
     uint32_t dead = listed && !live ? upto - (lane ? prev : 0u) : 0u;   // blocks that are no victims
     if (kBuild == kDense || __any_sync(kFull, dead != 0u)) {
@@ -904,14 +917,17 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
     bool valid = !(dirty & 1u);
     PROF_LAP(1);
     if (__any_sync(kFull, special || !rdy || (need != 0u && (soon || enough == 0u)))) {
+      PROF_LAP(2);
       const bool again = __any_sync(kFull, special);
       if (again) {
+        PROF_ADD(10, 1);
         uint32_t d = dirty;
         missing = commit_slow<MaskT, kExt>(a, sh, sa, istar, q - 1u, d);
         dirty = d;
         held = occ + missing;
         need = held > C ? held - C : 0u;
       }
+      PROF_LAP(6);
       if (need != 0u && (again || enough == 0u || __any_sync(kFull, soon))) {
         PROF_ADD(9, 1);
         dirty |= evict_slow<MaskT, kExt, kBuild>(a, sh, sa.mask, route_log, more, istar, q - 1u, need);
@@ -919,9 +935,11 @@ __device__ __forceinline__ void route_warp(const ReplayArgs& a, Shared<MaskT, kE
         need = 0u;
         held = C;
       }
+      PROF_LAP(11);
       valid = __all_sync(kFull, rdy) && !(dirty & 1u);
     }
     PROF_LAP(2);
+    PROF_LAP(12);                                               // (nothing: what a lap itself costs)
     if (need != 0u) {
       const uint32_t keep = upto - need;                        // (last of them: blocks the last victim keeps)
       const bool last = taken >> lane == 1u;

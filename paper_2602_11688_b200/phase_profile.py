@@ -17,9 +17,11 @@ import json
 import numpy as np
 
 ROLES = {
-    "route": (0, ["commit and score", "argmin, eviction vote", "out of line: commit, eviction", "eviction",
-                  "decided again: waits, staging", "publish, hand-over", None, "#requests decided again",
-                  "#requests staged again", "#evictions out of line"]),
+    "route": (0, ["commit and score", "argmin, eviction vote", "vote on the unusual", "eviction",
+                  "decided again: waits, staging", "publish, hand-over", "commit out of line", "#requests decided again",
+                  "#requests staged again", "#evictions out of line", "#commits out of line", "eviction out of line",
+                  "a lap of nothing"]),
+    "in it": (96, ["wait for the scout", "#waits for the scout", "later occurrences of listed victims", "#rounds"]),
     "time": (16, ["wait for a routed request", "times of a group"]),
     "expiry": (32, ["waits", "completions of one request"]),
     "file": (48, ["lists handed over", "outputs and lists filed"]),
