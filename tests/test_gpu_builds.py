@@ -96,3 +96,35 @@ def test_the_strategy_asks_for_the_workspace_of_one_candidate(R, steps, lam):
         assert gb.gorgo_es_run(sim.h, workspace=room, **kw)[0] == gb.GORGO_OK
     finally:
         sim.close()
+
+
+@pytest.mark.parametrize("R,C", [(8, 17), (40, 30)])
+def test_populations_on_several_streams_at_once(R, C):
+    """Launches of all builds side by side, on streams of their own, give what each gives alone."""
+    import torch
+    from paper_2602_11688_b200 import binding as gb
+    base = np.random.default_rng(R).normal(1.0, 0.3, size=(8, 3))
+    w = W.handmade(np.linspace(5.0, 60.0, R), shared_prompt_trace(R, 600), slots=2, cache_blocks=C, params=base)
+    sizes = [_sms() // 4, _sms(), _sms() + 1, 2 * _sms() + 3]
+    sims = [gb.GorgoSim(w) for _ in sizes]
+    try:
+        params = [np.tile(base, (P // 8 + 1, 1))[:P] for P in sizes]
+        alone = [gpu_eval(w, p, 1.0, stats=False, sim=s) for s, p in zip(sims, params)]
+        refs = oracle_eval(w, base[:2], 1.0)
+        for got in alone:
+            for p in (0, 1):
+                assert_candidate_matches(got, p, refs[p])
+        streams = [torch.cuda.Stream() for _ in sizes]
+        for _ in range(3):
+            outs = []
+            torch.cuda.synchronize()
+            for sim, p, st in zip(sims, params, streams):
+                with torch.cuda.stream(st):
+                    outs.append(sim.eval_population(p, 1.0, want_route=True, want_hit=True, want_digest=True))
+            torch.cuda.synchronize()
+            for got, want in zip(outs, alone):
+                for key in ("status", "route", "hit", "digest", "p95_ttft", "p95_e2e"):
+                    assert np.array_equal(got[key].cpu().numpy(), want[key]), key
+    finally:
+        for sim in sims:
+            sim.close()
