@@ -429,7 +429,7 @@ def main():
                 yard["l2_peak"] = {"value": gbs, "unit": "GB/s", "footprint_bytes": small}
 
     if rank == 0:
-        rc, ctas_per_sm, smem_cta = gb.gorgo_replay_occupancy(sim.h)
+        rc, ctas_per_sm, smem_cta = sim.replay_occupancy(min(P, resident))
         peak, peak_kind = measured_peak_gbs()
         launch_ms = replay["ms"] / max(1, replay["launches"])
         bytes_per_launch = alg_bytes / waves

@@ -505,6 +505,16 @@ class GorgoSim:
             self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
         return resident
 
+    def replay_occupancy(self, candidates: int):
+        """(status, CTAs an SM holds, shared memory of each) of the build that a launch of so many candidates
+        takes: up to a quarter of the SMs the one for few, of which an SM may hold fewer."""
+        few = candidates <= self.torch.cuda.get_device_properties(self.device).multi_processor_count // 4
+        gorgo_debug_set(self.h, GORGO_DEBUG_BUILD, 1 if few else 0)
+        try:
+            return gorgo_replay_occupancy(self.h)
+        finally:
+            gorgo_debug_set(self.h, GORGO_DEBUG_BUILD, 0)
+
     def eval_population(self, params, time_scale=1.0, *, want_route=False, want_hit=False,
                         want_digest=False, want_stats=False, resident=None, max_bytes=None):
         """Device-output evaluation; returns a dict of torch CUDA tensors."""

@@ -70,7 +70,7 @@ def main():
         rc, ms, _ = gb.gorgo_last_replay_ms(sim.h)
     lib.gorgo_debug_phase_cycles(sim.h, buf)
     cyc = np.array(list(buf), dtype=np.float64) / (float(P) * N)
-    rc, ctas, smem = gb.gorgo_replay_occupancy(sim.h)
+    rc, ctas, smem = sim.replay_occupancy(P)
     out = {"workload": w.spec.name, "requests": N, "population": P,
            "replay_ms": ms, "us_per_request": ms * 1e3 / N, "ctas_per_sm": ctas,
            "smem_bytes_per_cta": smem, "per_request": {}}

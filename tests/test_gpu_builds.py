@@ -128,3 +128,20 @@ def test_populations_on_several_streams_at_once(R, C):
     finally:
         for sim in sims:
             sim.close()
+
+
+def test_the_occupancy_reported_is_of_the_build_that_a_launch_takes():
+    from paper_2602_11688_b200 import binding as gb
+    w = W.handmade(np.linspace(5.0, 60.0, 16), small_trace(3, n_req=100), slots=2, cache_blocks=15, params=[(0.5, 1.0, 0.1)])
+    sim = gb.GorgoSim(w)
+    try:
+        by_build = {}
+        for build in (1, 2, 3):
+            assert gb.gorgo_debug_set(sim.h, gb.GORGO_DEBUG_BUILD, build) == gb.GORGO_OK
+            by_build[build] = gb.gorgo_replay_occupancy(sim.h)
+        sms = _sms()
+        for candidates, build in ((1, 1), (sms // 4, 1), (sms // 4 + 1, 2), (2 * sms, 2), (2 * sms + 1, 3)):
+            assert sim.replay_occupancy(candidates) == by_build[build], candidates
+        assert gb.gorgo_replay_occupancy(sim.h) == by_build[3]
+    finally:
+        sim.close()
